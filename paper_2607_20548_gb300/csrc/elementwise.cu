@@ -88,15 +88,15 @@ __device__ __forceinline__ float adam_one(float g, float m, float& v, float beta
   return (m * inv_bc1) / (sqrtf(vn) * inv_sqrt_bc2 + eps);
 }
 
+// N goes to the planes Np if they are given (cols a multiple of 4 then), else over G'.
 __global__ void adam_kernel(float* Gp, const float* Mp, float* V, int rows, int cols, float beta2,
                             float eps, float inv_bc1, float inv_sqrt_bc2, const uint8_t* skipL,
-                            const uint8_t* skipR, float* N_lo, int* status) {
+                            const uint8_t* skipR, Planes Np, int* status) {
   const int b = blockIdx.y;
   const int64_t elems = (int64_t)rows * cols;
   float* gp = Gp + (int64_t)b * elems;
   const float* mp = Mp + (int64_t)b * elems;
   float* v = V + (int64_t)b * elems;
-  float* nl = N_lo ? N_lo + (int64_t)b * elems : nullptr;
   const uint8_t* sl = skipL ? skipL + (int64_t)b * rows : nullptr;
   const uint8_t* sr = skipR ? skipR + (int64_t)b * cols : nullptr;
   const float c2 = 1.f - beta2;
@@ -115,9 +115,8 @@ __global__ void adam_kernel(float* Gp, const float* Mp, float* V, int rows, int 
       o.y = adam_one(g.y, m.y, vv.y, beta2, c2, eps, inv_bc1, inv_sqrt_bc2);
       o.z = adam_one(g.z, m.z, vv.z, beta2, c2, eps, inv_bc1, inv_sqrt_bc2);
       o.w = adam_one(g.w, m.w, vv.w, beta2, c2, eps, inv_bc1, inv_sqrt_bc2);
+      const int row = (int)(4 * i4 / cols), col = (int)(4 * i4 - (int64_t)row * cols);
       if (sl || sr) {
-        const int64_t row = (4 * i4) / cols;
-        const int col = (int)(4 * i4 - row * cols);
         if (sl && sl[row]) o = make_float4(0.f, 0.f, 0.f, 0.f);
         if (sr) {
           if (sr[col]) o.x = 0.f;
@@ -128,8 +127,8 @@ __global__ void adam_kernel(float* Gp, const float* Mp, float* V, int rows, int 
       }
       bad |= !isfinite(o.x) | !isfinite(o.y) | !isfinite(o.z) | !isfinite(o.w);
       reinterpret_cast<float4*>(v)[i4] = vv;
-      reinterpret_cast<float4*>(gp)[i4] = o;
-      if (nl) reinterpret_cast<float4*>(nl)[i4] = make_float4(lo_part(o.x), lo_part(o.y), lo_part(o.z), lo_part(o.w));
+      if (Np.p) b3_store4(Np.p + b * Np.stride + row * Np.ld + col, Np.plane, o);
+      else reinterpret_cast<float4*>(gp)[i4] = o;
     }
   } else {
     for (int64_t i = start; i < elems; i += stride) {
@@ -139,7 +138,6 @@ __global__ void adam_kernel(float* Gp, const float* Mp, float* V, int rows, int 
       if ((sl && sl[i / cols]) || (sr && sr[i % cols])) nv = 0.f;
       bad |= !isfinite(nv);
       gp[i] = nv;
-      if (nl) nl[i] = lo_part(nv);
     }
   }
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(status, kStatusNonFinite);
@@ -166,57 +164,88 @@ __global__ void identity_kernel(float* Q, int n) {
 }
 
 
-// One 32 x 32 tile of one matrix per block (32 x 8 threads). Reads G and writes the
-// tensor-core operands into the step's workspace: G and its lo part, G^T and its lo part, and
-// the momentum EMA M_hat <- b1 M_hat + (1-b1) G, stored back into the optimizer state (Mh) and
-// copied with its lo part beside G (Mc, Mc_lo), so that one batched product rotates both.
-// M_hat is kept in G's orientation or, with mh_transposed, as M_hat^T (the working orientation
-// of a matrix preconditioned on its left side only).
-__global__ void momentum_split_kernel(const float* const* grads, float* Gn, float* Gn_lo, float* Gt, float* Gt_lo,
-                                      float* Mh, float* Mc, float* Mc_lo, int rows, int cols, float beta1,
-                                      int mh_transposed, int* status) {
-  __shared__ float tile[32][33];
+// A 64 x 32 tile's work: 256 threads, four consecutive elements of a row each, two rows per thread
+// going in, and the same of the transposed tile coming out, so that both orientations are read and
+// written in 16-byte (planes: 8-byte) units. rows and cols are multiples of 4.
+constexpr int kTr = 64, kTc = 32;
+struct TileIn {
+  int r, c;  // row, first column inside the tile
+  __device__ TileIn(int i) : r((threadIdx.x >> 3) + 32 * i), c(4 * (threadIdx.x & 7)) {}
+};
+struct TileOut {
+  int c, r;  // row of the transpose (a column of the tile), first column of it
+  __device__ TileOut(int i) : c((threadIdx.x >> 4) + 16 * i), r(4 * (threadIdx.x & 15)) {}
+};
+struct TileBuf {
+  float v[kTr][kTc + 1];
+  __device__ void put(const TileIn& t, float4 x) {
+    v[t.r][t.c] = x.x;
+    v[t.r][t.c + 1] = x.y;
+    v[t.r][t.c + 2] = x.z;
+    v[t.r][t.c + 3] = x.w;
+  }
+  __device__ float4 get(const TileOut& t) const {
+    return make_float4(v[t.r][t.c], v[t.r + 1][t.c], v[t.r + 2][t.c], v[t.r + 3][t.c]);
+  }
+};
+__device__ __forceinline__ bool bad4(float4 x) {
+  return !isfinite(x.x) | !isfinite(x.y) | !isfinite(x.z) | !isfinite(x.w);
+}
+__device__ __forceinline__ float4 ema4(float beta, float4 m, float c1, float4 x) {
+  return make_float4(fmaf(beta, m.x, c1 * x.x), fmaf(beta, m.y, c1 * x.y), fmaf(beta, m.z, c1 * x.z),
+                     fmaf(beta, m.w, c1 * x.w));
+}
+
+// One 64 x 32 tile of one matrix per block. Reads G and writes the tensor-core operands into the
+// step's workspace, as planes: G, G^T, and the momentum EMA M_hat <- b1 M_hat + (1-b1) G, stored
+// back into the optimizer state (Mh) and written beside G (or G^T, if M_hat is kept transposed:
+// the working orientation of a matrix preconditioned on its left side only), so that one batched
+// product rotates both. Bound by memory: 12 bytes an element of gradient and state, 18 of planes.
+template <bool MT>
+__global__ void __launch_bounds__(256) momentum_split_kernel(const float* const* grads, Planes Gn, Planes Gt, Planes Mc,
+                                                             float* Mh, int rows, int cols, float beta1, int* status) {
+  __shared__ TileBuf tile;
   const int b = blockIdx.z;
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  const int r0 = blockIdx.y * kTr, c0 = blockIdx.x * kTc;
   const int64_t mn = (int64_t)rows * cols;
   const float* g = grads[b];
   const float c1 = 1.f - beta1;
   int bad = 0;
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int r = r0 + i, c = c0 + threadIdx.x;
-    float x = 0.f;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const TileIn t(i);
+    const int r = r0 + t.r, c = c0 + t.c;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
     if (r < rows && c < cols) {
-      const int64_t o = (int64_t)b * mn + (int64_t)r * cols + c;
-      x = g[(int64_t)r * cols + c];
-      bad |= !isfinite(x);
-      Gn[o] = x;
-      Gn_lo[o] = lo_part(x);
-      if (!mh_transposed) {
-        const float m = fmaf(beta1, Mh[o], c1 * x);
-        Mh[o] = m;
-        Mc[o] = m;
-        Mc_lo[o] = lo_part(m);
+      x = *reinterpret_cast<const float4*>(g + (int64_t)r * cols + c);
+      bad |= bad4(x);
+      b3_store4(Gn.p + b * Gn.stride + r * Gn.ld + c, Gn.plane, x);
+      if (!MT) {
+        float4* mp = reinterpret_cast<float4*>(Mh + b * mn + (int64_t)r * cols + c);
+        const float4 m = ema4(beta1, *mp, c1, x);
+        *mp = m;
+        b3_store4(Mc.p + b * Mc.stride + r * Mc.ld + c, Mc.plane, m);
       }
     }
-    tile[i][threadIdx.x] = x;
+    tile.put(t, x);
   }
   __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int c = c0 + i, r = r0 + threadIdx.x;  // G^T[c][r]
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const TileOut t(i);
+    const int c = c0 + t.c, r = r0 + t.r;  // G^T[c][r]
     if (r < rows && c < cols) {
-      const float x = tile[threadIdx.x][i];
-      const int64_t o = (int64_t)b * mn + (int64_t)c * rows + r;
-      Gt[o] = x;
-      Gt_lo[o] = lo_part(x);
-      if (mh_transposed) {
-        const float m = fmaf(beta1, Mh[o], c1 * x);
-        Mh[o] = m;
-        Mc[o] = m;
-        Mc_lo[o] = lo_part(m);
+      const float4 x = tile.get(t);
+      b3_store4(Gt.p + b * Gt.stride + c * Gt.ld + r, Gt.plane, x);
+      if (MT) {
+        float4* mp = reinterpret_cast<float4*>(Mh + b * mn + (int64_t)c * rows + r);
+        const float4 m = ema4(beta1, *mp, c1, x);
+        *mp = m;
+        b3_store4(Mc.p + b * Mc.stride + c * Mc.ld + r, Mc.plane, m);
       }
     }
   }
-  if (__syncthreads_or(bad) && threadIdx.x == 0 && threadIdx.y == 0) atomicOr(status, kStatusNonFinite);
+  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(status, kStatusNonFinite);
 }
 
 // Packed symmetric storage of an n x n factor: only its lower-triangular 32 x 32 tiles, tile
@@ -230,24 +259,23 @@ __device__ __forceinline__ void tri_tile(int t, int& I, int& J) {
   J = t - i * (i + 1) / 2;
 }
 
-// Full matrix (and, if F_lo is given, its lo part) from packed tiles: one lower tile per
+// Full matrix (and, if Fp is given, its planes) from packed tiles: one lower tile per
 // block (32 x 8 threads), written in place and, off the diagonal, mirrored through shared
 // memory.
-__global__ void unpack_sym_kernel(const float* P, float* F, float* F_lo, int n, int64_t packed) {
+__global__ void unpack_sym_kernel(const float* P, float* F, Planes Fp, int n, int64_t packed) {
   __shared__ float tile[32][33];
   const int b = blockIdx.y;
   int I, J;
   tri_tile(blockIdx.x, I, J);
   const float* p = P + (int64_t)b * packed + (int64_t)blockIdx.x * 1024;
   float* f = F + (int64_t)b * n * n;
-  float* fl = F_lo ? F_lo + (int64_t)b * n * n : nullptr;
   for (int i = threadIdx.y; i < 32; i += 8) {
     const float x = p[i * 32 + threadIdx.x];
     tile[i][threadIdx.x] = x;
     const int r = I * 32 + i, c = J * 32 + threadIdx.x;
     if (r < n && c < n) {
       f[(int64_t)r * n + c] = x;
-      if (fl) fl[(int64_t)r * n + c] = lo_part(x);
+      if (Fp.p) b3_store(Fp.p + b * Fp.stride + r * Fp.ld + c, Fp.plane, x);
     }
   }
   if (I == J) return;  // uniform over the block
@@ -257,7 +285,7 @@ __global__ void unpack_sym_kernel(const float* P, float* F, float* F_lo, int n, 
     if (r < n && c < n) {
       const float x = tile[threadIdx.x][i];
       f[(int64_t)r * n + c] = x;
-      if (fl) fl[(int64_t)r * n + c] = lo_part(x);
+      if (Fp.p) b3_store(Fp.p + b * Fp.stride + r * Fp.ld + c, Fp.plane, x);
     }
   }
 }
@@ -306,106 +334,94 @@ __global__ void transpose_kernel(const float* src, float* dst, int rows, int col
   }
 }
 
-// Q -> Q_lo, Q^T, Q^T_lo for `batch` n x n matrices (32 x 32 tiles, 32 x 8 threads).
-__global__ void basis_split_kernel(const float* Q, float* Q_lo, float* Qt, float* Qt_lo, int n) {
-  __shared__ float tile[32][33];
+// The planes of X^T, and of X if Xp is given, and X^T itself if Xt is given, for `batch` n x n
+// matrices (n a multiple of 4), one 64 x 32 tile per block.
+__global__ void __launch_bounds__(256) planes_transpose_kernel(const float* X, Planes Xp, Planes Xtp, float* Xt, int n) {
+  __shared__ TileBuf tile;
   const int b = blockIdx.z;
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  const int r0 = blockIdx.y * kTr, c0 = blockIdx.x * kTc;
   const int64_t nn = (int64_t)n * n;
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int r = r0 + i, c = c0 + threadIdx.x;
-    float x = 0.f;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const TileIn t(i);
+    const int r = r0 + t.r, c = c0 + t.c;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
     if (r < n && c < n) {
-      const int64_t o = (int64_t)b * nn + (int64_t)r * n + c;
-      x = Q[o];
-      if (Q_lo) Q_lo[o] = lo_part(x);
+      x = *reinterpret_cast<const float4*>(X + b * nn + (int64_t)r * n + c);
+      if (Xp.p) b3_store4(Xp.p + b * Xp.stride + r * Xp.ld + c, Xp.plane, x);
     }
-    tile[i][threadIdx.x] = x;
+    tile.put(t, x);
   }
   __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int c = c0 + i, r = r0 + threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const TileOut t(i);
+    const int c = c0 + t.c, r = r0 + t.r;
     if (r < n && c < n) {
-      const float x = tile[threadIdx.x][i];
-      const int64_t o = (int64_t)b * nn + (int64_t)c * n + r;
-      Qt[o] = x;
-      Qt_lo[o] = lo_part(x);
+      const float4 x = tile.get(t);
+      if (Xtp.p) b3_store4(Xtp.p + b * Xtp.stride + c * Xtp.ld + r, Xtp.plane, x);
+      if (Xt) *reinterpret_cast<float4*>(Xt + b * nn + (int64_t)c * n + r) = x;
     }
   }
 }
 
-// From Q^T and its lo part (one group slice of `batch` n x n bases): a copy of both, and Q
-// with its lo part, 32 x 32 tiles (32 x 8 threads). Any output may be null.
-__global__ void basis_from_qt_kernel(const float* Qt, const float* Qt_lo, float* Qt_out, float* Qt_lo_out, float* Q,
-                                     float* Q_lo, int n) {
-  __shared__ float tile[32][33];
-  const int b = blockIdx.z;
-  const int64_t nn = (int64_t)n * n;
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int r = r0 + i, c = c0 + threadIdx.x;
-    float x = 0.f;
-    if (r < n && c < n) {
-      const int64_t o = (int64_t)b * nn + (int64_t)r * n + c;
-      x = Qt[o];
-      if (Qt_out) Qt_out[o] = x;
-      if (Qt_lo_out) Qt_lo_out[o] = lo_part(x);
-    }
-    tile[i][threadIdx.x] = x;
-  }
-  __syncthreads();
-  if (!Q) return;
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int c = c0 + i, r = r0 + threadIdx.x;
-    if (r < n && c < n) {
-      const float x = tile[threadIdx.x][i];
-      const int64_t o = (int64_t)b * nn + (int64_t)c * n + r;
-      Q[o] = x;
-      if (Q_lo) Q_lo[o] = lo_part(x);
-    }
-  }
-}
-
-// lam[b][i] = sum_k C[b][i][k] Qt[b][i][k] = (Q^T F Q)_ii for C = Q^T F: one warp per row.
-__global__ void diag_dot_kernel(const float* C, const float* Qt, float* lam, int n) {
+// lam[b][i] = sum_k C[b][i][k] Qt[b][i][k] = (Q^T F Q)_ii for C = Q^T F, Q^T as planes: one warp
+// per row.
+__global__ void diag_dot_kernel(const float* C, Planes Qt, float* lam, int n) {
   const int b = blockIdx.y;
   const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
   if (row >= n) return;
-  const int64_t off = (int64_t)b * n * n + (int64_t)row * n;
-  const float4* c = reinterpret_cast<const float4*>(C + off);
-  const float4* q = reinterpret_cast<const float4*>(Qt + off);
+  const float4* c = reinterpret_cast<const float4*>(C + (int64_t)b * n * n + (int64_t)row * n);
+  const __nv_bfloat16* q = Qt.p + b * Qt.stride + row * Qt.ld;
   float acc = 0.f;
   for (int k = lane; k < n / 4; k += 32) {
-    const float4 x = c[k], y = q[k];
-    acc = fmaf(x.x, y.x, acc);
-    acc = fmaf(x.y, y.y, acc);
-    acc = fmaf(x.z, y.z, acc);
-    acc = fmaf(x.w, y.w, acc);
+    const float4 x = c[k];
+    float y[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int pl = 2; pl >= 0; --pl) {  // the smallest plane first
+      const uint2 w = *reinterpret_cast<const uint2*>(q + pl * Qt.plane + 4 * k);
+      const float2 lo = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162&>(w.x));
+      const float2 hi = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162&>(w.y));
+      y[0] += lo.x;
+      y[1] += lo.y;
+      y[2] += hi.x;
+      y[3] += hi.y;
+    }
+    acc = fmaf(x.x, y[0], acc);
+    acc = fmaf(x.y, y[1], acc);
+    acc = fmaf(x.z, y[2], acc);
+    acc = fmaf(x.w, y[3], acc);
   }
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) lam[(int64_t)b * n + row] = acc;
 }
 
-// X[b][i][j] <- X[b][i][j] * sqrt(coef / (max(lam[b][j], 0) + eps)) and its lo part (cols a
-// multiple of 4, rows of 16-byte multiples).
-__global__ void scale_cols_split_kernel(float* X, float* X_lo, const float* lam, int rows, int cols, float coef,
+// The planes of X[b][i][j] * sqrt(coef / (max(lam[b][j], 0) + eps)) (cols a multiple of 4).
+__global__ void scale_cols_split_kernel(const float* X, Planes Xp, const float* lam, int rows, int cols, float coef,
                                         float eps) {
   const int b = blockIdx.y;
   const int64_t e4 = (int64_t)rows * cols / 4;
-  float4* x = reinterpret_cast<float4*>(X + (int64_t)b * rows * cols);
-  float4* xl = reinterpret_cast<float4*>(X_lo + (int64_t)b * rows * cols);
+  const float4* x = reinterpret_cast<const float4*>(X + (int64_t)b * rows * cols);
   const float* l = lam + (int64_t)b * cols;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < e4; i += stride) {
-    const int j = (int)((i * 4) % cols);
+    const int r = (int)(i * 4 / cols), j = (int)(i * 4 - (int64_t)r * cols);
     float4 v = x[i];
     v.x *= sqrtf(coef / (fmaxf(l[j], 0.f) + eps));
     v.y *= sqrtf(coef / (fmaxf(l[j + 1], 0.f) + eps));
     v.z *= sqrtf(coef / (fmaxf(l[j + 2], 0.f) + eps));
     v.w *= sqrtf(coef / (fmaxf(l[j + 3], 0.f) + eps));
-    x[i] = v;
-    xl[i] = make_float4(lo_part(v.x), lo_part(v.y), lo_part(v.z), lo_part(v.w));
+    b3_store4(Xp.p + b * Xp.stride + r * Xp.ld + j, Xp.plane, v);
+  }
+}
+
+// The planes of `rows` rows of cols values (cols a multiple of 4).
+__global__ void split_planes_kernel(const float* X, Planes Xp, int64_t rows, int cols) {
+  const int64_t e4 = rows * cols / 4, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < e4; i += stride) {
+    const int64_t r = i * 4 / cols, j = i * 4 - r * cols;
+    b3_store4(Xp.p + r * Xp.ld + j, Xp.plane, reinterpret_cast<const float4*>(X)[i]);
   }
 }
 
@@ -420,16 +436,18 @@ __global__ void split_kernel(const float* x, float* hi, float* lo, int64_t n) {
 
 }  // namespace
 
-cudaError_t momentum_split(const float* const* grads, float* Gn, float* Gn_lo, float* Gt, float* Gt_lo, float* Mhat,
-                           float* Mcopy, float* Mcopy_lo, int rows, int cols, int batch, float beta1,
-                           bool mhat_transposed, int* status, cudaStream_t s) {
+cudaError_t momentum_split(const float* const* grads, const Planes& Gn, const Planes& Gt, const Planes& Mc, float* Mhat,
+                           int rows, int cols, int batch, float beta1, bool mhat_transposed, int* status,
+                           cudaStream_t s) {
   if (rows <= 0 || cols <= 0 || batch <= 0) return cudaSuccess;
-  if (batch > 65535 || (rows + 31) / 32 > 65535) return cudaErrorInvalidValue;
+  if (batch > 65535 || (rows + kTr - 1) / kTr > 65535 || ((rows | cols) & 3)) return cudaErrorInvalidValue;
   const double e = (double)rows * cols * batch;
-  ProfScope prof(kFamElementwise, 3.0 * e, 36.0 * e, s);
-  dim3 grid((cols + 31) / 32, (rows + 31) / 32, batch);
-  momentum_split_kernel<<<grid, dim3(32, 8), 0, s>>>(grads, Gn, Gn_lo, Gt, Gt_lo, Mhat, Mcopy, Mcopy_lo, rows, cols,
-                                                     beta1, mhat_transposed ? 1 : 0, status);
+  ProfScope prof(kFamElementwise, 3.0 * e, 30.0 * e, s);
+  dim3 grid((cols + kTc - 1) / kTc, (rows + kTr - 1) / kTr, batch);
+  if (mhat_transposed)
+    momentum_split_kernel<true><<<grid, 256, 0, s>>>(grads, Gn, Gt, Mc, Mhat, rows, cols, beta1, status);
+  else
+    momentum_split_kernel<false><<<grid, 256, 0, s>>>(grads, Gn, Gt, Mc, Mhat, rows, cols, beta1, status);
   return cudaGetLastError();
 }
 
@@ -438,13 +456,13 @@ int64_t packed_floats(int n) {
   return t * (t + 1) / 2 * 1024;
 }
 
-cudaError_t unpack_sym(const float* P, float* F, float* F_lo, int n, int batch, cudaStream_t s) {
+cudaError_t unpack_sym(const float* P, float* F, const Planes& Fp, int n, int batch, cudaStream_t s) {
   if (n <= 0 || batch <= 0) return cudaSuccess;
   if (batch > 65535) return cudaErrorInvalidValue;
   const int64_t tiles = packed_floats(n) / 1024;
   const double e = (double)n * n * batch;
-  ProfScope prof(kFamElementwise, 0.0, (2.0 + (F_lo ? 8.0 : 4.0)) * e, s);
-  unpack_sym_kernel<<<dim3((unsigned)tiles, batch), dim3(32, 8), 0, s>>>(P, F, F_lo, n, packed_floats(n));
+  ProfScope prof(kFamElementwise, 0.0, (2.0 + (Fp.p ? 10.0 : 4.0)) * e, s);
+  unpack_sym_kernel<<<dim3((unsigned)tiles, batch), dim3(32, 8), 0, s>>>(P, F, Fp, n, packed_floats(n));
   return cudaGetLastError();
 }
 
@@ -480,22 +498,22 @@ cudaError_t transpose(const float* src, float* dst, int rows, int cols, int batc
   return cudaGetLastError();
 }
 
-cudaError_t basis_split(const float* Q, float* Q_lo, float* Qt, float* Qt_lo, int n, int batch, cudaStream_t s) {
+cudaError_t planes_transpose(const float* X, const Planes& Xp, const Planes& Xtp, float* Xt, int n, int batch,
+                             cudaStream_t s) {
   if (n <= 0 || batch <= 0) return cudaSuccess;
+  if ((n & 3) || batch > 65535) return cudaErrorInvalidValue;
   const double e = (double)n * n * batch;
-  ProfScope prof(kFamElementwise, 2.0 * e, (Q_lo ? 16.0 : 12.0) * e, s);
-  dim3 grid((n + 31) / 32, (n + 31) / 32, batch);
-  basis_split_kernel<<<grid, dim3(32, 8), 0, s>>>(Q, Q_lo, Qt, Qt_lo, n);
+  ProfScope prof(kFamElementwise, 0.0, (4.0 + (Xp.p ? 6 : 0) + (Xtp.p ? 6 : 0) + (Xt ? 4 : 0)) * e, s);
+  dim3 grid((n + kTc - 1) / kTc, (n + kTr - 1) / kTr, batch);
+  planes_transpose_kernel<<<grid, 256, 0, s>>>(X, Xp, Xtp, Xt, n);
   return cudaGetLastError();
 }
 
-cudaError_t basis_from_qt(const float* Qt, const float* Qt_lo, float* Qt_out, float* Qt_lo_out, float* Q, float* Q_lo,
-                          int n, int batch, cudaStream_t s) {
-  if (n <= 0 || batch <= 0) return cudaSuccess;
-  const double e = (double)n * n * batch;
-  ProfScope prof(kFamElementwise, 0.0, (4.0 + (Qt_out ? 4 : 0) + (Qt_lo_out ? 8 : 0) + (Q ? 4 : 0) + (Q_lo ? 4 : 0)) * e, s);
-  dim3 grid((n + 31) / 32, (n + 31) / 32, batch);
-  basis_from_qt_kernel<<<grid, dim3(32, 8), 0, s>>>(Qt, Qt_lo, Qt_out, Qt_lo_out, Q, Q_lo, n);
+cudaError_t split_planes(const float* X, const Planes& Xp, int64_t rows, int cols, cudaStream_t s) {
+  if (rows <= 0 || cols <= 0) return cudaSuccess;
+  if (cols & 3) return cudaErrorInvalidValue;
+  ProfScope prof(kFamElementwise, 0.0, 10.0 * rows * cols, s);
+  split_planes_kernel<<<blocks_for(rows * cols, 1), kThreads, 0, s>>>(X, Xp, rows, cols);
   return cudaGetLastError();
 }
 
@@ -507,22 +525,22 @@ cudaError_t split_tf32(const float* x, float* hi, float* lo, int64_t n, cudaStre
   return cudaGetLastError();
 }
 
-cudaError_t diag_dot(const float* C, const float* Qt, float* lam, int n, int batch, cudaStream_t s) {
+cudaError_t diag_dot(const float* C, const Planes& Qt, float* lam, int n, int batch, cudaStream_t s) {
   if (n <= 0 || batch <= 0) return cudaSuccess;
   if ((n & 3) || batch > 65535) return cudaErrorInvalidValue;
   const double e = (double)n * n * batch;
-  ProfScope prof(kFamElementwise, 2.0 * e, 8.0 * e, s);
+  ProfScope prof(kFamElementwise, 2.0 * e, 10.0 * e, s);
   diag_dot_kernel<<<dim3((n + 7) / 8, batch), 256, 0, s>>>(C, Qt, lam, n);
   return cudaGetLastError();
 }
 
-cudaError_t scale_cols_split(float* X, float* X_lo, const float* lam, int rows, int cols, int batch, float coef,
-                             float eps, cudaStream_t s) {
+cudaError_t scale_cols_split(const float* X, const Planes& Xp, const float* lam, int rows, int cols, int batch,
+                             float coef, float eps, cudaStream_t s) {
   const int64_t elems = (int64_t)rows * cols;
   if (elems <= 0 || batch <= 0) return cudaSuccess;
   if ((cols & 3) || batch > 65535) return cudaErrorInvalidValue;
-  ProfScope prof(kFamElementwise, 4.0 * elems * batch, 12.0 * elems * batch, s);
-  scale_cols_split_kernel<<<dim3(blocks_for(elems, batch), batch), kThreads, 0, s>>>(X, X_lo, lam, rows, cols, coef,
+  ProfScope prof(kFamElementwise, 4.0 * elems * batch, 10.0 * elems * batch, s);
+  scale_cols_split_kernel<<<dim3(blocks_for(elems, batch), batch), kThreads, 0, s>>>(X, Xp, lam, rows, cols, coef,
                                                                                      eps);
   return cudaGetLastError();
 }
@@ -538,14 +556,15 @@ cudaError_t momentum_and_copy(const float* const* grads, float* Gc, float* Mhat,
 
 cudaError_t adam_in_basis(float* Gp, const float* Mp, float* V, int rows, int cols, int batch,
                           float beta1, float beta2, float eps, float bc1, float bc2,
-                          const uint8_t* skipL, const uint8_t* skipR, float* N_lo, int* status,
+                          const uint8_t* skipL, const uint8_t* skipR, const Planes& Np, int* status,
                           cudaStream_t s) {
   (void)beta1;
   const int64_t elems = (int64_t)rows * cols;
   if (elems <= 0 || batch <= 0) return cudaSuccess;
-  ProfScope prof(kFamElementwise, 8.0 * elems * batch, (N_lo ? 24.0 : 20.0) * elems * batch, s);
+  if (Np.p && (cols & 3)) return cudaErrorInvalidValue;
+  ProfScope prof(kFamElementwise, 8.0 * elems * batch, (Np.p ? 22.0 : 20.0) * elems * batch, s);
   adam_kernel<<<dim3(blocks_for(elems, batch), batch), kThreads, 0, s>>>(
-      Gp, Mp, V, rows, cols, beta2, eps, 1.f / bc1, 1.f / sqrtf(bc2), skipL, skipR, N_lo, status);
+      Gp, Mp, V, rows, cols, beta2, eps, 1.f / bc1, 1.f / sqrtf(bc2), skipL, skipR, Np, status);
   return cudaGetLastError();
 }
 

@@ -677,6 +677,11 @@ void set_wait_limit(uint64_t ns, const int* hold) {
   g_hold.store(hold, std::memory_order_relaxed);
 }
 
+void get_wait_limit(uint64_t* ns, const int** hold) {
+  *ns = g_wait_ns.load(std::memory_order_relaxed);
+  *hold = g_hold.load(std::memory_order_relaxed);
+}
+
 cudaError_t gemm_tc_nt(int M, int N, int K, int batch, const TcOperand& A, const TcOperand& B,
                        const TcEpilogue& ep_in, cudaStream_t s, int family, float* split_ws, size_t split_ws_floats) {
   if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;

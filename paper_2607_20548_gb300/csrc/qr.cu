@@ -20,7 +20,7 @@
 //   then Q^T is accumulated backwards from diag(d) (d_j = sign of R_jj) one block at a
 //   time, Q^T <- Q^T (I - V T^T V^T):
 //       W = Qt_sub Vt^T ;  Qt_sub -= W VTq^T
-//   and Q = (Q^T)^T is written with its lo part.
+//   and Q = (Q^T)^T.
 //
 // The column loop's panel of an n x n matrix spans up to n positions; it is spread over a
 // thread-block cluster of ceil((n-k0)/512) CTAs (<= 16 for n <= 8192), 512 positions each, or,
@@ -1020,28 +1020,6 @@ __global__ void signed_identity_kernel(float* Qt, const float* d, int n) {
   }
 }
 
-// Q = (Q^T)^T and its lo part, 32 x 32 tiles through shared memory
-__global__ void transpose_out_kernel(const float* Qt, float* Q, float* Q_lo, int n) {
-  __shared__ float tile[32][33];
-  const int b = blockIdx.z;
-  const int64_t nn = (int64_t)n * n;
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int r = r0 + i, cc = c0 + threadIdx.x;
-    tile[i][threadIdx.x] = (r < n && cc < n) ? Qt[(int64_t)b * nn + (int64_t)r * n + cc] : 0.f;
-  }
-  __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int r = c0 + i, cc = r0 + threadIdx.x;
-    if (r < n && cc < n) {
-      const float x = tile[threadIdx.x][i];
-      const int64_t o = (int64_t)b * nn + (int64_t)r * n + cc;
-      Q[o] = x;
-      if (Q_lo) Q_lo[o] = tf32_lo(x);
-    }
-  }
-}
-
 // The panel kernel variant for this device: 512 positions per CTA in clusters of up to 16
 // where the device runs 16-CTA clusters of it, else 1024 positions in clusters of up to 8.
 struct PanelKernel {
@@ -1194,8 +1172,8 @@ void qr_input_buffers(void* workspace, int n, int batch, float** At) {
   *At = w.At;
 }
 
-cudaError_t qr_q_t(int n, int batch, float* Qt, float* Qt_lo, float* Q, float* Q_lo, uint8_t* skip, float tol,
-                   void* workspace, size_t workspace_bytes, int* status, cudaStream_t s, const QrLookahead* lah) {
+cudaError_t qr_q_t(int n, int batch, float* Q, uint8_t* skip, float tol, void* workspace, size_t workspace_bytes,
+                   int* status, cudaStream_t s, const QrLookahead* lah) {
   if (n <= 0 || batch <= 0) return cudaSuccess;
   if (n > 8192 || batch > 65535 || (n & 3)) return cudaErrorInvalidValue;
   // look-ahead: a second stream and its events given, and a workspace sized for it
@@ -1206,7 +1184,7 @@ cudaError_t qr_q_t(int n, int batch, float* Qt, float* Qt_lo, float* Q, float* Q
   size_t need = 0;
   Workspace w = carve(workspace, n, batch, &need, la);
   if (workspace_bytes < need) return cudaErrorInvalidValue;
-  if (!Qt) Qt = w.At;  // the Q accumulation may reuse the factored matrix's buffer
+  float* Qt = w.At;  // the Q accumulation reuses the factored matrix's buffer
   const int nblock = (n + NBO - 1) / NBO;
   const int64_t nn = (int64_t)n * n, thin = (int64_t)n * NBO, vq_stride = (int64_t)nblock * thin;
   cudaError_t e;
@@ -1370,10 +1348,7 @@ cudaError_t qr_q_t(int n, int batch, float* Qt, float* Qt_lo, float* Q, float* Q
     if (e != cudaSuccess) return e;
   }
   if (Q) {
-    ProfScope prof(kFamOther, 0, 12.0 * nn * batch, s);
-    dim3 grid((n + 31) / 32, (n + 31) / 32, batch);
-    transpose_out_kernel<<<grid, dim3(32, 8), 0, s>>>(Qt, Q, Q_lo, n);
-    e = cudaGetLastError();
+    e = planes_transpose(Qt, Planes(), Planes(), Q, n, batch, s);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
@@ -1385,10 +1360,10 @@ cudaError_t qr_q(int n, int batch, const float* P, float* Q, uint8_t* skip, floa
   size_t need = 0;
   Workspace w = carve(workspace, n, batch, &need, false);
   if (workspace_bytes < need || (n & 3)) return cudaErrorInvalidValue;
-  // At = P^T and its lo part
-  cudaError_t e = transpose(P, w.At, n, n, batch, s);
+  // At = P^T
+  cudaError_t e = planes_transpose(P, Planes(), Planes(), w.At, n, batch, s);
   if (e != cudaSuccess) return e;
-  return qr_q_t(n, batch, nullptr, nullptr, Q, nullptr, skip, tol, workspace, workspace_bytes, status, s, nullptr);
+  return qr_q_t(n, batch, Q, skip, tol, workspace, workspace_bytes, status, s, nullptr);
 }
 
 }  // namespace soap

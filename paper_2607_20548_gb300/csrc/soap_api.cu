@@ -4,8 +4,9 @@
 // (rows x cols), the factors L and R as packed lower-triangular tiles (half of a full matrix),
 // and the bases Q_L, Q_R. Matrices with the same (rows, cols, sides) form a class, whose state
 // sits in contiguous arenas ([count][...]). Everything a step forms from that state -- the
-// gradient copy G and G^T, every tensor-core operand's tf32 lo part, Q^T, the unpacked
-// factors, the QR's workspace and the rotation intermediates -- lives in one workspace arena.
+// tensor-core operands (G, G^T, M_hat, Q, Q^T, the factors, each as three bf16 planes), the
+// unpacked factors, the QR's workspace and the rotation intermediates -- lives in one workspace
+// arena.
 // A step walks the classes in slices (runs of consecutive matrices of one class) grouped into
 // waves: a wave's slices are laid out side by side in the arena, and the next wave reuses it.
 // When the whole model fits, there is one wave holding every class whole; otherwise the waves
@@ -77,12 +78,14 @@ struct View {
   float *Mhat = nullptr, *V = nullptr, *L = nullptr, *QL = nullptr, *R = nullptr, *QR = nullptr;
   uint8_t *skipL = nullptr, *skipR = nullptr;
   float *lamL = nullptr, *lamR = nullptr;
-  // workspace: [G | M_hat copy] (or G alone if tr) and [G^T] (or [G^T | M_hat^T copy]), lo parts
-  float *Gc = nullptr, *Gc_lo = nullptr, *Gt = nullptr, *Gt_lo = nullptr;
-  float *Mc = nullptr, *Mc_lo = nullptr;  // the M_hat copy inside Gc or Gt
-  // workspace: unpacked factors with lo parts, and the bases' lo parts and transposes
-  float *Lf = nullptr, *Lf_lo = nullptr, *QL_lo = nullptr, *QLt = nullptr, *QLt_lo = nullptr;
-  float *Rf = nullptr, *Rf_lo = nullptr, *QR_lo = nullptr, *QRt = nullptr, *QRt_lo = nullptr;
+  // workspace, CUDA-core path: the gradient copy
+  float* Gc = nullptr;
+  // workspace, tensor-core path, as planes: [G | M_hat] (or G alone if tr) and [G^T] (or
+  // [G^T | M_hat^T]); M_hat's part of them
+  soap::Planes Gn, Gt, Mc;
+  // workspace: the unpacked factors, and the planes of the factors, the bases and their transposes
+  float *Lf = nullptr, *Rf = nullptr;
+  soap::Planes Lp, QLp, QLt, Rp, QRp, QRt;
 };
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -115,34 +118,31 @@ size_t make_view(const ClassState& c, int cls, int first, int count, char* base,
     off += align256(floats * sizeof(float));
     return base ? reinterpret_cast<float*>(base + o) : nullptr;
   };
+  auto take_planes = [&](int64_t rows, int64_t cols, int64_t n_mat) {
+    const size_t o = off;
+    off += align256(soap::planes_bytes(rows, cols, n_mat));
+    return soap::planes_in(base ? base + o : nullptr, rows, cols, n_mat);
+  };
   const size_t cmn = (size_t)count * mn, cmm = (size_t)count * m * m, cnn = (size_t)count * n * n;
   if (!c.tc) {
     w.Gc = take(cmn);  // the gradient copy; M_hat stays where it is
     w.Lf = w.L;
     w.Rf = w.R;
   } else {
-    const size_t ga = c.tr ? cmn : 2 * cmn, ta = c.tr ? 2 * cmn : cmn;
-    w.Gc = take(ga);
-    w.Gc_lo = take(ga);
-    w.Gt = take(ta);
-    w.Gt_lo = take(ta);
-    if (base) {
-      w.Mc = c.tr ? w.Gt + cmn : w.Gc + cmn;
-      w.Mc_lo = c.tr ? w.Gt_lo + cmn : w.Gc_lo + cmn;
-    }
+    w.Gn = take_planes(m, n, c.tr ? count : 2 * (int64_t)count);
+    w.Gt = take_planes(n, m, c.tr ? 2 * (int64_t)count : count);
+    if (base) w.Mc = c.tr ? w.Gt.at(count) : w.Gn.at(count);
     if (c.left) {
       w.Lf = take(cmm);
-      w.Lf_lo = take(cmm);
-      w.QL_lo = take(cmm);
-      w.QLt = take(cmm);
-      w.QLt_lo = take(cmm);
+      w.Lp = take_planes(m, m, count);
+      w.QLp = take_planes(m, m, count);
+      w.QLt = take_planes(m, m, count);
     }
     if (c.right) {
       w.Rf = take(cnn);
-      w.Rf_lo = take(cnn);
-      w.QR_lo = take(cnn);
-      w.QRt = take(cnn);
-      w.QRt_lo = take(cnn);
+      w.Rp = take_planes(n, n, count);
+      w.QRp = take_planes(n, n, count);
+      w.QRt = take_planes(n, n, count);
     }
   }
   if (v) *v = w;
@@ -225,11 +225,10 @@ struct soap_s {
   float* X2 = nullptr;
   float* Gp = nullptr;   // [G' | m'] for the tensor-core path: Gp .. Gp + 2 * ws_mat
   float* Mp = nullptr;   // m' for the CUDA-core path (Gp + ws_mat)
-  float* YMt = nullptr;  // (G Q_R)^T and (M_hat Q_R)^T
-  float* YMt_lo = nullptr;
-  float* N_lo = nullptr;
-  float* Zt = nullptr;   // (N Q_R^T)^T
-  float* Zt_lo = nullptr;
+  // as planes: (G Q_R)^T and (M_hat Q_R)^T, N, and (N Q_R^T)^T
+  void* YMt = nullptr;
+  void* Np = nullptr;
+  void* Zt = nullptr;
   float* lam_ws = nullptr;  // Q^T F of the KL form's eigenvalue estimate (two-sided classes)
   size_t ws_mat = 0;
   size_t rot_bytes = 0;
@@ -305,14 +304,26 @@ void free_all(soap_handle h) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-soap::TcOperand opnd(const float* hi, const float* lo, int64_t ld, int64_t stride, int batch) {
-  return soap::TcOperand{hi, lo, ld, stride, batch};
+soap::B3Epilogue epi(soap_handle h, float* C, int64_t ldc, int64_t c_stride, int transpose, float alpha, float beta) {
+  soap::B3Epilogue e{};
+  e.C = C;
+  e.ldc = ldc;
+  e.c_stride = c_stride;
+  e.transpose = transpose;
+  e.alpha = alpha;
+  e.beta = beta;
+  e.status = h->d_status;
+  return e;
 }
-
-soap::TcEpilogue epi(soap_handle h, float* C, int64_t ldc, int64_t c_stride, float* C_lo, int transpose, float alpha,
-                     float beta) {
-  return soap::TcEpilogue{C, nullptr, ldc, c_stride, C_lo, ldc, c_stride, transpose, alpha, beta, h->d_status};
+soap::B3Epilogue epi(soap_handle h, const soap::Planes& P, int transpose) {
+  soap::B3Epilogue e = epi(h, nullptr, 0, 0, transpose, 1.f, 0.f);
+  e.P = P.p;
+  e.p_plane = P.plane;
+  e.p_ld = P.ld;
+  e.p_stride = P.stride;
+  return e;
 }
+using soap::b3_op;
 
 View view_of(soap_handle h, const Wave& w, const Slice& sl) {
   View v;
@@ -346,22 +357,32 @@ soap_status_t prepare(soap_handle h, const ClassState& c, const View& v, const f
     SOAP_CUDA(h, soap::momentum_and_copy(d_grads, v.Gc, v.Mhat, mn, B, hp.beta1, h->d_status, s));
     return SOAP_OK;
   }
-  SOAP_CUDA(h, soap::momentum_split(d_grads, v.Gc, v.Gc_lo, v.Gt, v.Gt_lo, v.Mhat, v.Mc, v.Mc_lo, m, n, B, hp.beta1,
-                                    c.tr, h->d_status, s));
-  // the factors' lo parts are read before S1 rewrites them by the KL form's eigenvalue product
+  SOAP_CUDA(h, soap::momentum_split(d_grads, v.Gn, v.Gt, v.Mc, v.Mhat, m, n, B, hp.beta1, c.tr, h->d_status, s));
+  // the factors' planes are read before S1 rewrites them by the KL form's eigenvalue product
   // and by the stale variant's refresh
-  const bool lo = hp.kl || hp.stale;
-  // Q^T and its lo part feed S2 (and the KL eigenvalues); Q's own lo part only the rotations,
-  // for which a refresh writes it anew
+  const bool fp = hp.kl || hp.stale;
+  // Q^T's planes feed S2 (and the KL eigenvalues); Q's own only the rotations, for which a refresh
+  // writes them anew
   if (c.left) {
-    SOAP_CUDA(h, soap::basis_split(v.QL, refresh ? nullptr : v.QL_lo, v.QLt, v.QLt_lo, m, B, s));
-    SOAP_CUDA(h, soap::unpack_sym(v.L, v.Lf, lo ? v.Lf_lo : nullptr, m, B, s));
+    SOAP_CUDA(h, soap::planes_transpose(v.QL, refresh ? soap::Planes() : v.QLp, v.QLt, nullptr, m, B, s));
+    SOAP_CUDA(h, soap::unpack_sym(v.L, v.Lf, fp ? v.Lp : soap::Planes(), m, B, s));
   }
   if (c.right) {
-    SOAP_CUDA(h, soap::basis_split(v.QR, refresh ? nullptr : v.QR_lo, v.QRt, v.QRt_lo, n, B, s));
-    SOAP_CUDA(h, soap::unpack_sym(v.R, v.Rf, lo ? v.Rf_lo : nullptr, n, B, s));
+    SOAP_CUDA(h, soap::planes_transpose(v.QR, refresh ? soap::Planes() : v.QRp, v.QRt, nullptr, n, B, s));
+    SOAP_CUDA(h, soap::unpack_sym(v.R, v.Rf, fp ? v.Rp : soap::Planes(), n, B, s));
   }
   return SOAP_OK;
+}
+
+// F <- alpha A A^T + beta F in fp32, and F's planes
+soap::B3Epilogue factor_epi(soap_handle h, float* F, const soap::Planes& Fp, int n, float alpha, float beta) {
+  soap::B3Epilogue e = epi(h, Fp, 0);
+  e.C = F;
+  e.ldc = n;
+  e.c_stride = (int64_t)n * n;
+  e.alpha = alpha;
+  e.beta = beta;
+  return e;
 }
 
 // S1 for one slice (after prepare): the standard factor EMAs, or Alg. 1's KL form, on the
@@ -393,35 +414,27 @@ soap_status_t accumulate_factors(soap_handle h, const ClassState& c, const View&
     //   Y = G Q_R diag(sqrt(w_R)),  w_R = (1-b) / (cols (lam_R + eps))
     //   X = G^T Q_L diag(sqrt(w_L)), w_L = (1-b) / (rows (lam_L + eps))
     //   L <- b L + Y Y^T,  R <- b R + X X^T
-    // Y and X (with their lo parts) live in the rotation workspace, free until phase C.
+    // Y and X and their planes live in the rotation workspace, free until phase C.
     const int64_t cls = (int64_t)B * mn;
     float* C = h->lam_ws;
-    SOAP_CUDA(h, soap::gemm_tc_nt(m, m, m, B, opnd(v.QLt, v.QLt_lo, m, mm, B), opnd(v.Lf, v.Lf_lo, m, mm, B),
-                                  epi(h, C, m, mm, nullptr, 0, 1.f, 0.f), s));
+    SOAP_CUDA(h, soap::gemm_b3(m, m, m, B, b3_op(v.QLt, B), b3_op(v.Lp, B), epi(h, C, m, mm, 0, 1.f, 0.f), s));
     SOAP_CUDA(h, soap::diag_dot(C, v.QLt, v.lamL, m, B, s));
-    SOAP_CUDA(h, soap::gemm_tc_nt(n, n, n, B, opnd(v.QRt, v.QRt_lo, n, nn, B), opnd(v.Rf, v.Rf_lo, n, nn, B),
-                                  epi(h, C, n, nn, nullptr, 0, 1.f, 0.f), s));
+    SOAP_CUDA(h, soap::gemm_b3(n, n, n, B, b3_op(v.QRt, B), b3_op(v.Rp, B), epi(h, C, n, nn, 0, 1.f, 0.f), s));
     SOAP_CUDA(h, soap::diag_dot(C, v.QRt, v.lamR, n, B, s));
-    float* Y = h->YMt;
-    float* Y_lo = h->YMt_lo;
-    float* X = h->YMt + cls;
-    float* X_lo = h->YMt_lo + cls;
-    SOAP_CUDA(h, soap::gemm_tc_nt(m, n, n, B, opnd(v.Gc, v.Gc_lo, n, mn, B), opnd(v.QRt, v.QRt_lo, n, nn, B),
-                                  epi(h, Y, n, mn, nullptr, 0, 1.f, 0.f), s));
-    SOAP_CUDA(h, soap::scale_cols_split(Y, Y_lo, v.lamR, m, n, B, (float)((1.0 - fb) / n), hp.eps, s));
-    SOAP_CUDA(h, soap::gemm_tc_nt(n, m, m, B, opnd(v.Gt, v.Gt_lo, m, mn, B), opnd(v.QLt, v.QLt_lo, m, mm, B),
-                                  epi(h, X, m, mn, nullptr, 0, 1.f, 0.f), s));
-    SOAP_CUDA(h, soap::scale_cols_split(X, X_lo, v.lamL, n, m, B, (float)((1.0 - fb) / m), hp.eps, s));
-    SOAP_CUDA(h, soap::gemm_tc_syrk(m, n, B, opnd(Y, Y_lo, n, mn, B), epi(h, v.Lf, m, mm, v.Lf_lo, 0, 1.f, fb), s));
-    SOAP_CUDA(h, soap::gemm_tc_syrk(n, m, B, opnd(X, X_lo, m, mn, B), epi(h, v.Rf, n, nn, v.Rf_lo, 0, 1.f, fb), s));
+    float* Y = h->Gp;
+    float* X = h->Gp + cls;
+    const soap::Planes Yp = soap::planes_in(h->YMt, m, n, B);
+    const soap::Planes Xp = soap::planes_in(static_cast<char*>(h->YMt) + soap::planes_bytes(m, n, B), n, m, B);
+    SOAP_CUDA(h, soap::gemm_b3(m, n, n, B, b3_op(v.Gn, B), b3_op(v.QRt, B), epi(h, Y, n, mn, 0, 1.f, 0.f), s));
+    SOAP_CUDA(h, soap::scale_cols_split(Y, Yp, v.lamR, m, n, B, (float)((1.0 - fb) / n), hp.eps, s));
+    SOAP_CUDA(h, soap::gemm_b3(n, m, m, B, b3_op(v.Gt, B), b3_op(v.QLt, B), epi(h, X, m, mn, 0, 1.f, 0.f), s));
+    SOAP_CUDA(h, soap::scale_cols_split(X, Xp, v.lamL, n, m, B, (float)((1.0 - fb) / m), hp.eps, s));
+    SOAP_CUDA(h, soap::gemm_b3_syrk(m, n, B, b3_op(Yp, B), factor_epi(h, v.Lf, v.Lp, m, 1.f, fb), s));
+    SOAP_CUDA(h, soap::gemm_b3_syrk(n, m, B, b3_op(Xp, B), factor_epi(h, v.Rf, v.Rp, n, 1.f, fb), s));
   } else {
     // S1 as symmetric products: the lower tiles of G G^T (G^T G), mirrored
-    if (c.left)
-      SOAP_CUDA(h, soap::gemm_tc_syrk(m, n, B, opnd(v.Gc, v.Gc_lo, n, mn, B), epi(h, v.Lf, m, mm, v.Lf_lo, 0, aL, fb),
-                                      s));
-    if (c.right)
-      SOAP_CUDA(h, soap::gemm_tc_syrk(n, m, B, opnd(v.Gt, v.Gt_lo, m, mn, B), epi(h, v.Rf, n, nn, v.Rf_lo, 0, aR, fb),
-                                      s));
+    if (c.left) SOAP_CUDA(h, soap::gemm_b3_syrk(m, n, B, b3_op(v.Gn, B), factor_epi(h, v.Lf, v.Lp, m, aL, fb), s));
+    if (c.right) SOAP_CUDA(h, soap::gemm_b3_syrk(n, m, B, b3_op(v.Gt, B), factor_epi(h, v.Rf, v.Rp, n, aR, fb), s));
   }
   if (c.left) SOAP_CUDA(h, soap::pack_sym(v.Lf, v.L, m, B, s));
   if (c.right) SOAP_CUDA(h, soap::pack_sym(v.Rf, v.R, n, B, s));
@@ -452,10 +465,8 @@ soap_status_t refresh_group(soap_handle h, const Wave& w, const QrGroup& g, cuda
     const View v = view_of(h, w, sl);
     float* at = At + (int64_t)j.offset * nn;
     if (c.tc) {
-      SOAP_CUDA(h, soap::gemm_tc_nt(n, n, n, v.count, opnd(j.left ? v.QLt : v.QRt, j.left ? v.QLt_lo : v.QRt_lo, n, nn,
-                                                           v.count),
-                                    opnd(j.left ? v.Lf : v.Rf, j.left ? v.Lf_lo : v.Rf_lo, n, nn, v.count),
-                                    epi(h, at, n, nn, nullptr, 0, 1.f, 0.f), gs.stream));
+      SOAP_CUDA(h, soap::gemm_b3(n, n, n, v.count, b3_op(j.left ? v.QLt : v.QRt, v.count),
+                                 b3_op(j.left ? v.Lp : v.Rp, v.count), epi(h, at, n, nn, 0, 1.f, 0.f), gs.stream));
     } else {
       SOAP_CUDA(h, soap::gemm(true, false, n, n, n, 1.f, strided(j.left ? v.QL : v.QR, n, nn),
                               strided(j.left ? v.L : v.R, n, nn), 0.f, strided_mut(at, n, nn), v.count, gs.stream));
@@ -463,19 +474,15 @@ soap_status_t refresh_group(soap_handle h, const Wave& w, const QrGroup& g, cuda
   }
   // the Q accumulation ends with Q^T in the input buffers
   const soap::QrLookahead la{gs.far, gs.ev_vt, gs.ev_far, {gs.ev_vq[0], gs.ev_vq[1]}};
-  SOAP_CUDA(h, soap::qr_q_t(n, g.batch, nullptr, nullptr, nullptr, nullptr, skip, hp.qr_tol, ws, g.ws_bytes,
-                            h->d_status, gs.stream, &la));
+  SOAP_CUDA(h, soap::qr_q_t(n, g.batch, nullptr, skip, hp.qr_tol, ws, g.ws_bytes, h->d_status, gs.stream, &la));
   for (const QrJob& j : g.jobs) {
     const Slice& sl = w.slices[j.slice];
     const ClassState& c = h->classes[sl.cls];
     const View v = view_of(h, w, sl);
     const float* qt = At + (int64_t)j.offset * nn;
     float* Q = j.left ? v.QL : v.QR;
-    if (c.tc)
-      SOAP_CUDA(h, soap::basis_from_qt(qt, nullptr, j.left ? v.QLt : v.QRt, j.left ? v.QLt_lo : v.QRt_lo, Q,
-                                       j.left ? v.QL_lo : v.QR_lo, n, v.count, gs.stream));
-    else
-      SOAP_CUDA(h, soap::basis_from_qt(qt, nullptr, nullptr, nullptr, Q, nullptr, n, v.count, gs.stream));
+    // (views of a CUDA-core slice have no planes: Q alone is written)
+    SOAP_CUDA(h, soap::planes_transpose(qt, j.left ? v.QLt : v.QRt, j.left ? v.QLp : v.QRp, Q, n, v.count, gs.stream));
     SOAP_CUDA(h, cudaMemcpyAsync(j.left ? v.skipL : v.skipR, skip + (int64_t)j.offset * n, (size_t)v.count * n,
                                  cudaMemcpyDeviceToDevice, gs.stream));
   }
@@ -497,38 +504,31 @@ soap_status_t rotate_update(soap_handle h, const ClassState& c, const View& v, f
     //   N = Adam(G', m', v)
     //   W <- (1 - lr wd) W - lr N Q^T  A = N,  B = Q   (epilogue into W, transposed if c.tr)
     const int rr = c.tr ? n : m, cc = c.tr ? m : n;
-    const int64_t cls = (int64_t)B * mn, qq = (int64_t)cc * cc;
-    const float* X = c.tr ? v.Gt : v.Gc;
-    const float* X_lo = c.tr ? v.Gt_lo : v.Gc_lo;
-    const float* Q = c.tr ? v.QL : v.QR;
-    const float* Q_lo = c.tr ? v.QL_lo : v.QR_lo;
-    const float* Qt = c.tr ? v.QLt : v.QRt;
-    const float* Qt_lo = c.tr ? v.QLt_lo : v.QRt_lo;
-    SOAP_CUDA(h, soap::gemm_tc_nt(rr, cc, cc, 2 * B, opnd(X, X_lo, cc, mn, 2 * B), opnd(Qt, Qt_lo, cc, qq, B),
-                                  epi(h, h->Gp, cc, mn, nullptr, 0, 1.f, 0.f), s));
+    const int64_t cls = (int64_t)B * mn;
+    const soap::Planes N = soap::planes_in(h->Np, rr, cc, B);
+    SOAP_CUDA(h, soap::gemm_b3(rr, cc, cc, 2 * B, b3_op(c.tr ? v.Gt : v.Gn, 2 * B), b3_op(c.tr ? v.QLt : v.QRt, B),
+                               epi(h, h->Gp, cc, mn, 0, 1.f, 0.f), s));
     const uint8_t* skip = hp.guard ? (c.tr ? v.skipL : v.skipR) : nullptr;
     SOAP_CUDA(h, soap::adam_in_basis(h->Gp, h->Gp + cls, v.V, rr, cc, B, hp.beta1, hp.beta2, hp.eps, bc1, bc2, nullptr,
-                                     skip, h->N_lo, h->d_status, s));
-    soap::TcEpilogue ew = epi(h, nullptr, n, 0, nullptr, c.tr ? 1 : 0, -h->lr, 1.f - h->lr * h->wd);
+                                     skip, N, h->d_status, s));
+    soap::B3Epilogue ew = epi(h, nullptr, n, 0, c.tr ? 1 : 0, -h->lr, 1.f - h->lr * h->wd);
     ew.C_ptrs = d_params;
-    SOAP_CUDA(h, soap::gemm_tc_nt(rr, cc, cc, B, opnd(h->Gp, h->N_lo, cc, mn, B), opnd(Q, Q_lo, cc, qq, B), ew, s));
+    SOAP_CUDA(h, soap::gemm_b3(rr, cc, cc, B, b3_op(N, B), b3_op(c.tr ? v.QLp : v.QRp, B), ew, s));
     return SOAP_OK;
   }
   if (c.tc) {
     const int64_t cls = (int64_t)B * mn;
+    const soap::Planes YMt = soap::planes_in(h->YMt, n, m, 2 * (int64_t)B), N = soap::planes_in(h->Np, m, n, B),
+                       Zt = soap::planes_in(h->Zt, n, m, B);
     // rotations of the gradient and of the momentum in one launch each (batch 2B)
-    SOAP_CUDA(h, soap::gemm_tc_nt(m, n, n, 2 * B, opnd(v.Gc, v.Gc_lo, n, mn, 2 * B), opnd(v.QRt, v.QRt_lo, n, nn, B),
-                                  epi(h, h->YMt, m, mn, h->YMt_lo, 1, 1.f, 0.f), s));
-    SOAP_CUDA(h, soap::gemm_tc_nt(m, n, m, 2 * B, opnd(v.QLt, v.QLt_lo, m, mm, B),
-                                  opnd(h->YMt, h->YMt_lo, m, mn, 2 * B), epi(h, h->Gp, n, mn, nullptr, 0, 1.f, 0.f), s));
+    SOAP_CUDA(h, soap::gemm_b3(m, n, n, 2 * B, b3_op(v.Gn, 2 * B), b3_op(v.QRt, B), epi(h, YMt, 1), s));
+    SOAP_CUDA(h, soap::gemm_b3(m, n, m, 2 * B, b3_op(v.QLt, B), b3_op(YMt, 2 * B), epi(h, h->Gp, n, mn, 0, 1.f, 0.f), s));
     SOAP_CUDA(h, soap::adam_in_basis(h->Gp, h->Gp + cls, v.V, m, n, B, hp.beta1, hp.beta2, hp.eps, bc1, bc2,
-                                     hp.guard ? v.skipL : nullptr, hp.guard ? v.skipR : nullptr, h->N_lo, h->d_status,
-                                     s));
-    SOAP_CUDA(h, soap::gemm_tc_nt(m, n, n, B, opnd(h->Gp, h->N_lo, n, mn, B), opnd(v.QR, v.QR_lo, n, nn, B),
-                                  epi(h, h->Zt, m, mn, h->Zt_lo, 1, 1.f, 0.f), s));
-    soap::TcEpilogue ew = epi(h, nullptr, n, 0, nullptr, 0, -h->lr, 1.f - h->lr * h->wd);
+                                     hp.guard ? v.skipL : nullptr, hp.guard ? v.skipR : nullptr, N, h->d_status, s));
+    SOAP_CUDA(h, soap::gemm_b3(m, n, n, B, b3_op(N, B), b3_op(v.QRp, B), epi(h, Zt, 1), s));
+    soap::B3Epilogue ew = epi(h, nullptr, n, 0, 0, -h->lr, 1.f - h->lr * h->wd);
     ew.C_ptrs = d_params;
-    SOAP_CUDA(h, soap::gemm_tc_nt(m, n, m, B, opnd(v.QL, v.QL_lo, m, mm, B), opnd(h->Zt, h->Zt_lo, m, mn, B), ew, s));
+    SOAP_CUDA(h, soap::gemm_b3(m, n, m, B, b3_op(v.QLp, B), b3_op(Zt, B), ew, s));
     return SOAP_OK;
   }
   // S5 and the re-projected first moment: G' = Q_L^T G Q_R, m = Q_L^T M_hat Q_R
@@ -558,7 +558,7 @@ soap_status_t rotate_update(soap_handle h, const ClassState& c, const View& v, f
   // S6
   SOAP_CUDA(h, soap::adam_in_basis(gp, mp, v.V, m, n, B, hp.beta1, hp.beta2, hp.eps, bc1, bc2,
                                    (hp.guard && c.left) ? v.skipL : nullptr, (hp.guard && c.right) ? v.skipR : nullptr,
-                                   nullptr, h->d_status, s));
+                                   soap::Planes(), h->d_status, s));
   // S7 + S8: W <- (1 - lr wd) W - lr Q_L N Q_R^T
   const float keep = 1.f - h->lr * h->wd;
   soap::MutOperand W{nullptr, d_params, 0, 0, n};
@@ -582,27 +582,36 @@ int largest_side(const ClassState& c) {
   return (int)std::max(c.left ? c.rows : (int64_t)0, c.right ? c.cols : (int64_t)0);
 }
 
-// Rotation intermediates (floats) that a slice of `count` matrices of class c needs.
+// Rotation intermediates that a slice of `count` matrices of class c needs: floats (mat, x, lam) and
+// bytes of planes.
 struct RotSizes {
-  size_t mat = 0, tc = 0, two = 0, x = 0, lam = 0;
+  size_t mat = 0, x = 0, lam = 0, n_planes = 0, ym_planes = 0, z_planes = 0;
   void grow(const RotSizes& o) {
     mat = std::max(mat, o.mat);
-    tc = std::max(tc, o.tc);
-    two = std::max(two, o.two);
     x = std::max(x, o.x);
     lam = std::max(lam, o.lam);
+    n_planes = std::max(n_planes, o.n_planes);
+    ym_planes = std::max(ym_planes, o.ym_planes);
+    z_planes = std::max(z_planes, o.z_planes);
   }
-  size_t bytes() const { return 4 * (2 * mat + tc + 4 * two + 2 * two + 2 * x + lam) + 16 * 256; }
+  size_t bytes() const { return 4 * (2 * mat + 2 * x + lam) + n_planes + ym_planes + z_planes + 16 * 256; }
 };
 RotSizes rot_sizes(const ClassState& c, int count, bool kl) {
   RotSizes r;
   const size_t mn = (size_t)count * c.rows * c.cols;
   r.mat = mn;
-  if (c.tc) r.tc = mn;
-  if (c.tc && c.left && c.right) r.two = mn;
+  const bool two = c.tc && c.left && c.right;
+  if (c.tc) r.n_planes = c.tr ? soap::planes_bytes(c.cols, c.rows, count) : soap::planes_bytes(c.rows, c.cols, count);
+  if (two) {
+    // (G Q_R)^T and (M_hat Q_R)^T; the KL form's Y and X
+    r.ym_planes = soap::planes_bytes(c.cols, c.rows, 2 * (int64_t)count);
+    if (kl)
+      r.ym_planes = std::max(r.ym_planes, soap::planes_bytes(c.rows, c.cols, count) + soap::planes_bytes(c.cols, c.rows, count));
+    r.z_planes = soap::planes_bytes(c.cols, c.rows, count);
+  }
   // X1/X2: a CUDA-core slice's intermediates, or one matrix (state reads and writes)
   r.x = c.tc ? (size_t)(c.rows * c.cols) : mn;
-  if (kl && c.tc && c.left && c.right) r.lam = (size_t)count * std::max(c.rows * c.rows, c.cols * c.cols);
+  if (kl && two) r.lam = (size_t)count * std::max(c.rows * c.rows, c.cols * c.cols);
   return r;
 }
 
@@ -898,8 +907,8 @@ soap_status_t soap_create_ex(const soap_shape* shapes, int32_t n, const soap_hpa
     for (cudaEvent_t* ev : {&gs.done, &gs.fork, &gs.ev_vt, &gs.ev_far, &gs.ev_vq[0], &gs.ev_vq[1]})
       if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
   }
-  // rotation intermediates: [G' | m'] for every slice; N's lo part for tensor-core slices; the
-  // intermediate products of two-sided tensor-core slices; X1/X2 for CUDA-core slices and for
+  // rotation intermediates: [G' | m'] for every slice; N's planes for tensor-core slices; the
+  // planes of the intermediate products of two-sided tensor-core slices; X1/X2 for CUDA-core slices and for
   // single-matrix state reads and writes; Q^T F for the KL form's eigenvalues
   h->ws_mat = rot.mat;
   h->rot_bytes = rot.bytes();
@@ -907,11 +916,9 @@ soap_status_t soap_create_ex(const soap_shape* shapes, int32_t n, const soap_hpa
   if (e == cudaSuccess) e = dalloc(h, (void**)&h->X2, rot.x * 4);
   if (e == cudaSuccess) e = dalloc(h, (void**)&h->Gp, 2 * rot.mat * 4);
   h->Mp = h->Gp ? h->Gp + rot.mat : nullptr;
-  if (e == cudaSuccess) e = dalloc(h, (void**)&h->N_lo, rot.tc * 4);
-  if (e == cudaSuccess) e = dalloc(h, (void**)&h->YMt, 2 * rot.two * 4);
-  if (e == cudaSuccess) e = dalloc(h, (void**)&h->YMt_lo, 2 * rot.two * 4);
-  if (e == cudaSuccess) e = dalloc(h, (void**)&h->Zt, rot.two * 4);
-  if (e == cudaSuccess) e = dalloc(h, (void**)&h->Zt_lo, rot.two * 4);
+  if (e == cudaSuccess) e = dalloc(h, &h->Np, rot.n_planes);
+  if (e == cudaSuccess) e = dalloc(h, &h->YMt, rot.ym_planes);
+  if (e == cudaSuccess) e = dalloc(h, &h->Zt, rot.z_planes);
   if (e == cudaSuccess) e = dalloc(h, (void**)&h->lam_ws, rot.lam * 4);
   if (e != cudaSuccess) {
     soap_status_t code = e == cudaErrorMemoryAllocation ? SOAP_ERR_OOM : SOAP_ERR_CUDA;
@@ -1161,7 +1168,7 @@ soap_status_t state_get_impl(soap_handle h, int32_t idx, int32_t which, void* ds
     const bool left = which == SOAP_STATE_L;
     const float* F = left ? v.L : v.R;
     if (c.tc) {
-      SOAP_CUDA(h, soap::unpack_sym(F, left ? v.Lf : v.Rf, nullptr, left ? m : nc, 1, s));
+      SOAP_CUDA(h, soap::unpack_sym(F, left ? v.Lf : v.Rf, soap::Planes(), left ? m : nc, 1, s));
       F = left ? v.Lf : v.Rf;
     }
     SOAP_CUDA(h, cudaMemcpyAsync(dst, F, bytes, cudaMemcpyDefault, s));
@@ -1174,28 +1181,23 @@ soap_status_t state_get_impl(soap_handle h, int32_t idx, int32_t which, void* ds
   // m = Q_L^T M_hat Q_R, computed into the workspace with the operands and products of the step
   const float* x = v.Mhat;
   if (c.tc) {
-    if (c.left) SOAP_CUDA(h, soap::basis_split(v.QL, v.QL_lo, v.QLt, v.QLt_lo, m, 1, s));
-    if (c.right) SOAP_CUDA(h, soap::basis_split(v.QR, v.QR_lo, v.QRt, v.QRt_lo, nc, 1, s));
-    float* x_lo = v.Mc_lo;
-    SOAP_CUDA(h, soap::split_tf32(x, nullptr, x_lo, mn, s));
+    if (c.left) SOAP_CUDA(h, soap::planes_transpose(v.QL, soap::Planes(), v.QLt, nullptr, m, 1, s));
+    if (c.right) SOAP_CUDA(h, soap::planes_transpose(v.QR, soap::Planes(), v.QRt, nullptr, nc, 1, s));
+    SOAP_CUDA(h, soap::split_planes(x, v.Mc, c.tr ? nc : m, c.tr ? m : nc, s));
     if (!(c.left && c.right)) {
       // the step's product [X | M_hat] Q for this matrix alone (bit-identical), written in the
       // original orientation
       const int rr = c.tr ? nc : m, cc = c.tr ? m : nc;
-      const int64_t qq = (int64_t)cc * cc;
-      SOAP_CUDA(h, soap::gemm_tc_nt(rr, cc, cc, 1, opnd(x, x_lo, cc, mn, 1),
-                                    opnd(c.tr ? v.QLt : v.QRt, c.tr ? v.QLt_lo : v.QRt_lo, cc, qq, 1),
-                                    epi(h, h->Gp, c.tr ? rr : cc, mn, nullptr, c.tr ? 1 : 0, 1.f, 0.f), s));
+      SOAP_CUDA(h, soap::gemm_b3(rr, cc, cc, 1, b3_op(v.Mc, 1), b3_op(c.tr ? v.QLt : v.QRt, 1),
+                                 epi(h, h->Gp, c.tr ? rr : cc, mn, c.tr ? 1 : 0, 1.f, 0.f), s));
       SOAP_CUDA(h, cudaMemcpyAsync(dst, h->Gp, bytes, cudaMemcpyDefault, s));
       return SOAP_OK;
     }
     // the same tensor-core products, on the same operands, as the step's rotation of M_hat:
     // bit-identical to the m the last step used
-    const int64_t mm = (int64_t)m * m, nn = (int64_t)nc * nc;
-    SOAP_CUDA(h, soap::gemm_tc_nt(m, nc, nc, 1, opnd(x, x_lo, nc, mn, 1), opnd(v.QRt, v.QRt_lo, nc, nn, 1),
-                                  epi(h, h->X1, m, mn, h->X2, 1, 1.f, 0.f), s));
-    SOAP_CUDA(h, soap::gemm_tc_nt(m, nc, m, 1, opnd(v.QLt, v.QLt_lo, m, mm, 1), opnd(h->X1, h->X2, m, mn, 1),
-                                  epi(h, h->Gp, nc, mn, nullptr, 0, 1.f, 0.f), s));
+    const soap::Planes Yt = soap::planes_in(h->YMt, nc, m, 1);
+    SOAP_CUDA(h, soap::gemm_b3(m, nc, nc, 1, b3_op(v.Mc, 1), b3_op(v.QRt, 1), epi(h, Yt, 1), s));
+    SOAP_CUDA(h, soap::gemm_b3(m, nc, m, 1, b3_op(v.QLt, 1), b3_op(Yt, 1), epi(h, h->Gp, nc, mn, 0, 1.f, 0.f), s));
     SOAP_CUDA(h, cudaMemcpyAsync(dst, h->Gp, bytes, cudaMemcpyDefault, s));
     return SOAP_OK;
   }

@@ -89,6 +89,92 @@ void set_wait_limit(uint64_t ns, const int* hold);
 // position. Needs a row-major, 16-byte aligned C with its lo part; other forms go to gemm_tc_nt.
 cudaError_t gemm_tc_syrk(int M, int K, int batch, const TcOperand& A, const TcEpilogue& ep, cudaStream_t stream,
                          int family = kFamGemmTc);
+// The settings in force (0: the default bound).
+void get_wait_limit(uint64_t* ns, const int** hold);
+
+// ---- fp32-accurate products of operands kept as three bf16 planes (gemm_b3.cu) -----------------
+// x = h + m + l to 2^-26, each plane the rounding to nearest bf16 of what the ones before it leave.
+// `count` row-major rows x cols matrices as planes: element (i, j) of matrix b of plane q at
+// q * plane + b * stride + i * ld + j; rows start on 16 bytes (TMA).
+inline int64_t plane_ld(int64_t cols) { return (cols + 7) & ~(int64_t)7; }
+struct Planes {
+  __nv_bfloat16* p = nullptr;
+  int64_t plane = 0, stride = 0, ld = 0;
+  __host__ __device__ Planes at(int64_t b, int64_t row = 0, int64_t col = 0) const {  // from matrix b, row, column on
+    Planes o = *this;
+    o.p += b * stride + row * ld + col;
+    return o;
+  }
+};
+inline size_t planes_bytes(int64_t rows, int64_t cols, int64_t count) {
+  return (size_t)(6 * count * rows * plane_ld(cols));
+}
+inline Planes planes_in(void* base, int64_t rows, int64_t cols, int64_t count) {
+  const int64_t ld = plane_ld(cols);
+  return Planes{static_cast<__nv_bfloat16*>(base), count * rows * ld, rows * ld, ld};
+}
+struct B3Operand {
+  const __nv_bfloat16* p;
+  int64_t plane, ld, stride;
+  int batch;               // distinct matrices (0: one per launch batch entry)
+};
+inline B3Operand b3_op(const Planes& x, int batch) { return B3Operand{x.p, x.plane, x.ld, x.stride, batch}; }
+struct B3Epilogue {
+  float* C;                // fp32 output (or nullptr), matrix b at b * c_stride ...
+  float* const* C_ptrs;    // ... or a device array of per-matrix output pointers (16-byte aligned)
+  int64_t ldc, c_stride;
+  __nv_bfloat16* P;        // output as planes (or nullptr)
+  int64_t p_plane, p_ld, p_stride;
+  int transpose;           // write C^T (N x M)
+  float alpha, beta;       // beta != 0 reads C
+  int* status;             // device status word for a timed-out wait (may be nullptr)
+  uint64_t wait_ns;        // set by gemm_b3 from the library's wait settings
+  const int* hold;
+};
+// C_b = alpha A_b B_(b mod B.batch)^T + beta C_b, in fp32 or (transposed only) as planes. The
+// dimension that C's rows run along must be a multiple of 4, C and its rows 16-byte aligned.
+cudaError_t gemm_b3(int M, int N, int K, int batch, const B3Operand& A, const B3Operand& B, const B3Epilogue& ep,
+                    cudaStream_t s, int family = kFamGemmTc);
+// C_b = alpha A_b A_b^T + beta C_b (M x M): only the tiles on or below the diagonal are computed,
+// each below it also stored in the mirror position; C in fp32 (read) and as planes.
+cudaError_t gemm_b3_syrk(int M, int K, int batch, const B3Operand& A, const B3Epilogue& ep, cudaStream_t s,
+                         int family = kFamGemmTc);
+
+#ifdef __CUDACC__
+// The three planes of a value, and of four (one 8-byte word of each plane).
+__device__ __forceinline__ void b3_split(float x, __nv_bfloat16& h, __nv_bfloat16& m, __nv_bfloat16& l) {
+  h = __float2bfloat16_rn(x);
+  const float r = x - __bfloat162float(h);
+  m = __float2bfloat16_rn(r);
+  l = __float2bfloat16_rn(r - __bfloat162float(m));
+}
+__device__ __forceinline__ void b3_split2(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l) {
+  const __nv_bfloat162 hh = __floats2bfloat162_rn(x, y);
+  const float2 hf = __bfloat1622float2(hh);
+  const float rx = x - hf.x, ry = y - hf.y;
+  const __nv_bfloat162 mm = __floats2bfloat162_rn(rx, ry);
+  const float2 mf = __bfloat1622float2(mm);
+  const __nv_bfloat162 ll = __floats2bfloat162_rn(rx - mf.x, ry - mf.y);
+  h = reinterpret_cast<const uint32_t&>(hh);
+  m = reinterpret_cast<const uint32_t&>(mm);
+  l = reinterpret_cast<const uint32_t&>(ll);
+}
+__device__ __forceinline__ void b3_split4(float4 x, uint2& h, uint2& m, uint2& l) {
+  b3_split2(x.x, x.y, h.x, m.x, l.x);
+  b3_split2(x.z, x.w, h.y, m.y, l.y);
+}
+__device__ __forceinline__ void b3_store(__nv_bfloat16* p, int64_t plane, float x) {
+  b3_split(x, p[0], p[plane], p[2 * plane]);
+}
+__device__ __forceinline__ void b3_store4(__nv_bfloat16* p, int64_t plane, float4 x) {  // 8-byte aligned
+  uint2 h, m, l;
+  b3_split4(x, h, m, l);
+  *reinterpret_cast<uint2*>(p) = h;
+  *reinterpret_cast<uint2*>(p + plane) = m;
+  *reinterpret_cast<uint2*>(p + 2 * plane) = l;
+}
+#endif
+
 // hi = trunc_tf32(x), lo = x - hi (exact), elementwise over n values.
 cudaError_t split_tf32(const float* x, float* hi, float* lo, int64_t n, cudaStream_t stream);
 
@@ -100,9 +186,8 @@ cudaError_t qr_q(int n, int batch, const float* P, float* Q, uint8_t* skip, floa
                  void* workspace, size_t workspace_bytes, int* status, cudaStream_t stream);
 // Where the factored matrix P^T must be placed before qr_q_t.
 void qr_input_buffers(void* workspace, int n, int batch, float** At);
-// QR of P whose transpose is already in qr_input_buffers(). Writes Q^T into Qt (or, if Qt is
-// nullptr, into the workspace) and, if Q is given, Q and (if Q_lo is given) its lo part.
-// Qt_lo is not written.
+// QR of P whose transpose is already in qr_input_buffers(). Leaves Q^T there and, if Q is given,
+// writes Q.
 // The look-ahead schedule of qr_q_t: a second (low-priority) stream and its events.
 struct QrLookahead {
   cudaStream_t far;     // trailing updates beyond the next block, and V T for the Q accumulation
@@ -113,9 +198,8 @@ struct QrLookahead {
 // With `la` (all members set, and a workspace sized with lookahead) the trailing update of each
 // 128-column block, except the next block's rows, and the block's V T run on la->far and
 // overlap the next block's panels; everything is joined back on `stream` before return.
-cudaError_t qr_q_t(int n, int batch, float* Qt, float* Qt_lo, float* Q, float* Q_lo, uint8_t* skip,
-                   float tol, void* workspace, size_t workspace_bytes, int* status,
-                   cudaStream_t stream, const QrLookahead* la = nullptr);
+cudaError_t qr_q_t(int n, int batch, float* Q, uint8_t* skip, float tol, void* workspace, size_t workspace_bytes,
+                   int* status, cudaStream_t stream, const QrLookahead* la = nullptr);
 
 // bf16 tensor-core product out_b = alpha A_b B_b^T + beta Cin_b (A_b M x K, B_b N x K, bf16
 // row-major; fp32 accumulation). Outputs (any may be null): out (bf16, ld, stride; Cin has the
@@ -153,24 +237,23 @@ cudaError_t muon_update(float* const* params, const __nv_bfloat16* O, int64_t el
 // M_hat <- b1 M_hat + (1-b1) G and Gc <- G for each matrix of a class.
 cudaError_t momentum_and_copy(const float* const* grads, float* Gc, float* Mhat, int64_t elems,
                               int batch, float beta1, int* status, cudaStream_t stream);
-// v <- b2 v + (1-b2) G'^2; N = m' / (sqrt(v) + eps) (bias-corrected if t > 0 given),
-// written over Gp; guard rows/cols zeroed.
+// v <- b2 v + (1-b2) G'^2; N = m' / (sqrt(v) + eps) (bias-corrected if t > 0 given), written as
+// the planes Np if given (cols a multiple of 4), else over Gp; guard rows/cols zeroed.
 cudaError_t adam_in_basis(float* Gp, const float* Mp, float* V, int rows, int cols, int batch,
                           float beta1, float beta2, float eps, float bc1, float bc2,
-                          const uint8_t* skipL, const uint8_t* skipR, float* N_lo, int* status,
-                          cudaStream_t stream);
-// Tensor-core operand preparation: G and G^T with their lo parts, and the momentum EMA
-// M_hat <- b1 M_hat + (1-b1) G in place, with a copy of the new M_hat and its lo part
-// (Mcopy, Mcopy_lo); M_hat is stored in G's orientation or (if mhat_transposed) as M_hat^T,
-// and so is its copy.
-cudaError_t momentum_split(const float* const* grads, float* Gn, float* Gn_lo, float* Gt, float* Gt_lo,
-                           float* Mhat, float* Mcopy, float* Mcopy_lo, int rows, int cols, int batch, float beta1,
-                           bool mhat_transposed, int* status, cudaStream_t stream);
+                          const uint8_t* skipL, const uint8_t* skipR, const Planes& Np, int* status,
+                          cudaStream_t s);
+// Tensor-core operand preparation (rows and cols multiples of 4): the planes of G and of G^T, and
+// the momentum EMA M_hat <- b1 M_hat + (1-b1) G in place, with its planes (Mc); M_hat is stored
+// in G's orientation or (if mhat_transposed) as M_hat^T, and so are its planes.
+cudaError_t momentum_split(const float* const* grads, const Planes& Gn, const Planes& Gt, const Planes& Mc, float* Mhat,
+                           int rows, int cols, int batch, float beta1, bool mhat_transposed, int* status,
+                           cudaStream_t stream);
 // Packed symmetric storage: the lower-triangular 32 x 32 tiles of an n x n matrix, tile (I, J)
 // (I >= J) at tile index I (I + 1) / 2 + J, each row-major; packed_floats(n) per matrix.
 int64_t packed_floats(int n);
-// F_b (full, n x n) and, if F_lo is given, its lo part from the packed tiles P_b.
-cudaError_t unpack_sym(const float* P, float* F, float* F_lo, int n, int batch, cudaStream_t stream);
+// F_b (full, n x n) and, if Fp is given, its planes from the packed tiles P_b.
+cudaError_t unpack_sym(const float* P, float* F, const Planes& Fp, int n, int batch, cudaStream_t stream);
 // P_b from the lower triangle of F_b.
 cudaError_t pack_sym(const float* F, float* P, int n, int batch, cudaStream_t stream);
 // Device pointer table written from a host array through kernel parameters (no host buffer
@@ -182,22 +265,20 @@ struct PtrChunk {
 cudaError_t put_ptrs(void** dst, void* const* src, int64_t n, cudaStream_t stream);
 // dst_b = src_b^T for `batch` contiguous rows x cols matrices.
 cudaError_t transpose(const float* src, float* dst, int rows, int cols, int batch, cudaStream_t stream);
-// From Q^T: a copy of it with its lo part, and Q with its lo part (any output may be null;
-// the lo parts are formed from the values, Qt_lo is not read).
-cudaError_t basis_from_qt(const float* Qt, const float* Qt_lo, float* Qt_out, float* Qt_lo_out, float* Q,
-                          float* Q_lo, int n, int batch, cudaStream_t stream);
-// Q -> lo part, Q^T, lo part of Q^T for `batch` n x n bases.
-cudaError_t basis_split(const float* Q, float* Q_lo, float* Qt, float* Qt_lo, int n, int batch,
-                        cudaStream_t stream);
+// For `batch` n x n matrices X (n a multiple of 4), any output left out if null: the planes of X
+// and of X^T, and X^T itself.
+cudaError_t planes_transpose(const float* X, const Planes& Xp, const Planes& Xtp, float* Xt, int n, int batch,
+                             cudaStream_t stream);
+// The planes of `rows` contiguous rows of cols values (cols a multiple of 4).
+cudaError_t split_planes(const float* X, const Planes& Xp, int64_t rows, int cols, cudaStream_t stream);
 // W <- (1 - lr*wd) W - lr * D (both sides identity).
 cudaError_t weight_update(float* const* params, const float* D, int64_t elems, int batch,
                           float lr, float wd, cudaStream_t stream);
 // KL-Shampoo factor form: lam[b][i] = sum_k C[b][i][k] Qt[b][i][k], the diagonal of Q^T F Q
-// from C = Q^T F (n a multiple of 4).
-cudaError_t diag_dot(const float* C, const float* Qt, float* lam, int n, int batch, cudaStream_t stream);
-// X[b][:, j] *= sqrt(coef / (max(lam[b][j], 0) + eps)) in place, with the lo part into X_lo
-// (cols a multiple of 4).
-cudaError_t scale_cols_split(float* X, float* X_lo, const float* lam, int rows, int cols, int batch,
+// from C = Q^T F and the planes of Q^T (n a multiple of 4).
+cudaError_t diag_dot(const float* C, const Planes& Qt, float* lam, int n, int batch, cudaStream_t stream);
+// The planes of X[b][:, j] * sqrt(coef / (max(lam[b][j], 0) + eps)) (cols a multiple of 4).
+cudaError_t scale_cols_split(const float* X, const Planes& Xp, const float* lam, int rows, int cols, int batch,
                              float coef, float eps, cudaStream_t stream);
 // Sets `batch` n x n matrices to the identity.
 cudaError_t set_identity(float* Q, int n, int batch, cudaStream_t stream);
