@@ -70,50 +70,6 @@ struct Cfg {
   static_assert(SMEM <= 232448, "shared memory budget");
 };
 
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-// Address in the pair's first CTA of this CTA's shared-memory address.
-template <int CG>
-__device__ __forceinline__ uint32_t lead_addr(uint32_t a) {
-  if (CG == 1) return a;
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(a));
-  return r;
-}
-// One arrival at a barrier of the pair's first CTA.
-template <int CG>
-__device__ __forceinline__ void arrive_lead(uint64_t* bar) {
-  if (CG == 1)
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-  else
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(lead_addr<CG>(smem_u32(bar)))
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_cluster(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait; the barrier may have been arrived at from the other CTA.
-template <int CG>
-__device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
-  if (CG == 1) return tc::mbar_wait(bar, parity, limit_ns);
-  if (mbar_try_cluster(bar, parity)) return true;
-  const uint64_t t0 = tc::globaltimer();
-  for (;;) {
-    for (int i = 0; i < 16; ++i)
-      if (mbar_try_cluster(bar, parity)) return true;
-    if (tc::globaltimer() - t0 > limit_ns) return false;
-  }
-}
 __device__ __forceinline__ bool flag_wait(const int* flag, uint64_t limit_ns) {
   const volatile int* f = flag;
   if (*f != 0) return true;
@@ -138,39 +94,6 @@ __device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, u
         "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, "
         "%5, %6}], [%2];" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(0)
-        : "memory");
-}
-
-// Instruction descriptor for kind::f16: D = f32, A = B = bf16, both K-major.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(N >> 3) << 17) |
-         (static_cast<uint32_t>(M >> 4) << 24);
-}
-template <int CG>
-__device__ __forceinline__ void umma(uint32_t d, uint32_t a, uint32_t b, uint32_t idesc, uint32_t accumulate) {
-  if (CG == 1)
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-        "l"(tc::desc_sw128(a)), "l"(tc::desc_sw128(b)), "r"(idesc), "r"(accumulate));
-  else
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-        "l"(tc::desc_sw128(a)), "l"(tc::desc_sw128(b)), "r"(idesc), "r"(accumulate));
-}
-// Completion of the MMAs issued so far, to the same barrier of every CTA of the tile.
-template <int CG>
-__device__ __forceinline__ void commit(uint64_t* bar) {
-  if (CG == 1)
-    tc::umma_commit(bar);
-  else
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-            smem_u32(bar)),
-        "h"((uint16_t)3)
         : "memory");
 }
 
@@ -295,13 +218,13 @@ __global__ void __launch_bounds__(THREADS, 1)
         tile(t, m0, n0, b);
         for (int kb = 0; kb < kblocks; ++kb, ++g) {
           const int s = g % STAGES;
-          if (!wait<CG>(&empty[s], ((g / STAGES) & 1) ^ 1, lim) || *abort_flag) {
+          if (!tc::wait<CG>(&empty[s], ((g / STAGES) & 1) ^ 1, lim) || *abort_flag) {
             *abort_flag = 1;
             if (ep.status) atomicOr(ep.status, kStatusTimeout);
             break;
           }
-          if (lead) mbar_expect_tx(&full[s], CG * C::STAGE);
-          const uint32_t st = smem_u32(smem + s * C::STAGE), bar = lead_addr<CG>(smem_u32(&full[s]));
+          if (lead) tc::mbar_expect_tx(&full[s], CG * C::STAGE);
+          const uint32_t st = smem_u32(smem + s * C::STAGE), bar = tc::lead_addr<CG>(smem_u32(&full[s]));
           tma_load<CG>(st, &ta, bar, kb * BK, m0 + rank * BM, b % p.a_mod);
           tma_load<CG>(st + 3 * PLANE_A, &tb, bar, kb * BK, n0 + rank * C::BROWS, b % p.b_mod);
           issued = g + 1;
@@ -310,19 +233,19 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (*abort_flag && lead) {
         // let copies already in flight land before the CTAs' shared memory goes away (the second
         // CTA's copies count on this CTA's barriers too, and it waits at the last cluster barrier)
-        for (int gg = *consumed; gg < issued; ++gg) wait<CG>(&full[gg % STAGES], (gg / STAGES) & 1, kWaitNs);
+        for (int gg = *consumed; gg < issued; ++gg) tc::wait<CG>(&full[gg % STAGES], (gg / STAGES) & 1, kWaitNs);
       }
     }
   } else if (warp == 1) {
     if (lane == 0 && lead) {
-      constexpr uint32_t idesc = idesc_bf16(TM, BN);
+      constexpr uint32_t idesc = tc::idesc_bf16(TM, BN);
       int g = 0;
       bool ok = true;
       for (int t = t_begin; t < t_end && ok && !*abort_flag; ++t) {
         for (int kb = 0; kb < kblocks; ++kb, ++g) {
           const int s = g % STAGES, a = g % NACC;
-          if (!wait<CG>(&full[s], (g / STAGES) & 1, lim) ||
-              (g >= NACC && !wait<CG>(&acc_empty[a], ((g / NACC) & 1) ^ 1, lim)) || *abort_flag) {
+          if (!tc::wait<CG>(&full[s], (g / STAGES) & 1, lim) ||
+              (g >= NACC && !tc::wait<CG>(&acc_empty[a], ((g / NACC) & 1) ^ 1, lim)) || *abort_flag) {
             ok = false;
             break;
           }
@@ -334,20 +257,20 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk) {
             const uint32_t o = kk * 32;  // 16 bf16 along K inside the swizzle row
-            umma<CG>(d, as + o, bs + 2 * C::PLANE_B + o, idesc, kk != 0);
-            umma<CG>(d, as + 2 * PLANE_A + o, bs + o, idesc, 1u);
-            umma<CG>(d, as + PLANE_A + o, bs + C::PLANE_B + o, idesc, 1u);
+            tc::umma_f16<CG>(d, as + o, bs + 2 * C::PLANE_B + o, idesc, kk != 0);
+            tc::umma_f16<CG>(d, as + 2 * PLANE_A + o, bs + o, idesc, 1u);
+            tc::umma_f16<CG>(d, as + PLANE_A + o, bs + C::PLANE_B + o, idesc, 1u);
           }
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk) {
             const uint32_t o = kk * 32;
-            umma<CG>(d, as + o, bs + C::PLANE_B + o, idesc, 1u);
-            umma<CG>(d, as + PLANE_A + o, bs + o, idesc, 1u);
+            tc::umma_f16<CG>(d, as + o, bs + C::PLANE_B + o, idesc, 1u);
+            tc::umma_f16<CG>(d, as + PLANE_A + o, bs + o, idesc, 1u);
           }
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) umma<CG>(d, as + kk * 32, bs + kk * 32, idesc, 1u);
-          commit<CG>(&empty[s]);     // frees the stage once these MMAs have read it
-          commit<CG>(&acc_full[a]);  // hands the K block's sum to the epilogue warps
+          for (int kk = 0; kk < BK / 16; ++kk) tc::umma_f16<CG>(d, as + kk * 32, bs + kk * 32, idesc, 1u);
+          tc::commit<CG>(&empty[s]);     // frees the stage once these MMAs have read it
+          tc::commit<CG>(&acc_full[a]);  // hands the K block's sum to the epilogue warps
         }
       }
       if (!ok) {
@@ -357,8 +280,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       // the tensor memory is freed below: every MMA issued must have completed first (this
       // matters only when a wait gave up; otherwise the epilogue has drained them all)
       if (g > 0) {
-        commit<CG>(mma_done);
-        wait<CG>(mma_done, 0, kWaitNs);
+        tc::commit<CG>(mma_done);
+        tc::wait<CG>(mma_done, 0, kWaitNs);
       }
     }
   } else {
@@ -400,7 +323,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int j = 0; j < 32; ++j) acc[c][j] = 0.f;
       for (int kb = 0; kb < kblocks; ++kb, ++g) {
         const int a = g % NACC;
-        if (!wait<CG>(&acc_full[a], (g / NACC) & 1, lim) || *abort_flag) {
+        if (!tc::wait<CG>(&acc_full[a], (g / NACC) & 1, lim) || *abort_flag) {
           valid = false;
           break;
         }
@@ -417,7 +340,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         tc::tc_fence_before();
         __syncwarp();
-        if (lane == 0) arrive_lead<CG>(&acc_empty[a]);
+        if (lane == 0) tc::arrive_lead<CG>(&acc_empty[a]);
       }
       if (!valid) {
         *abort_flag = 1;

@@ -72,11 +72,6 @@ struct Cfg {
   static_assert(SMEM <= 232448, "shared memory budget");
 };
 
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-
 // Bounded wait until *flag != 0 (a flag set from outside the kernel): false after `limit_ns`.
 __device__ __forceinline__ bool flag_wait(const int* flag, uint64_t limit_ns) {
   const volatile int* f = flag;
@@ -124,19 +119,6 @@ __device__ __forceinline__ void tile_coords(int t, int ntm, int ntn, int BN_, in
   n0 = (w / gsz) * BN_;
 }
 
-// Symmetric products (C = alpha A A^T + beta C, M = N): tile t -> (m0, n0, batch index) over the
-// tiles on or below the diagonal only, row by row (tile (i, j), j <= i, at i (i + 1) / 2 + j).
-__device__ __forceinline__ void tile_coords_sym(int t, int ntm, int& m0, int& n0, int& b) {
-  const int per = ntm * (ntm + 1) / 2;
-  b = t / per;
-  const int r = t - b * per;
-  int i = (int)((sqrtf(8.f * (float)r + 1.f) - 1.f) * 0.5f);
-  while ((i + 1) * (i + 2) / 2 <= r) ++i;
-  while (i * (i + 1) / 2 > r) --i;
-  m0 = i * BM;
-  n0 = (r - i * (i + 1) / 2) * BM;
-}
-
 // A CTA takes `tpc` consecutive tiles, so that the loads and MMAs of its next tile overlap
 // the epilogue of the current one. With ksplit > 1 the K blocks are split into ksplit
 // consecutive ranges; split s of matrix b is written as output matrix s * batch + b (partial
@@ -144,10 +126,7 @@ __device__ __forceinline__ void tile_coords_sym(int t, int ntm, int& m0, int& n0
 // With CVTA the A operand comes as fp32 only: the epilogue warps form its lo part in shared
 // memory, beside the tile TMA brought in (for HBM-bound products whose A is read once; the
 // extra shared-memory traffic would slow a compute-bound product).
-// With SYM (A = B, M = N, BN = BM) only the tiles on or below the diagonal are computed, and each
-// one below it is also stored transposed in the mirror position, so C stays exactly symmetric
-// with about half of the MMAs.
-template <int BN, int STAGES, bool PRE, bool CVTA, bool TR, bool LO, bool VEC, bool SYM>
+template <int BN, int STAGES, bool PRE, bool CVTA, bool TR, bool LO, bool VEC>
 __global__ void __launch_bounds__(Cfg<BN, STAGES, PRE>::THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUtensorMap ta_lo,
                    const __grid_constant__ CUtensorMap tb_hi, const __grid_constant__ CUtensorMap tb_lo, int M,
@@ -171,7 +150,7 @@ __global__ void __launch_bounds__(Cfg<BN, STAGES, PRE>::THREADS, 1)
   const int kblocks = (K + BK - 1) / BK;
   const int kper = (kblocks + ksplit - 1) / ksplit;  // K blocks of one split
   const int ntn = (N + BN - 1) / BN, ntm = (M + BM - 1) / BM;
-  const int ntiles = (SYM ? ntm * (ntm + 1) / 2 : ntn * ntm) * batch * ksplit;
+  const int ntiles = ntn * ntm * batch * ksplit;
   // the K blocks [kb0, kb1) of tile t, and its operand and output matrix indices
   auto krange = [&](int bo, int& kb0, int& kb1) {
     kb0 = (bo / batch) * kper;
@@ -216,8 +195,7 @@ __global__ void __launch_bounds__(Cfg<BN, STAGES, PRE>::THREADS, 1)
       int g = 0, issued = 0;  // k blocks over all of this CTA's tiles
       for (int t = t_begin; t < t_end && !*abort_flag; ++t) {
         int m0, n0, bo, kb0, kb1;
-        if (SYM) tile_coords_sym(t, ntm, m0, n0, bo);
-        else tile_coords(t, ntm, ntn, BN, m0, n0, bo);
+        tile_coords(t, ntm, ntn, BN, m0, n0, bo);
         krange(bo, kb0, kb1);
         const int b = bo % batch;
         for (int kb = kb0; kb < kb1; ++kb, ++g) {
@@ -250,8 +228,7 @@ __global__ void __launch_bounds__(Cfg<BN, STAGES, PRE>::THREADS, 1)
       bool ok = true;
       for (int t = t_begin; t < t_end && ok && !*abort_flag; ++t) {
         int m0, n0, bo, kb0, kb1;
-        if (SYM) tile_coords_sym(t, ntm, m0, n0, bo);
-        else tile_coords(t, ntm, ntn, BN, m0, n0, bo);
+        tile_coords(t, ntm, ntn, BN, m0, n0, bo);
         krange(bo, kb0, kb1);
         for (int kb = kb0; kb < kb1; ++kb, ++g) {
           const int s = g % STAGES;
@@ -322,8 +299,7 @@ __global__ void __launch_bounds__(Cfg<BN, STAGES, PRE>::THREADS, 1)
     if (CVTA)
       for (int t = t_begin; t < t_end; ++t) {
         int m0, n0, bo, kb0, kb1;
-        if (SYM) tile_coords_sym(t, ntm, m0, n0, bo);
-        else tile_coords(t, ntm, ntn, BN, m0, n0, bo);
+        tile_coords(t, ntm, ntn, BN, m0, n0, bo);
         krange(bo, kb0, kb1);
         gtotal += kb1 - kb0;
       }
@@ -338,16 +314,15 @@ __global__ void __launch_bounds__(Cfg<BN, STAGES, PRE>::THREADS, 1)
     }
     for (int t = t_begin; t < t_end && valid; ++t) {
       int m0, n0, b, kb0, kb1;  // b: output matrix (split * batch + operand matrix)
-      if (SYM) tile_coords_sym(t, ntm, m0, n0, b);
-      else tile_coords(t, ntm, ntn, BN, m0, n0, b);
+      tile_coords(t, ntm, ntn, BN, m0, n0, b);
       krange(b, kb0, kb1);
-      float* Cb = ep.C_ptrs ? ep.C_ptrs[b] : (ep.C ? ep.C + (int64_t)b * ep.c_stride : nullptr);
+      float* Cb = ep.C + (int64_t)b * ep.c_stride;
       float* Lb = LO && ep.C_lo ? ep.C_lo + (int64_t)b * ep.lo_stride : nullptr;
       const int row0 = m0 + 32 * q;   // first of this warp's 32 rows
       const int col0 = n0 + colbase;  // first of its CPW columns
       // 16-byte vector access to C (and C_lo) needs 16-byte aligned rows
       // (a kernel that prefetches C is only launched on 16-byte aligned C, lo part and rows)
-      const bool vec = PRE || VEC || Cb && (ep.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 15) == 0 &&
+      const bool vec = PRE || VEC || (ep.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 15) == 0 &&
                        (!Lb || ((ep.ld_lo & 3) == 0 && (reinterpret_cast<uintptr_t>(Lb) & 15) == 0));
       // the prefetch copies whole 16-byte units: the dimension they run along must be a multiple of 4
       const bool pre = PRE;
@@ -428,7 +403,7 @@ __global__ void __launch_bounds__(Cfg<BN, STAGES, PRE>::THREADS, 1)
               } else {
                 const int col = cc0 + 4 * j4;
                 const float* src = Cb + (int64_t)r * ep.ldc + col;
-                const bool in = Cb && r < M;
+                const bool in = r < M;
                 cv.x = (in && col < N) ? src[0] : 0.f;
                 cv.y = (in && col + 1 < N) ? src[1] : 0.f;
                 cv.z = (in && col + 2 < N) ? src[2] : 0.f;
@@ -450,30 +425,15 @@ __global__ void __launch_bounds__(Cfg<BN, STAGES, PRE>::THREADS, 1)
             const float4 o = *reinterpret_cast<const float4*>(cb + swz(rr, 4 * j4));
             const float ov[4] = {o.x, o.y, o.z, o.w};
             if (vec && col + 3 < N) {
-              if (Cb) *reinterpret_cast<float4*>(Cb + (int64_t)r2 * ep.ldc + col) = o;
+              *reinterpret_cast<float4*>(Cb + (int64_t)r2 * ep.ldc + col) = o;
               if (Lb)
                 *reinterpret_cast<float4*>(Lb + (int64_t)r2 * ep.ld_lo + col) =
                     make_float4(tf32_lo(o.x), tf32_lo(o.y), tf32_lo(o.z), tf32_lo(o.w));
             } else {
               for (int e = 0; e < 4 && col + e < N; ++e) {
-                if (Cb) Cb[(int64_t)r2 * ep.ldc + col + e] = ov[e];
+                Cb[(int64_t)r2 * ep.ldc + col + e] = ov[e];
                 if (Lb) Lb[(int64_t)r2 * ep.ld_lo + col + e] = tf32_lo(ov[e]);
               }
-            }
-          }
-          if (SYM && m0 != n0) {
-            // the mirror tile: element (r, j) of this block also goes to C[j][r]
-#pragma unroll 1
-            for (int it = 0; it < 8; ++it) {
-              const int jj = 4 * it + (lane >> 3), r4 = 4 * (lane & 7);
-              const int mrow = cc0 + jj, mcol = row0 + r4;  // row and column in C
-              if (mrow >= N || mcol + 3 >= M) continue;    // M = N, a multiple of 4
-              const float4 o = make_float4(cb[swz(r4, jj)], cb[swz(r4 + 1, jj)], cb[swz(r4 + 2, jj)],
-                                           cb[swz(r4 + 3, jj)]);
-              *reinterpret_cast<float4*>(Cb + (int64_t)mrow * ep.ldc + mcol) = o;
-              if (Lb)
-                *reinterpret_cast<float4*>(Lb + (int64_t)mrow * ep.ld_lo + mcol) =
-                    make_float4(tf32_lo(o.x), tf32_lo(o.y), tf32_lo(o.z), tf32_lo(o.w));
             }
           }
           __syncwarp();
@@ -486,7 +446,7 @@ __global__ void __launch_bounds__(Cfg<BN, STAGES, PRE>::THREADS, 1)
             float* slot = cb + swz(j, lane);
             if (ep.beta != 0.f) {
               const int col = cc0 + j;
-              const float cv = pre ? *slot : ((Cb && r < M && col < N) ? Cb[(int64_t)col * ep.ldc + r] : 0.f);
+              const float cv = pre ? *slot : ((r < M && col < N) ? Cb[(int64_t)col * ep.ldc + r] : 0.f);
               o = fmaf(ep.beta, cv, o);
             }
             *slot = o;
@@ -500,13 +460,13 @@ __global__ void __launch_bounds__(Cfg<BN, STAGES, PRE>::THREADS, 1)
             const float4 o = *reinterpret_cast<const float4*>(cb + swz(jj, 4 * r4));
             const float ov[4] = {o.x, o.y, o.z, o.w};
             if (vec && r2 + 3 < M) {
-              if (Cb) *reinterpret_cast<float4*>(Cb + (int64_t)col * ep.ldc + r2) = o;
+              *reinterpret_cast<float4*>(Cb + (int64_t)col * ep.ldc + r2) = o;
               if (Lb)
                 *reinterpret_cast<float4*>(Lb + (int64_t)col * ep.ld_lo + r2) =
                     make_float4(tf32_lo(o.x), tf32_lo(o.y), tf32_lo(o.z), tf32_lo(o.w));
             } else {
               for (int e = 0; e < 4 && r2 + e < M; ++e) {
-                if (Cb) Cb[(int64_t)col * ep.ldc + r2 + e] = ov[e];
+                Cb[(int64_t)col * ep.ldc + r2 + e] = ov[e];
                 if (Lb) Lb[(int64_t)col * ep.ld_lo + r2 + e] = tf32_lo(ov[e]);
               }
             }
@@ -560,8 +520,7 @@ bool make_map(CUtensorMap* map, const float* base, int rows, int K, int64_t ld, 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, int STAGES, bool PRE, bool CVTA = false, bool TR = false, bool LO = false, bool VEC = false,
-          bool SYM = false>
+template <int BN, int STAGES, bool PRE, bool CVTA = false, bool TR = false, bool LO = false, bool VEC = false>
 cudaError_t launch(const TcOperand& A, const TcOperand& B, int M, int N, int K, int batch, const TcEpilogue& ep,
                    cudaStream_t s, int ksplit = 1) {
   using C = Cfg<BN, STAGES, PRE>;
@@ -579,13 +538,13 @@ cudaError_t launch(const TcOperand& A, const TcOperand& B, int M, int N, int K, 
   const uint64_t bit = (dev >= 0 && dev < 64) ? uint64_t(1) << dev : 0;
   if (bit == 0 || !(attr_set.load(std::memory_order_relaxed) & bit)) {
     cudaError_t e =
-        cudaFuncSetAttribute(gemm_tc_kernel<BN, STAGES, PRE, CVTA, TR, LO, VEC, SYM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(gemm_tc_kernel<BN, STAGES, PRE, CVTA, TR, LO, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              C::SMEM);
     if (e != cudaSuccess) return e;
     attr_set.fetch_or(bit, std::memory_order_relaxed);
   }
   const int64_t ntm = (M + BM - 1) / BM;
-  const int64_t ntiles = (SYM ? ntm * (ntm + 1) / 2 : (int64_t)((N + BN - 1) / BN) * ntm) * batch * ksplit;
+  const int64_t ntiles = (int64_t)((N + BN - 1) / BN) * ntm * batch * ksplit;
   if (ntiles > (int64_t)1 << 30) return cudaErrorInvalidValue;
   // K up to 2048: a CTA runs several tiles so that the next tile's loads and MMAs overlap the
   // current epilogue, keeping about four waves of CTAs over the 152 SMs (for longer K the
@@ -593,7 +552,7 @@ cudaError_t launch(const TcOperand& A, const TcOperand& B, int M, int N, int K, 
   const int kblocks = (K + BK - 1) / BK;
   const int tpc = kblocks > 64 ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(8, ntiles / (4 * 152)));
   const int grid = (int)((ntiles + tpc - 1) / tpc);
-  gemm_tc_kernel<BN, STAGES, PRE, CVTA, TR, LO, VEC, SYM><<<grid, C::THREADS, C::SMEM, s>>>(m[0], m[1], m[2], m[3], M, N, K, batch, amod,
+  gemm_tc_kernel<BN, STAGES, PRE, CVTA, TR, LO, VEC><<<grid, C::THREADS, C::SMEM, s>>>(m[0], m[1], m[2], m[3], M, N, K, batch, amod,
                                                                      bmod, tpc, ksplit, ep);
   return cudaGetLastError();
 }
@@ -698,12 +657,11 @@ cudaError_t gemm_tc_nt(int M, int N, int K, int batch, const TcOperand& A, const
   // prefetches in 16-byte units: C (and its lo part) 16-byte aligned with rows of 16-byte
   // multiples; otherwise the kernel without the prefetch reads C element by element
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  const bool pre = ep.beta != 0.f && (ep.C || ep.C_ptrs) && (ep.ldc & 3) == 0 && (ep.c_stride & 3) == 0 &&
-                   (!ep.C || al16(ep.C)) && ((ep.transpose ? M : N) & 3) == 0 &&
+  const bool pre = ep.beta != 0.f && (ep.ldc & 3) == 0 && (ep.c_stride & 3) == 0 && al16(ep.C) && ((ep.transpose ? M : N) & 3) == 0 &&
                    (!ep.C_lo || ((ep.ld_lo & 3) == 0 && (ep.lo_stride & 3) == 0 && al16(ep.C_lo)));
   // few tiles and a long K: split K over more CTAs (plain row-major outputs only)
   int ksplit = 1;
-  const bool splittable = split_ws && ep.C && !ep.C_ptrs && !ep.transpose && ep.beta == 0.f && (N & 3) == 0 &&
+  const bool splittable = split_ws && !ep.transpose && ep.beta == 0.f && (N & 3) == 0 &&
                           (ep.ldc & 3) == 0 && (ep.c_stride & 3) == 0 && (!ep.C_lo || (ep.ld_lo == ep.ldc && ep.lo_stride == ep.c_stride)) &&
                           (reinterpret_cast<uintptr_t>(ep.C) & 15) == 0;
   if (splittable) {
@@ -716,7 +674,7 @@ cudaError_t gemm_tc_nt(int M, int N, int K, int batch, const TcOperand& A, const
   if (cvt && (pre || ep.transpose)) return cudaErrorInvalidValue;
   if (B.lo == nullptr) return cudaErrorInvalidValue;
   if (ksplit > 1) {
-    TcEpilogue pe{split_ws, nullptr, N, (int64_t)M * N, nullptr, N, (int64_t)M * N, 0, 1.f, 0.f, ep.status};
+    TcEpilogue pe{split_ws, N, (int64_t)M * N, nullptr, N, (int64_t)M * N, 0, 1.f, 0.f, ep.status};
     pe.wait_ns = ep.wait_ns;
     pe.hold = ep.hold;
     cudaError_t e = N <= 32 ? (cvt ? tc::launch<32, 5, false, true>(A, B, M, N, K, batch, pe, s, ksplit)
@@ -731,7 +689,7 @@ cudaError_t gemm_tc_nt(int M, int N, int K, int batch, const TcOperand& A, const
     return cudaGetLastError();
   }
   const bool tr = ep.transpose != 0, lo = ep.C_lo != nullptr;
-  const bool vec = !ep.C_ptrs && ep.C && al16(ep.C) && (ep.ldc & 3) == 0 && (ep.c_stride & 3) == 0 &&
+  const bool vec = al16(ep.C) && (ep.ldc & 3) == 0 && (ep.c_stride & 3) == 0 &&
                    ((tr ? M : N) & 3) == 0 &&
                    (!ep.C_lo || ((ep.ld_lo & 3) == 0 && (ep.lo_stride & 3) == 0 && al16(ep.C_lo)));
   if (cvt)
@@ -742,29 +700,6 @@ cudaError_t gemm_tc_nt(int M, int N, int K, int batch, const TcOperand& A, const
                : tc::launch_tl<32, 5, false, false>(tr, lo, vec, A, B, M, N, K, batch, ep, s);
   return pre ? tc::launch_tl<128, 2, true, false>(tr, lo, vec, A, B, M, N, K, batch, ep, s)
              : tc::launch_tl<128, 3, false, false>(tr, lo, vec, A, B, M, N, K, batch, ep, s);
-}
-
-cudaError_t gemm_tc_syrk(int M, int K, int batch, const TcOperand& A, const TcEpilogue& ep_in, cudaStream_t s,
-                         int family) {
-  if (M <= 0 || batch <= 0) return cudaSuccess;
-  if (batch > 65535) return cudaErrorInvalidValue;
-  auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  // the symmetric kernel stores row-major C and its lo part with 16-byte stores, both halves
-  const bool ok = ep_in.C && !ep_in.C_ptrs && !ep_in.transpose && ep_in.C_lo && A.lo && al16(ep_in.C) &&
-                  al16(ep_in.C_lo) && (M & 3) == 0 && (ep_in.ldc & 3) == 0 && (ep_in.c_stride & 3) == 0 &&
-                  (ep_in.ld_lo & 3) == 0 && (ep_in.lo_stride & 3) == 0;
-  if (!ok) return gemm_tc_nt(M, M, K, batch, A, A, ep_in, s, family);
-  TcEpilogue ep = ep_in;
-  ep.wait_ns = g_wait_ns.load(std::memory_order_relaxed);
-  ep.hold = g_hold.load(std::memory_order_relaxed);
-  const double ntm = (double)((M + tc::BM - 1) / tc::BM);
-  const double tiles = ntm * (ntm + 1) / 2 * batch;
-  const double flops = 2.0 * tc::BM * tc::BM * (double)K * tiles;  // the lower tiles' products
-  const double bytes = 4.0 * (2.0 * (double)M * K * (A.batch > 0 ? A.batch : batch) +
-                              (double)M * M * batch * ((ep.beta != 0.f ? 1.5 : 1.0) + 1.0));
-  ProfScope prof(family, flops, bytes, s);
-  return ep.beta != 0.f ? tc::launch<128, 2, true, false, false, true, true, true>(A, A, M, M, K, batch, ep, s)
-                        : tc::launch<128, 3, false, false, false, true, true, true>(A, A, M, M, K, batch, ep, s);
 }
 
 }  // namespace soap

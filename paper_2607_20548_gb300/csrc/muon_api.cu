@@ -135,12 +135,16 @@ soap_status_t step_class(muon_handle h, MuonClass& c, float* const* params, cons
   for (int i = 0; i < h->hp.ns_steps; ++i) {
     const float a = h->coeffs[3 * i], b = h->coeffs[3 * i + 1], cc = h->coeffs[3 * i + 2];
     // A = X X^T
-    MUON_CUDA(h, soap::gemm_bf16_nt(r, r, k, B, X, k, rk, X, k, rk, bepi(h, h->A, r, rr, nullptr, 1.f, 0.f), s));
+    soap::Bf16Epilogue ea = bepi(h, h->A, r, rr, nullptr, 1.f, 0.f);
+    ea.symmetric = true;
+    MUON_CUDA(h, soap::gemm_bf16_nt(r, r, k, B, X, k, rk, X, k, rk, ea, s));
     const __nv_bfloat16* P = h->A;
     float alpha = b;
     if (cc != 0.f) {
       // B = c A A^T + b A
-      MUON_CUDA(h, soap::gemm_bf16_nt(r, r, r, B, h->A, r, rr, h->A, r, rr, bepi(h, h->B, r, rr, h->A, cc, b), s));
+      soap::Bf16Epilogue eb = bepi(h, h->B, r, rr, h->A, cc, b);
+      eb.symmetric = true;
+      MUON_CUDA(h, soap::gemm_bf16_nt(r, r, r, B, h->A, r, rr, h->A, r, rr, eb, s));
       P = h->B;
       alpha = 1.f;
     }

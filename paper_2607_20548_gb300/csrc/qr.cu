@@ -1156,7 +1156,7 @@ TcOperand op(const float* hi, const float* lo, int64_t ld, int64_t stride, int b
 }
 
 TcEpilogue out(float* C, float* C_lo, int64_t ldc, int64_t stride, float alpha, float beta, int* status) {
-  return TcEpilogue{C, nullptr, ldc, stride, C_lo, ldc, stride, 0, alpha, beta, status};
+  return TcEpilogue{C, ldc, stride, C_lo, ldc, stride, 0, alpha, beta, status};
 }
 
 }  // namespace

@@ -1495,7 +1495,7 @@ soap_status_t soap_gemm_tf32x4(int32_t M, int32_t N, int32_t K, int32_t batch, c
   if (lda < K || ldb < K || ldc < (transpose_c ? M : N)) return SOAP_ERR_INVALID_ARG;
   soap::TcOperand A{A_hi, A_lo, lda, stride_a, batch};
   soap::TcOperand B{B_hi, B_lo, ldb, stride_b, b_batch > 0 ? b_batch : batch};
-  soap::TcEpilogue ep{C, nullptr, ldc, stride_c, C_lo, ldc, stride_c, transpose_c, alpha, beta,
+  soap::TcEpilogue ep{C, ldc, stride_c, C_lo, ldc, stride_c, transpose_c, alpha, beta,
                       reinterpret_cast<int*>(status)};
   cudaError_t e = soap::gemm_tc_nt(M, N, K, batch, A, B, ep, (cudaStream_t)stream);
   return e == cudaSuccess ? SOAP_OK : (e == cudaErrorInvalidValue ? SOAP_ERR_INVALID_ARG : SOAP_ERR_CUDA);

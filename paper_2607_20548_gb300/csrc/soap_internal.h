@@ -61,8 +61,7 @@ struct TcOperand {
   int batch;       // distinct matrices (0: one per launch batch entry)
 };
 struct TcEpilogue {
-  float* C;              // output (or nullptr), offset b * c_stride ...
-  float* const* C_ptrs;  // ... or a device array of per-matrix output pointers
+  float* C;              // output, matrix b at b * c_stride
   int64_t ldc;
   int64_t c_stride;
   float* C_lo;           // optional: also write out - tf32(out) here (same layout, ld_lo)
@@ -84,11 +83,6 @@ cudaError_t gemm_tc_nt(int M, int N, int K, int batch, const TcOperand& A, const
 // Bound of the tensor-core products' device waits (0: 2 s) and, for testing the timeout path, a
 // device flag their epilogues first wait for (nullptr: none); applies to later launches.
 void set_wait_limit(uint64_t ns, const int* hold);
-// Symmetric product C_b = alpha A_b A_b^T + beta C_b (M x M, A_b M x K): only the 128 x 128 tiles on
-// or below the diagonal are computed, each below it also stored (with its lo part) in the mirror
-// position. Needs a row-major, 16-byte aligned C with its lo part; other forms go to gemm_tc_nt.
-cudaError_t gemm_tc_syrk(int M, int K, int batch, const TcOperand& A, const TcEpilogue& ep, cudaStream_t stream,
-                         int family = kFamGemmTc);
 // The settings in force (0: the default bound).
 void get_wait_limit(uint64_t* ns, const int** hold);
 
@@ -202,19 +196,19 @@ cudaError_t qr_q_t(int n, int batch, float* Q, uint8_t* skip, float tol, void* w
                    int* status, cudaStream_t stream, const QrLookahead* la = nullptr);
 
 // bf16 tensor-core product out_b = alpha A_b B_b^T + beta Cin_b (A_b M x K, B_b N x K, bf16
-// row-major; fp32 accumulation). Outputs (any may be null): out (bf16, ld, stride; Cin has the
-// same layout), out_t (bf16, transposed: element (r, c) at c * ld_t + r) and out_f32.
-// N and K must be multiples of 8.
+// row-major; fp32 accumulation). Outputs: out (bf16, ld, stride; Cin has the same layout) and, if
+// given, out_t (bf16, transposed: element (r, c) at c * ld_t + r). M, N and K must be multiples of
+// 8. `symmetric` promises a symmetric result (B = A, and Cin, if read, symmetric): one half of it
+// is computed and mirrored.
 struct Bf16Epilogue {
   __nv_bfloat16* out;
   int64_t ld, stride;
   const __nv_bfloat16* cin;
   __nv_bfloat16* out_t;
   int64_t ld_t, stride_t;
-  float* out_f32;
-  int64_t ld_f32, stride_f32;
   float alpha, beta;
   int* status;
+  bool symmetric;
 };
 cudaError_t gemm_bf16_nt(int M, int N, int K, int batch, const __nv_bfloat16* A, int64_t lda, int64_t a_stride,
                          const __nv_bfloat16* B, int64_t ldb, int64_t b_stride, const Bf16Epilogue& ep,
