@@ -1,4 +1,4 @@
-"""The CUDA-core product at the edges of its tiles and of the rule that chooses them, against 64 bits."""
+"""The CUDA-core product at the edges of its tiles and of the rule that chooses them, and the tf32 parts."""
 import pytest
 import torch
 
@@ -23,3 +23,14 @@ def test_simt_tiles(ta, tb, batch, M, N, K):
     # a chain of K fused multiply-adds and one product by alpha: gamma_(K+1) |a| |b|
     bound = (K + 1) * 2.0 ** -24 * 1.01 * 0.75 * (a.abs() @ b.abs())
     assert ((C.double() - 0.75 * (a @ b)).abs() <= bound + 1e-37).all()
+
+
+@pytest.mark.parametrize("n", [1, 3, 5, 4096, 8 * 152 * 256 * 16 + 7])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_split_parts(n, offset):
+    """16-byte and 4-byte accesses give the same two parts: hi truncated to tf32, lo the rest rounded."""
+    x = torch.randn(n + offset, device="cuda")[offset:]
+    hi, lo = S.soap_split_tf32(x)
+    assert torch.equal(hi.view(torch.int32), x.view(torch.int32) & ~0x1FFF)
+    rest = (x - hi).view(torch.int32)  # exact; nearest tf32, ties away from zero
+    assert torch.equal(lo.view(torch.int32), (rest + 0x1000) & ~0x1FFF)
