@@ -425,6 +425,40 @@ __global__ void split_planes_kernel(const float* X, Planes Xp, int64_t rows, int
   }
 }
 
+// 64 rows x 32 columns at a time: the planes as they are, or of the transpose, its rows scaled by d if
+// given; with `tri` the blocks of `tri` rows and columns left of the diagonal ones are taken as zero.
+__global__ void __launch_bounds__(256) split_blocks_kernel(const float* X, int64_t ld, int64_t stride,
+                                                           bool transposed, const float* d, int64_t d_stride, int tri,
+                                                           Planes Xp, int rows, int cols) {
+  __shared__ TileBuf tile;
+  const int b = blockIdx.z;
+  const int r0 = blockIdx.y * kTr, c0 = blockIdx.x * kTc;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const TileIn t(i);
+    const int r = r0 + t.r, c = c0 + t.c;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < rows && c < cols) {
+      if (!tri || c / tri >= r / tri) x = *reinterpret_cast<const float4*>(X + b * stride + r * ld + c);
+      if (!transposed) b3_store4(Xp.p + b * Xp.stride + r * Xp.ld + c, Xp.plane, x);
+    }
+    if (transposed) tile.put(t, x);
+  }
+  if (!transposed) return;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const TileOut t(i);
+    const int c = c0 + t.c, r = r0 + t.r;
+    if (r < rows && c < cols) {
+      float4 x = tile.get(t);
+      const float f = d ? d[b * d_stride + c] : 1.f;
+      x.x *= f; x.y *= f; x.z *= f; x.w *= f;
+      b3_store4(Xp.p + b * Xp.stride + c * Xp.ld + r, Xp.plane, x);
+    }
+  }
+}
+
 // hi (if given) and lo parts; with `vec` (every pointer 16-byte aligned) four values at a time,
 // four units in flight per thread: bound by memory (12 bytes a value; 4-byte accesses took
 // 47 us for 16.8 M values, these 36).
@@ -529,6 +563,16 @@ cudaError_t planes_transpose(const float* X, const Planes& Xp, const Planes& Xtp
   ProfScope prof(kFamElementwise, 0.0, (4.0 + (Xp.p ? 6 : 0) + (Xtp.p ? 6 : 0) + (Xt ? 4 : 0)) * e, s);
   dim3 grid((n + kTc - 1) / kTc, (n + kTr - 1) / kTr, batch);
   planes_transpose_kernel<<<grid, 256, 0, s>>>(X, Xp, Xtp, Xt, n);
+  return cudaGetLastError();
+}
+
+cudaError_t split_blocks(const float* X, int64_t ld, int64_t stride, bool transposed, const float* d, int64_t d_stride,
+                         int tri, const Planes& Xp, int rows, int cols, int batch, cudaStream_t s) {
+  if (rows <= 0 || cols <= 0 || batch <= 0) return cudaSuccess;
+  if (((rows | cols | ld | stride | tri) & 3) || batch > 65535) return cudaErrorInvalidValue;
+  ProfScope prof(kFamElementwise, 0.0, 10.0 * rows * cols * batch, s);
+  const dim3 grid((cols + kTc - 1) / kTc, (rows + kTr - 1) / kTr, batch);
+  split_blocks_kernel<<<grid, 256, 0, s>>>(X, ld, stride, transposed, d, d_stride, tri, Xp, rows, cols);
   return cudaGetLastError();
 }
 

@@ -24,8 +24,8 @@
 // tile (a pair's N = 128 MMA takes as long as its N = 256).
 //
 // CTA: warp 0 issues the TMA loads, warp 1 allocates tensor memory and (in the pair's first CTA)
-// issues the MMAs, warps 2-9 drain the accumulators and store the tile through swizzled 32 x 32
-// blocks in shared memory. Stages are handed over with mbarriers; every wait gives up after a
+// issues the MMAs, warps 2-17 drain the accumulators and store the tile through swizzled blocks in
+// shared memory. Stages are handed over with mbarriers; every wait gives up after a
 // bounded time (2 s of %globaltimer time unless soap_wait_limit set another), records
 // kStatusTimeout and lets the CTAs drain -- copies already issued land, issued MMAs complete -- and
 // free their tensor memory. The drains themselves always keep the full 2 s bound.
@@ -50,12 +50,15 @@ constexpr int BM = 128;  // rows of A per CTA
 constexpr int BK = 64;   // bf16 elements per K block = one 128-byte swizzle row
 constexpr int STAGES = 2;
 constexpr int NACC = 2;
-constexpr int EPI = 8;
+// Epilogue warps, each a quarter of the tile's columns: with 16 more loads of C are in flight than with
+// 8 (16 of 2048 x 2048 x 512, C read and written as planes: 0.54 ms with 8, 0.44 with 16; 64 of
+// 2048 x 768 x 768, written only: 0.60 and 0.57; 8192 x 8192 x 512 with C in fp32: 0.326 and 0.333)
+constexpr int EPI = 16;
 constexpr int THREADS = 64 + 32 * EPI;
 constexpr int PLANE_A = BM * BK * 2;
 constexpr uint64_t kWaitNs = 2000000000ull;
 
-enum : int { kF32 = 1, kPlanes = 2, kTr = 4, kBeta = 8, kSym = 16 };
+enum : int { kF32 = 1, kPlanes = 2, kTr = 4, kBeta = 8, kSym = 16, kBetaP = 32 };
 
 // CG CTAs work on a CG * 128 x BN tile, each with its 128 rows of A and BN / CG rows of B.
 template <int CG, int BN>
@@ -63,9 +66,9 @@ struct Cfg {
   static constexpr int BROWS = BN / CG;
   static constexpr int PLANE_B = BROWS * BK * 2;
   static constexpr int STAGE = 3 * (PLANE_A + PLANE_B);
-  static constexpr int CPW = BN / 2;  // accumulator columns drained by one warp
+  static constexpr int CPW = BN * 4 / EPI;  // accumulator columns drained by one warp
   static constexpr int NCH = CPW / 32;
-  static constexpr int SMEM = STAGES * STAGE + EPI * 4096 + 1024 + 256;
+  static constexpr int SMEM = STAGES * STAGE + EPI * 2048 + 1024 + 256;
   static constexpr uint32_t TMEM_COLS = NACC * BN;
   static_assert(SMEM <= 232448, "shared memory budget");
 };
@@ -101,6 +104,8 @@ __device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, u
 // XOR-swizzled by r mod 8: a warp touching one 16-byte unit per row, or one row, is
 // conflict-free.
 __device__ __forceinline__ int swz(int r, int j) { return r * 32 + ((((j >> 2) ^ (r & 7))) << 2) + (j & 3); }
+// The same for a 32 x 16 block (two rows to a 128-byte line), element (r, 4 q).
+__device__ __forceinline__ int swzh(int r, int q) { return r * 16 + ((q ^ ((r >> 1) & 3)) << 2); }
 __device__ __forceinline__ int swz16(int r, int q) { return (r >> 3) * 1024 + (r & 7) * 128 + ((q ^ (r & 7)) << 4); }
 
 // Tile t of a launch -> (m0, n0, batch index). Within a matrix the tiles go in groups of GM row
@@ -130,6 +135,10 @@ __device__ __forceinline__ void tile_coords_sym(int t, int ntm, int tile, int& m
   n0 = (r - i * (i + 1) / 2) * tile;
 }
 
+__device__ __forceinline__ float4 b3_unit4(int i, float x) {
+  return make_float4(i == 0 ? x : 0.f, i == 1 ? x : 0.f, i == 2 ? x : 0.f, i == 3 ? x : 0.f);
+}
+
 struct Args {
   int M, N, K, batch, a_mod, b_mod;
   B3Epilogue ep;
@@ -144,11 +153,11 @@ __global__ void __launch_bounds__(THREADS, 1)
     gemm_b3_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
                    const __grid_constant__ Args p) {
   using C = Cfg<CG, BN>;
-  constexpr bool F32 = MODE & kF32, PL = MODE & kPlanes, TR = MODE & kTr, BETA = MODE & kBeta, SYM = MODE & kSym;
+  constexpr bool F32 = MODE & kF32, PL = MODE & kPlanes, TR = MODE & kTr, BETA = MODE & kBeta, SYM = MODE & kSym, BETAP = MODE & kBetaP;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   float* obuf_all = reinterpret_cast<float*>(smem + STAGES * C::STAGE);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * C::STAGE + EPI * 4096);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * C::STAGE + EPI * 2048);
   uint64_t* empty = full + STAGES;
   uint64_t* acc_full = empty + STAGES;
   uint64_t* acc_empty = acc_full + NACC;
@@ -290,7 +299,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int ew = warp - 2;
     const int colbase = (ew / 4) * C::CPW;
     const uint32_t lane_base = tmem + (static_cast<uint32_t>(32 * q) << 16);
-    float* cb = obuf_all + ew * 1024;
+    float* cb = obuf_all + ew * 512;
     int g = 0;
     bool valid = true;
     if (ep.hold && !flag_wait(ep.hold, lim)) {
@@ -304,6 +313,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       tile(t, m0, n0, b);
       float* Cb = F32 ? (ep.C_ptrs ? ep.C_ptrs[b] : ep.C + (int64_t)b * ep.c_stride) : nullptr;
       __nv_bfloat16* Pb = PL ? ep.P + (int64_t)b * ep.p_stride : nullptr;
+      const __nv_bfloat16* Ib = BETAP ? ep.cin + (int64_t)b * ep.p_stride : nullptr;
+      const float* Db = BETAP ? ep.cin_diag + (int64_t)b * ep.cin_diag_stride : nullptr;
       const int row0 = m0 + rank * BM + 32 * q;  // first of this warp's 32 rows
       const int col0 = n0 + colbase;             // first of its CPW columns
       if (BETA) {
@@ -315,6 +326,15 @@ __global__ void __launch_bounds__(THREADS, 1)
           if (r < p.M && col < p.N)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(TR ? Cb + (int64_t)col * ep.ldc + r
                                                              : Cb + (int64_t)r * ep.ldc + col));
+        }
+      }
+      if (BETAP) {
+        static_assert(C::CPW <= 64, "one line of each plane per row");
+        const int r = row0 + lane, col = col0;
+        if (r < p.M && col < p.N && r >= ep.cin_from && col >= ep.cin_from) {
+#pragma unroll
+          for (int pl = 0; pl < 3; ++pl)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(Ib + pl * ep.p_plane + (int64_t)r * ep.p_ld + col));
         }
       }
       float acc[C::NCH][32];
@@ -349,94 +369,93 @@ __global__ void __launch_bounds__(THREADS, 1)
         break;
       }
       if (row0 >= p.M) continue;
-      // out = alpha acc + beta C through the warp's shared block; C, its rows and columns come in
-      // whole 16-byte units (checked on the host)
+      // out = alpha acc + beta C through the warp's shared block, 32 rows x 16 columns at a time; C, its
+      // rows and columns come in whole 16-byte units (checked on the host)
 #pragma unroll
-      for (int c = 0; c < C::NCH; ++c) {
-        const int cc0 = col0 + 32 * c;
+      for (int ch = 0; ch < 2 * C::NCH; ++ch) {
+        const float* av = &acc[ch >> 1][16 * (ch & 1)];
+        const int cc0 = col0 + 16 * ch;
         if (!TR) {
-#pragma unroll
-          for (int j4 = 0; j4 < 8; ++j4)
-            *reinterpret_cast<float4*>(cb + swz(lane, 4 * j4)) =
-                make_float4(ep.alpha * acc[c][4 * j4], ep.alpha * acc[c][4 * j4 + 1], ep.alpha * acc[c][4 * j4 + 2],
-                            ep.alpha * acc[c][4 * j4 + 3]);
-          __syncwarp();
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
-            float4 cv[4];
-            if (BETA) {
-#pragma unroll
-              for (int it = 0; it < 4; ++it) {
-                const int r2 = row0 + 16 * hf + 4 * it + (lane >> 3), col = cc0 + 4 * (lane & 7);
-                cv[it] = (r2 < p.M && col < p.N) ? *reinterpret_cast<const float4*>(Cb + (int64_t)r2 * ep.ldc + col)
-                                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-              }
-            }
+          const int col = cc0 + 4 * (lane & 3), rl = lane >> 2;  // this lane's unit, in rows rl + 8 it
+          float4 cv[4];
+          if (BETA || BETAP) {
 #pragma unroll
             for (int it = 0; it < 4; ++it) {
-              const int rr = 16 * hf + 4 * it + (lane >> 3), j4 = lane & 7;
-              const int r2 = row0 + rr, col = cc0 + 4 * j4;
-              float4* slot = reinterpret_cast<float4*>(cb + swz(rr, 4 * j4));
-              float4 o = *slot;
-              if (BETA) {
-                o.x = fmaf(ep.beta, cv[it].x, o.x);
-                o.y = fmaf(ep.beta, cv[it].y, o.y);
-                o.z = fmaf(ep.beta, cv[it].z, o.z);
-                o.w = fmaf(ep.beta, cv[it].w, o.w);
-                if (SYM) *slot = o;
-              }
+              const int r2 = row0 + 8 * it + rl;
+              cv[it] = make_float4(0.f, 0.f, 0.f, 0.f);
               if (r2 < p.M && col < p.N) {
-                if (F32) *reinterpret_cast<float4*>(Cb + (int64_t)r2 * ep.ldc + col) = o;
-                if (PL) b3_store4(Pb + (int64_t)r2 * ep.p_ld + col, ep.p_plane, o);
+                if (BETA) cv[it] = *reinterpret_cast<const float4*>(Cb + (int64_t)r2 * ep.ldc + col);
+                else if (r2 >= ep.cin_from && col >= ep.cin_from)
+                  cv[it] = b3_load4(Ib + (int64_t)r2 * ep.p_ld + col, ep.p_plane);
+                else if ((unsigned)(r2 - col) < 4u) cv[it] = b3_unit4(r2 - col, Db[r2]);
               }
+            }
+          }
+#pragma unroll
+          for (int j4 = 0; j4 < 4; ++j4)
+            *reinterpret_cast<float4*>(cb + swzh(lane, j4)) = make_float4(
+                ep.alpha * av[4 * j4], ep.alpha * av[4 * j4 + 1], ep.alpha * av[4 * j4 + 2], ep.alpha * av[4 * j4 + 3]);
+          __syncwarp();
+#pragma unroll
+          for (int it = 0; it < 4; ++it) {
+            const int rr = 8 * it + rl, r2 = row0 + rr;
+            float4* slot = reinterpret_cast<float4*>(cb + swzh(rr, lane & 3));
+            float4 o = *slot;
+            if (BETA || BETAP) {
+              o.x = fmaf(ep.beta, cv[it].x, o.x);
+              o.y = fmaf(ep.beta, cv[it].y, o.y);
+              o.z = fmaf(ep.beta, cv[it].z, o.z);
+              o.w = fmaf(ep.beta, cv[it].w, o.w);
+              if (SYM) *slot = o;
+            }
+            if (r2 < p.M && col < p.N) {
+              if (F32) *reinterpret_cast<float4*>(Cb + (int64_t)r2 * ep.ldc + col) = o;
+              if (PL) b3_store4(Pb + (int64_t)r2 * ep.p_ld + col, ep.p_plane, o);
             }
           }
           if (SYM && m0 != n0) {
             // the mirror tile: element (r, j) of this block also goes to C[j][r]
             __syncwarp();
 #pragma unroll 1
-            for (int it = 0; it < 8; ++it) {
+            for (int it = 0; it < 4; ++it) {
               const int jj = 4 * it + (lane >> 3), r4 = 4 * (lane & 7);
               const int mrow = cc0 + jj, mcol = row0 + r4;  // row and column in C
               if (mrow >= p.N || mcol >= p.M) continue;     // M = N, a multiple of 4
-              const float4 o = make_float4(cb[swz(r4, jj)], cb[swz(r4 + 1, jj)], cb[swz(r4 + 2, jj)],
-                                           cb[swz(r4 + 3, jj)]);
+              auto at = [&](int r) { return cb[swzh(r, jj >> 2) + (jj & 3)]; };
+              const float4 o = make_float4(at(r4), at(r4 + 1), at(r4 + 2), at(r4 + 3));
               if (F32) *reinterpret_cast<float4*>(Cb + (int64_t)mrow * ep.ldc + mcol) = o;
               if (PL) b3_store4(Pb + (int64_t)mrow * ep.p_ld + mcol, ep.p_plane, o);
             }
           }
           __syncwarp();
         } else {
-          // C^T: element (row r = this lane, column j) goes to row j of the staged block
-#pragma unroll
-          for (int j = 0; j < 32; ++j) cb[swz(j, lane)] = ep.alpha * acc[c][j];
-          __syncwarp();
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
-            float4 cv[4];
-            if (BETA) {
-#pragma unroll
-              for (int it = 0; it < 4; ++it) {
-                const int col = cc0 + 16 * hf + 4 * it + (lane >> 3), r2 = row0 + 4 * (lane & 7);
-                cv[it] = (r2 < p.M && col < p.N) ? *reinterpret_cast<const float4*>(Cb + (int64_t)col * ep.ldc + r2)
-                                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-              }
-            }
+          // C^T: element (row r = this lane, column j) goes to row j of the staged 16 x 32 block
+          const int r2 = row0 + 4 * (lane & 7), jl = lane >> 3;  // this lane's unit, in rows jl + 4 it
+          float4 cv[4];
+          if (BETA) {
 #pragma unroll
             for (int it = 0; it < 4; ++it) {
-              const int jj = 16 * hf + 4 * it + (lane >> 3), r4 = lane & 7;
-              const int col = cc0 + jj, r2 = row0 + 4 * r4;
-              float4 o = *reinterpret_cast<const float4*>(cb + swz(jj, 4 * r4));
-              if (BETA) {
-                o.x = fmaf(ep.beta, cv[it].x, o.x);
-                o.y = fmaf(ep.beta, cv[it].y, o.y);
-                o.z = fmaf(ep.beta, cv[it].z, o.z);
-                o.w = fmaf(ep.beta, cv[it].w, o.w);
-              }
-              if (r2 < p.M && col < p.N) {
-                if (F32) *reinterpret_cast<float4*>(Cb + (int64_t)col * ep.ldc + r2) = o;
-                if (PL) b3_store4(Pb + (int64_t)col * ep.p_ld + r2, ep.p_plane, o);
-              }
+              const int col = cc0 + 4 * it + jl;
+              cv[it] = (r2 < p.M && col < p.N) ? *reinterpret_cast<const float4*>(Cb + (int64_t)col * ep.ldc + r2)
+                                               : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 16; ++j) cb[swz(j, lane)] = ep.alpha * av[j];
+          __syncwarp();
+#pragma unroll
+          for (int it = 0; it < 4; ++it) {
+            const int jj = 4 * it + jl, col = cc0 + jj;
+            float4 o = *reinterpret_cast<const float4*>(cb + swz(jj, 4 * (lane & 7)));
+            if (BETA) {
+              o.x = fmaf(ep.beta, cv[it].x, o.x);
+              o.y = fmaf(ep.beta, cv[it].y, o.y);
+              o.z = fmaf(ep.beta, cv[it].z, o.z);
+              o.w = fmaf(ep.beta, cv[it].w, o.w);
+            }
+            if (r2 < p.M && col < p.N) {
+              if (F32) *reinterpret_cast<float4*>(Cb + (int64_t)col * ep.ldc + r2) = o;
+              if (PL) b3_store4(Pb + (int64_t)col * ep.p_ld + r2, ep.p_plane, o);
             }
           }
           __syncwarp();
@@ -572,22 +591,26 @@ cudaError_t gemm_b3(int M, int N, int K, int batch, const B3Operand& A, const B3
   get_wait_limit(&ep.wait_ns, &ep.hold);
   if (batch > 65535 || K <= 0) return cudaErrorInvalidValue;
   const bool f32 = ep.C || ep.C_ptrs, pl = ep.P != nullptr, tr = ep.transpose != 0, beta = ep.beta != 0.f;
+  const bool betap = beta && ep.cin;
   // outputs are read and written in 16-byte units of fp32 (8-byte units of a plane)
   const int along = tr ? M : N;
-  if ((along & 3) || f32 == pl || (beta && !f32) || (f32 && ((ep.ldc & 3) || (ep.c_stride & 3) || !al16(ep.C))) ||
-      (pl && ((ep.p_ld & 3) || (ep.p_stride & 3) || (ep.p_plane & 3) || !al16(ep.P))))
+  if ((along & 3) || f32 == pl || (beta && !f32 && !betap) || (betap && (tr || (pl && ep.cin != ep.P))) || (f32 && ((ep.ldc & 3) || (ep.c_stride & 3) || !al16(ep.C))) ||
+      ((pl || betap) && ((ep.p_ld & 3) || (ep.p_stride & 3) || (ep.p_plane & 3) || !al16(ep.P) || !al16(ep.cin))))
     return cudaErrorInvalidValue;
   const double e = (double)M * N * batch;
   const double flops = 2.0 * e * K;  // algorithmic (six bf16 products each on the pipe)
   const double bytes = 6.0 * (double)M * K * (A.batch > 0 ? A.batch : batch) +
-                       6.0 * (double)N * K * (B.batch > 0 ? B.batch : batch) + e * (pl ? 6.0 : beta ? 8.0 : 4.0);
+                       6.0 * (double)N * K * (B.batch > 0 ? B.batch : batch) + e * ((pl ? 6.0 : 4.0) + (betap ? 6.0 : beta ? 4.0 : 0.0));
   ProfScope prof(family, flops, bytes, s);
   if (tr) {
     if (pl) return launch_shape<kPlanes | kTr>(M, N, K, batch, A, B, ep, s);
     return beta ? launch_shape<kF32 | kTr | kBeta>(M, N, K, batch, A, B, ep, s)
                 : launch_shape<kF32 | kTr>(M, N, K, batch, A, B, ep, s);
   }
-  if (pl) return cudaErrorInvalidValue;  // no caller has one
+  if (betap)
+    return pl ? launch_shape<kPlanes | kBetaP>(M, N, K, batch, A, B, ep, s)
+              : launch_shape<kF32 | kBetaP>(M, N, K, batch, A, B, ep, s);
+  if (pl) return launch_shape<kPlanes>(M, N, K, batch, A, B, ep, s);
   return beta ? launch_shape<kF32 | kBeta>(M, N, K, batch, A, B, ep, s)
               : launch_shape<kF32>(M, N, K, batch, A, B, ep, s);
 }

@@ -13,14 +13,15 @@
 //       I - V T V^T); where it leaves a matrix to the column loop, qr_panel_kernel factors
 //       that matrix's block in 32-column panels in distributed shared memory, with the same
 //       results;
-//     VTr = V T^T and VTq = V T                     (tensor cores, K = 128)
+//     VTr = V T^T                                   (tensor cores, K = 128)
 //     trailing rows r >= k0+128: a_r <- a_r - (a_r V) T V^T, i.e.
 //       W  = At_trail Vt^T                          (tensor cores: N = 128, K = positions)
 //       At_trail -= W VTr^T                         (tensor cores: K = 128, C read in place)
-//   then Q^T is accumulated backwards from diag(d) (d_j = sign of R_jj) one block at a
-//   time, Q^T <- Q^T (I - V T^T V^T):
-//       W = Qt_sub Vt^T ;  Qt_sub -= W VTq^T
-//   and Q = (Q^T)^T.
+//   then Q^T is accumulated backwards from diag(d) (d_j = sign of R_jj) a superblock of three or
+//   four blocks, with one T, at a time, Q^T <- Q^T (I - V T^T V^T), on operands in bf16 planes:
+//       W = (Qt_sub Vt^T) T^T ;  Qt_sub -= W V^T
+//   and Q = (Q^T)^T. (A block at a time, in TF32, this took 2.2 of the 6.6 ms of 16 matrices of
+//   2048 rows; so 1.4, and 0.5 more for the superblocks' T.)
 //
 // The column loop's panel of an n x n matrix spans up to n positions; it is spread over a
 // thread-block cluster of ceil((n-k0)/512) CTAs (<= 16 for n <= 8192), 512 positions each, or,
@@ -997,6 +998,24 @@ __global__ void frob_partial_kernel(const float* P, int64_t nn, double* part) {
   }
 }
 
+// T_j of a superblock's block into its place in the superblock's T, zeros left of it.
+__global__ void put_block_kernel(const float* T, const float* T_lo, float* D, float* D_lo, int64_t stride, int ld,
+                                 int off, int w) {
+  const int b = blockIdx.y, cols4 = (off + w) / 4;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < w * cols4; e += gridDim.x * blockDim.x) {
+    const int r = e / cols4, c = 4 * (e - r * cols4);
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+    if (c >= off) {
+      const int64_t o = ((int64_t)b * NBO + r) * NBO + c - off;
+      x = *reinterpret_cast<const float4*>(T + o);
+      y = *reinterpret_cast<const float4*>(T_lo + o);
+    }
+    const int64_t d = b * stride + (int64_t)(off + r) * ld + c;
+    *reinterpret_cast<float4*>(D + d) = x;
+    *reinterpret_cast<float4*>(D_lo + d) = y;
+  }
+}
+
 // The zero-column threshold tol * ||P_b||_F; a non-finite norm (a NaN or Inf anywhere in P_b,
 // wherever the Householder steps would meet it) is a breakdown of that QR.
 __global__ void thresh_kernel(const double* part, float tol, int batch, float* thresh, int* status) {
@@ -1006,18 +1025,6 @@ __global__ void thresh_kernel(const double* part, float tol, int batch, float* t
   for (int i = 0; i < NORM_CHUNKS; ++i) s += part[(int64_t)b * NORM_CHUNKS + i];
   if (!isfinite(s) && status) atomicOr(status, kStatusQrBreakdown);
   thresh[b] = (float)((double)tol * sqrt(s));
-}
-
-// Q^T <- diag(d)
-__global__ void signed_identity_kernel(float* Qt, const float* d, int n) {
-  const int b = blockIdx.y;
-  const int64_t nn = (int64_t)n * n;
-  float* q = Qt + (int64_t)b * nn;
-  const float* db = d + (int64_t)b * n;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / n, cc = i % n;
-    q[i] = r == cc ? db[r] : 0.f;
-  }
 }
 
 // The panel kernel variant for this device: 512 positions per CTA in clusters of up to 16
@@ -1076,23 +1083,21 @@ cudaError_t panel_kernel(PanelKernel* pk, int n) {
 
 struct Workspace {
   float* At;
-  float* At_lo;   // unused (null): the products form A's lo part themselves
+  float* Vt_lo;   // after At: the two hold the planes of Q^T once the factorisation is over
   float* Vt;
-  float* Vt_lo;
-  float* VTq;     // [batch][nblock][n][NBO] V T of every block (kept for the Q accumulation)
-  float* VTq_lo;
-  float* VTr;     // [batch][n][NBO] V T^T of the current block
-  float* VTr_lo;
+  float* Tg;      // T of every superblock (see superblock()), then one operand of the Q accumulation
+  float* VTr;     // [batch][n][NBO] V T^T of the current block; from here to Wsplit's end also the
+  float* VTr_lo;  // operand planes of the Q accumulation
   float* Vpos;    // [batch][n][NBO]
   float* Vpos_lo;
   float* W;       // [batch][n][NBO]
   float* W_lo;
+  float* Wsplit;  // [KSPLIT][batch][n][NBO] partial sums of split-K products
   float* T;       // [batch][NBO][NBO], and T^T, each with its lo part
   float* T_lo;
   float* Tt;
   float* Tt_lo;
   float* Ypart;   // [batch][MAXC][NBO][NB]
-  float* Wsplit;  // [KSPLIT][batch][n][NBO] partial sums of split-K products
   // for the look-ahead schedule only (null otherwise): the far update's own W and split-K
   // buffers, and second V T^T, Vpos and T buffers (blocks alternate: a block's V T^T is read
   // by its far update and its Vpos and T by its V T while the next block is factored)
@@ -1112,6 +1117,27 @@ struct Workspace {
   double* part;
 };
 
+// The Q accumulation goes by superblocks of up to 4 blocks (512 columns): its last product reads and
+// writes all of Q^T from the superblock on, so fewer, wider ones move less (16 of 2048 x 2048: four
+// times 160 us with K = 128 and fp32 Q^T, 393 us with K = 512 and planes). 3 blocks below n = 1024, where the three operands of 4 do
+// not fit the workspace that the factorisation leaves free.
+struct Superblock {
+  int ks, j, wk, blocks;      // first column, the block's index in it, its columns and blocks
+  int64_t t_off, t_stride;    // its T (wk x wk) in a matrix's array, and between matrices (floats)
+};
+Superblock superblock(int n, int blk) {
+  const int nblock = (n + NBO - 1) / NBO, per = n >= 1024 ? 4 : 3, sb = blk / per;
+  const int64_t w = per * NBO, full = n / w, rest = n - full * w;
+  Superblock o;
+  o.ks = (int)(sb * w);
+  o.j = blk - sb * per;
+  o.wk = (int)std::min<int64_t>(w, n - o.ks);
+  o.blocks = std::min(per, nblock - sb * per);
+  o.t_off = sb * w * w;
+  o.t_stride = full * w * w + rest * rest;
+  return o;
+}
+
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 Workspace carve(void* base, int n, int batch, size_t* total, bool lookahead) {
@@ -1126,12 +1152,12 @@ Workspace carve(void* base, int n, int batch, size_t* total, bool lookahead) {
   const size_t blocks = (size_t)batch * nblock * n * NBO * sizeof(float);
   const size_t thin = (size_t)batch * n * NBO * sizeof(float);
   const size_t tsq = (size_t)batch * NBO * NBO * sizeof(float);
-  const size_t oAt = take(mat), oVt = take(mat), oVtl = take(mat);
-  const size_t oVq = take(blocks), oVql = take(blocks), oVr = take(thin), oVrl = take(thin);
+  const size_t oAt = take(mat), oVtl = take(mat), oVt = take(mat);
+  const size_t oTg = take(2 * blocks), oVr = take(thin), oVrl = take(thin);
   const size_t oVp = take(thin), oVpl = take(thin), oW = take(thin), oWl = take(thin);
+  const size_t oWs = take((size_t)KSPLIT * thin);
   const size_t oT = take(tsq), oTl = take(tsq), oTt = take(tsq), oTtl = take(tsq);
   const size_t oY = take((size_t)batch * MAXC * NBO * NB * sizeof(float));
-  const size_t oWs = take((size_t)KSPLIT * thin);
   const size_t oW2 = lookahead ? take(thin) : 0, oW2l = lookahead ? take(thin) : 0;
   const size_t oWs2 = lookahead ? take((size_t)KSPLIT * thin) : 0;
   const size_t oVr2 = lookahead ? take(thin) : 0, oVr2l = lookahead ? take(thin) : 0;
@@ -1145,8 +1171,8 @@ Workspace carve(void* base, int n, int batch, size_t* total, bool lookahead) {
   char* c = (char*)base;
   auto f = [&](size_t o) { return (float*)(c + o); };
   auto g = [&](size_t o) { return lookahead ? (float*)(c + o) : nullptr; };
-  return Workspace{f(oAt), nullptr, f(oVt), f(oVtl), f(oVq), f(oVql), f(oVr), f(oVrl), f(oVp),  f(oVpl),
-                   f(oW),  f(oWl),  f(oT),  f(oTl),  f(oTt), f(oTtl), f(oY),  f(oWs), g(oW2),  g(oW2l),
+  return Workspace{f(oAt), f(oVtl), f(oVt), f(oTg), f(oVr), f(oVrl), f(oVp),  f(oVpl),
+                   f(oW),  f(oWl),  f(oWs), f(oT),  f(oTl),  f(oTt), f(oTtl), f(oY),  g(oW2),  g(oW2l),
                    g(oWs2), g(oVr2), g(oVr2l), g(oVp2), g(oVp2l), g(oT2),  g(oT2l),  g(oTt2), g(oTt2l),
                    f(oth), f(osg), (double*)(c + opart)};
 }
@@ -1173,7 +1199,7 @@ void qr_input_buffers(void* workspace, int n, int batch, float** At) {
 }
 
 cudaError_t qr_q_t(int n, int batch, float* Q, uint8_t* skip, float tol, void* workspace, size_t workspace_bytes,
-                   int* status, cudaStream_t s, const QrLookahead* lah) {
+                   int* status, cudaStream_t s, const QrLookahead* lah, float** Qt_out) {
   if (n <= 0 || batch <= 0) return cudaSuccess;
   if (n > 8192 || batch > 65535 || (n & 3)) return cudaErrorInvalidValue;
   // look-ahead: a second stream and its events given, and a workspace sized for it
@@ -1184,9 +1210,8 @@ cudaError_t qr_q_t(int n, int batch, float* Q, uint8_t* skip, float tol, void* w
   size_t need = 0;
   Workspace w = carve(workspace, n, batch, &need, la);
   if (workspace_bytes < need) return cudaErrorInvalidValue;
-  float* Qt = w.At;  // the Q accumulation reuses the factored matrix's buffer
   const int nblock = (n + NBO - 1) / NBO;
-  const int64_t nn = (int64_t)n * n, thin = (int64_t)n * NBO, vq_stride = (int64_t)nblock * thin;
+  const int64_t nn = (int64_t)n * n, thin = (int64_t)n * NBO;
   cudaError_t e;
 
   {
@@ -1255,22 +1280,42 @@ cudaError_t qr_q_t(int n, int batch, float* Q, uint8_t* skip, float tol, void* w
       e = cudaLaunchKernelEx(&cfg, pk.fn, a);
       if (e != cudaSuccess) return e;
     }
-    // VTq = V T (the Q accumulation) and VTr = V T^T (this block's trailing update); with the
-    // look-ahead the V T^T buffers alternate between blocks, since the far update of block b
-    // still reads its V T^T while block b+1 forms its own
+    // VTr = V T^T (this block's trailing update); with the look-ahead the V T^T buffers alternate
+    // between blocks, since the far update of block b still reads its V T^T while block b+1 forms
+    // its own
     float* vtr = alt ? w.VTr2 : w.VTr;
     float* vtr_lo = alt ? w.VTr2_lo : w.VTr_lo;
-    float* vq = w.VTq + (int64_t)blk * thin + (int64_t)k0 * NBO;
-    float* vq_lo = w.VTq_lo + (int64_t)blk * thin + (int64_t)k0 * NBO;
     const TcOperand vpos = op(vp + (int64_t)k0 * NBO, vp_lo + (int64_t)k0 * NBO, NBO, thin, batch);
-    auto form_vtq = [&](cudaStream_t st) {
-      return gemm_tc_nt(m, kbo, kbo, batch, vpos, op(Ttb, Ttb_lo, NBO, NBO * NBO, batch),
-                        out(vq, vq_lo, NBO, vq_stride, 1.f, 0.f, status), st, kFamQrUpdate);
+    // The superblock's H_ks ... H_k0+kbo-1 = I - V T V^T: block j's columns of T are
+    // [-T_prev X ; T_j] with X = (V_prev^T V_j) T_j. All on one stream, in order; the block's W and
+    // V T^T buffers are free by then (its trailing update has read them).
+    auto grow_t = [&](cudaStream_t st) -> cudaError_t {
+      const Superblock sb = superblock(n, blk);
+      if (sb.blocks == 1) return cudaSuccess;  // the block's own T is all of it
+      float* t = w.Tg + sb.t_off;
+      float* t_lo = t + batch * sb.t_stride;
+      const int kp = k0 - sb.ks;  // columns before this block
+      {
+        ProfScope prof(kFamOther, 0.0, 16.0 * kbo * (kp + kbo) * batch, st);
+        put_block_kernel<<<dim3(8, batch), 256, 0, st>>>(Tb, Tb_lo, t, t_lo, sb.t_stride, sb.wk, kp, kbo);
+      }
+      cudaError_t e2 = cudaGetLastError();
+      if (e2 != cudaSuccess || kp == 0) return e2;
+      float* g = la ? w.W2 : w.W;
+      float* g_lo = la ? w.W2_lo : w.W_lo;
+      const int64_t vp0 = (int64_t)sb.ks * n + k0, vj0 = (int64_t)k0 * n + k0;
+      e2 = gemm_tc_nt(kp, kbo, m, batch, op(w.Vt + vp0, w.Vt_lo + vp0, n, nn, batch),
+                      op(w.Vt + vj0, w.Vt_lo + vj0, n, nn, batch), out(g, g_lo, NBO, thin, 1.f, 0.f, status), st,
+                      kFamQrUpdate, la ? w.Wsplit2 : w.Wsplit, (size_t)KSPLIT * batch * n * NBO);
+      if (e2 != cudaSuccess) return e2;
+      TcEpilogue xt = out(vtr, vtr_lo, kp, thin, 1.f, 0.f, status);  // X^T
+      xt.transpose = 1;
+      e2 = gemm_tc_nt(kp, kbo, kbo, batch, op(g, g_lo, NBO, thin, batch), op(Ttb, Ttb_lo, NBO, NBO * NBO, batch), xt,
+                      st, kFamQrUpdate);
+      if (e2 != cudaSuccess) return e2;
+      return gemm_tc_nt(kp, kbo, kp, batch, op(t, t_lo, sb.wk, sb.t_stride, batch), op(vtr, vtr_lo, kp, thin, batch),
+                        out(t + kp, t_lo + kp, sb.wk, sb.t_stride, -1.f, 0.f, status), st, kFamQrUpdate);
     };
-    if (!la) {
-      e = form_vtq(s);
-      if (e != cudaSuccess) return e;
-    }
     const int nc = n - k0 - kbo;  // trailing rows of At (columns of P)
     if (nc > 0) {
       e = gemm_tc_nt(m, kbo, kbo, batch, vpos, op(Tb, Tb_lo, NBO, NBO * NBO, batch),
@@ -1278,7 +1323,6 @@ cudaError_t qr_q_t(int n, int batch, float* Q, uint8_t* skip, float tol, void* w
                      kFamQrUpdate);
       if (e != cudaSuccess) return e;
     }
-    if (nc <= 0 && !la) continue;
     const TcOperand vtr_trail =
         op(vtr + (int64_t)(k0 + kbo) * NBO, vtr_lo + (int64_t)(k0 + kbo) * NBO, NBO, thin, batch);
     const TcOperand vt_blk = op(w.Vt + (int64_t)k0 * n + k0, w.Vt_lo + (int64_t)k0 * n + k0, n, nn, batch);
@@ -1296,13 +1340,14 @@ cudaError_t qr_q_t(int n, int batch, float* Q, uint8_t* skip, float tol, void* w
                         kFamQrUpdate);
     };
     if (!la) {
-      e = update_rows(k0 + kbo, nc, w.W, w.W_lo, w.Wsplit, s);
+      e = nc > 0 ? update_rows(k0 + kbo, nc, w.W, w.W_lo, w.Wsplit, s) : cudaSuccess;
+      if (e == cudaSuccess) e = grow_t(s);
       if (e != cudaSuccess) return e;
       continue;
     }
     // look-ahead: the next block's rows now (they gate its panels), the rest on the far stream,
     // where it overlaps the next block's panels; the next block's rows wait for the previous
-    // far update, which covered them. The block's V T follows its far update on the far stream.
+    // far update, which covered them. The block's part of T follows its far update there.
     const int knext = std::min(NBO, std::max(nc, 0));
     // (the far update starts once the next block's rows are done, so that those small products
     // do not wait for SMs behind it)
@@ -1313,40 +1358,72 @@ cudaError_t qr_q_t(int n, int batch, float* Q, uint8_t* skip, float tol, void* w
     if (e == cudaSuccess) e = cudaStreamWaitEvent(far, ev_vt, 0);
     if (e == cudaSuccess && nc > knext) e = update_rows(k0 + kbo + knext, nc - knext, w.W2, w.W2_lo, w.Wsplit2, far);
     if (e == cudaSuccess) e = cudaEventRecord(ev_far, far);
-    if (e == cudaSuccess) e = form_vtq(far);
+    if (e == cudaSuccess) e = grow_t(far);
     if (e == cudaSuccess) e = cudaEventRecord(lah->vq[par], far);
     if (e != cudaSuccess) return e;
   }
   if (la) {
-    // the last far update and the last V T before the Q accumulation
+    // the last far update and the last of T before the Q accumulation
     e = cudaEventRecord(ev_far, far);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev_far, 0);
     if (e != cudaSuccess) return e;
   }
 
-  {
-    // Q^T = diag(d) H_n ... H_1 accumulated backwards: start from diag(d)
-    ProfScope prof(kFamOther, 0, 4.0 * nn * batch, s);
-    const int blocks = (int)std::min<int64_t>((nn + 255) / 256, 1024);
-    signed_identity_kernel<<<dim3(blocks, batch), 256, 0, s>>>(Qt, w.dsign, n);
-    e = cudaGetLastError();
+  // Q^T = diag(d) H_n ... H_1 accumulated backwards, a superblock at a time, on planes: the sub-matrix
+  // from ks on becomes Qt_sub - ((Qt_sub V) T^T) V^T, where the superblock's own rows and columns of
+  // Qt_sub are still those of diag(d), and are neither multiplied nor read. With one superblock Q^T
+  // ends in fp32 in place of P^T; else it is kept as planes and the last product writes it in fp32
+  // over V, dead by then.
+  const Superblock last = superblock(n, nblock - 1);
+  const bool one = last.ks == 0;
+  const Planes Qp = planes_in(w.At, n, n, batch);  // over At and Vt_lo
+  float* Qt = one ? w.At : w.Vt;
+  for (int blk = nblock - last.blocks; blk >= 0;) {
+    const Superblock sb = superblock(n, blk);
+    const int m = n - sb.ks, wk = sb.wk;
+    const float* v = w.Vt + (int64_t)sb.ks * n + sb.ks;
+    // operands: W, then V; W T^T; and V^T, then T
+    char* room = reinterpret_cast<char*>(w.VTr);
+    const size_t tall = align256(planes_bytes(m, wk, batch));
+    const Planes A = planes_in(room, m, wk, batch), B = planes_in(room + tall, m, wk, batch);
+    void* third = n >= 1024 ? (void*)((char*)w.Tg + align256(2 * batch * sb.t_stride * sizeof(float))) : room + 2 * tall;
+    const Planes Tp = planes_in(third, wk, wk, batch);
+    auto into = [&](const Planes& o) {
+      B3Epilogue ep{};
+      ep.P = o.p, ep.p_plane = o.plane, ep.p_ld = o.ld, ep.p_stride = o.stride;
+      ep.alpha = 1.f, ep.status = status;
+      return ep;
+    };
+    // Qt_sub V: the rows of diag(d) and, below them, the product with what is accumulated so far
+    e = split_blocks(v, n, nn, true, w.dsign + sb.ks, n, NBO, A, wk, wk, batch, s);
+    if (e == cudaSuccess && m > wk) {
+      const Planes Vp = planes_in(third, wk, m - wk, batch);
+      e = split_blocks(v + wk, n, nn, false, nullptr, 0, 0, Vp, wk, m - wk, batch, s);
+      if (e == cudaSuccess)
+        e = gemm_b3(m - wk, wk, m - wk, batch, b3_op(Qp.at(0, sb.ks + wk, sb.ks + wk), batch), b3_op(Vp, batch),
+                    into(A.at(0, wk)), s, kFamQrUpdate);
+    }
+    if (e == cudaSuccess) {
+      if (sb.blocks == 1) {
+        const float* t = la && (blk & 1) ? w.T2 : w.T;
+        e = split_blocks(t, NBO, NBO * NBO, false, nullptr, 0, 0, Tp, wk, wk, batch, s);
+      } else {
+        e = split_blocks(w.Tg + sb.t_off, wk, sb.t_stride, false, nullptr, 0, NBO, Tp, wk, wk, batch, s);
+      }
+    }
+    if (e == cudaSuccess) e = gemm_b3(m, wk, wk, batch, b3_op(A, batch), b3_op(Tp, batch), into(B), s, kFamQrUpdate);
+    if (e == cudaSuccess) e = split_blocks(v, n, nn, true, nullptr, 0, NBO, A, wk, m, batch, s);
     if (e != cudaSuccess) return e;
+    const Planes Qs = Qp.at(0, sb.ks, sb.ks);
+    B3Epilogue eq = into(Qs);
+    eq.alpha = -1.f, eq.beta = 1.f;
+    eq.cin = Qs.p, eq.cin_diag = w.dsign + sb.ks, eq.cin_diag_stride = n, eq.cin_from = wk;
+    if (sb.ks == 0) eq.P = nullptr, eq.C = Qt, eq.ldc = n, eq.c_stride = nn;
+    e = gemm_b3(m, m, wk, batch, b3_op(B, batch), b3_op(A, batch), eq, s, kFamQrUpdate);
+    if (e != cudaSuccess) return e;
+    blk -= n >= 1024 ? 4 : 3;
   }
-  for (int blk = nblock - 1; blk >= 0; --blk) {
-    const int k0 = blk * NBO, kbo = std::min(NBO, n - k0), m = n - k0;
-    const int64_t sub = (int64_t)k0 * n + k0;
-    // W = Qt_sub Vt^T  (m x kbo)
-    e = gemm_tc_nt(m, kbo, m, batch, op(Qt + sub, nullptr, n, nn, batch),
-                   op(w.Vt + sub, w.Vt_lo + sub, n, nn, batch), out(w.W, w.W_lo, NBO, thin, 1.f, 0.f, status), s,
-                   kFamQrUpdate, w.Wsplit, (size_t)KSPLIT * batch * n * NBO);
-    if (e != cudaSuccess) return e;
-    // Qt_sub -= W VTq^T
-    const int64_t vq = (int64_t)blk * thin + (int64_t)k0 * NBO;
-    e = gemm_tc_nt(m, m, kbo, batch, op(w.W, w.W_lo, NBO, thin, batch),
-                   op(w.VTq + vq, w.VTq_lo + vq, NBO, vq_stride, batch),
-                   out(Qt + sub, nullptr, n, nn, -1.f, 1.f, status), s, kFamQrUpdate);
-    if (e != cudaSuccess) return e;
-  }
+  if (Qt_out) *Qt_out = Qt;
   if (Q) {
     e = planes_transpose(Qt, Planes(), Planes(), Q, n, batch, s);
     if (e != cudaSuccess) return e;
@@ -1363,7 +1440,7 @@ cudaError_t qr_q(int n, int batch, const float* P, float* Q, uint8_t* skip, floa
   // At = P^T
   cudaError_t e = planes_transpose(P, Planes(), Planes(), w.At, n, batch, s);
   if (e != cudaSuccess) return e;
-  return qr_q_t(n, batch, Q, skip, tol, workspace, workspace_bytes, status, s, nullptr);
+  return qr_q_t(n, batch, Q, skip, tol, workspace, workspace_bytes, status, s);
 }
 
 }  // namespace soap

@@ -472,14 +472,14 @@ soap_status_t refresh_group(soap_handle h, const Wave& w, const QrGroup& g, cuda
                               strided(j.left ? v.L : v.R, n, nn), 0.f, strided_mut(at, n, nn), v.count, gs.stream));
     }
   }
-  // the Q accumulation ends with Q^T in the input buffers
+  float* Qt;
   const soap::QrLookahead la{gs.far, gs.ev_vt, gs.ev_far, {gs.ev_vq[0], gs.ev_vq[1]}};
-  SOAP_CUDA(h, soap::qr_q_t(n, g.batch, nullptr, skip, hp.qr_tol, ws, g.ws_bytes, h->d_status, gs.stream, &la));
+  SOAP_CUDA(h, soap::qr_q_t(n, g.batch, nullptr, skip, hp.qr_tol, ws, g.ws_bytes, h->d_status, gs.stream, &la, &Qt));
   for (const QrJob& j : g.jobs) {
     const Slice& sl = w.slices[j.slice];
     const ClassState& c = h->classes[sl.cls];
     const View v = view_of(h, w, sl);
-    const float* qt = At + (int64_t)j.offset * nn;
+    const float* qt = Qt + (int64_t)j.offset * nn;
     float* Q = j.left ? v.QL : v.QR;
     // (views of a CUDA-core slice have no planes: Q alone is written)
     SOAP_CUDA(h, soap::planes_transpose(qt, j.left ? v.QLt : v.QRt, j.left ? v.QLp : v.QRp, Q, n, v.count, gs.stream));

@@ -124,9 +124,15 @@ struct B3Epilogue {
   int* status;             // device status word for a timed-out wait (may be nullptr)
   uint64_t wait_ns;        // set by gemm_b3 from the library's wait settings
   const int* hold;
+  // the C of beta != 0 as planes (layout of P; not transposed): P itself, or P null. Its rows and columns
+  // before cin_from are not read: they are those of diag(d), d_i at cin_diag[b * cin_diag_stride + i].
+  const __nv_bfloat16* cin = nullptr;
+  const float* cin_diag = nullptr;
+  int64_t cin_diag_stride = 0;
+  int cin_from = 0;
 };
-// C_b = alpha A_b B_(b mod B.batch)^T + beta C_b, in fp32 or (transposed only) as planes. The
-// dimension that C's rows run along must be a multiple of 4, C and its rows 16-byte aligned.
+// C_b = alpha A_b B_(b mod B.batch)^T + beta C_b, in fp32 or as planes. The dimension that C's rows
+// run along must be a multiple of 4, C and its rows 16-byte aligned.
 cudaError_t gemm_b3(int M, int N, int K, int batch, const B3Operand& A, const B3Operand& B, const B3Epilogue& ep,
                     cudaStream_t s, int family = kFamGemmTc);
 // C_b = alpha A_b A_b^T + beta C_b (M x M): only the tiles on or below the diagonal are computed,
@@ -160,6 +166,17 @@ __device__ __forceinline__ void b3_split4(float4 x, uint2& h, uint2& m, uint2& l
 __device__ __forceinline__ void b3_store(__nv_bfloat16* p, int64_t plane, float x) {
   b3_split(x, p[0], p[plane], p[2 * plane]);
 }
+__device__ __forceinline__ float4 b3_load4(const __nv_bfloat16* p, int64_t plane) {  // h + m + l, 8-byte aligned
+  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int pl = 2; pl >= 0; --pl) {  // the smallest plane first
+    const uint2 w = *reinterpret_cast<const uint2*>(p + pl * plane);
+    const float2 a = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162&>(w.x));
+    const float2 b = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162&>(w.y));
+    o.x += a.x; o.y += a.y; o.z += b.x; o.w += b.y;
+  }
+  return o;
+}
 __device__ __forceinline__ void b3_store4(__nv_bfloat16* p, int64_t plane, float4 x) {  // 8-byte aligned
   uint2 h, m, l;
   b3_split4(x, h, m, l);
@@ -180,20 +197,20 @@ cudaError_t qr_q(int n, int batch, const float* P, float* Q, uint8_t* skip, floa
                  void* workspace, size_t workspace_bytes, int* status, cudaStream_t stream);
 // Where the factored matrix P^T must be placed before qr_q_t.
 void qr_input_buffers(void* workspace, int n, int batch, float** At);
-// QR of P whose transpose is already in qr_input_buffers(). Leaves Q^T there and, if Q is given,
-// writes Q.
+// QR of P whose transpose is already in qr_input_buffers(). Leaves Q^T in the workspace, contiguous
+// at *Qt (if given), and, if Q is given, writes Q.
 // The look-ahead schedule of qr_q_t: a second (low-priority) stream and its events.
 struct QrLookahead {
-  cudaStream_t far;     // trailing updates beyond the next block, and V T for the Q accumulation
+  cudaStream_t far;     // trailing updates beyond the next block, and the Q accumulation's factors
   cudaEvent_t vt;       // this block's V T^T and the next block's rows are ready (caller's stream)
   cudaEvent_t far_done; // the far update of the previous block is done (recorded on `far`)
-  cudaEvent_t vq[2];    // V T of the block using buffer 0 / 1 is done (recorded on `far`)
+  cudaEvent_t vq[2];    // what the Q accumulation needs of the block using buffer 0 / 1 is done (on `far`)
 };
 // With `la` (all members set, and a workspace sized with lookahead) the trailing update of each
-// 128-column block, except the next block's rows, and the block's V T run on la->far and
-// overlap the next block's panels; everything is joined back on `stream` before return.
+// 128-column block, except the next block's rows, and the block's part of the Q accumulation's
+// factors run on la->far and overlap the next block's panels; everything is joined back on `stream` before return.
 cudaError_t qr_q_t(int n, int batch, float* Q, uint8_t* skip, float tol, void* workspace, size_t workspace_bytes,
-                   int* status, cudaStream_t stream, const QrLookahead* la = nullptr);
+                   int* status, cudaStream_t stream, const QrLookahead* la = nullptr, float** Qt = nullptr);
 
 // bf16 tensor-core product out_b = alpha A_b B_b^T + beta Cin_b (A_b M x K, B_b N x K, bf16
 // row-major; fp32 accumulation). Outputs: out (bf16, ld, stride; Cin has the same layout) and, if
@@ -263,6 +280,12 @@ cudaError_t transpose(const float* src, float* dst, int rows, int cols, int batc
 // and of X^T, and X^T itself.
 cudaError_t planes_transpose(const float* X, const Planes& Xp, const Planes& Xtp, float* Xt, int n, int batch,
                              cudaStream_t stream);
+// The planes of `batch` rows x cols matrices with leading dimension ld, `stride` apart, or of their
+// transposes, whose row i is scaled by d_i (at b * d_stride + i) if d is given; with tri > 0 the
+// tri x tri blocks left of the diagonal ones are taken as zero, whatever they hold (rows, cols and
+// tri multiples of 4).
+cudaError_t split_blocks(const float* X, int64_t ld, int64_t stride, bool transposed, const float* d, int64_t d_stride,
+                         int tri, const Planes& Xp, int rows, int cols, int batch, cudaStream_t stream);
 // The planes of `rows` contiguous rows of cols values (cols a multiple of 4).
 cudaError_t split_planes(const float* X, const Planes& Xp, int64_t rows, int cols, cudaStream_t stream);
 // W <- (1 - lr*wd) W - lr * D (both sides identity).

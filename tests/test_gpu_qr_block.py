@@ -58,3 +58,12 @@ def test_block_factorisation_matches_oracle(cuda, n, batch, kind):
         assert np.abs(Q[b].astype(np.float64).T @ Q[b] - np.eye(n)).max() <= 1e-5
         rel = lambda x: np.linalg.norm(x.astype(np.float64) - Q64) / np.linalg.norm(Q64)  # noqa: E731
         assert rel(Q[b]) <= max(1e-5, 4 * rel(Q32)), (b, rel(Q[b]), rel(Q32))
+
+
+@pytest.mark.parametrize("n,batch,kind", [
+    (380, 1, "steady"), (384, 2, "steady"), (388, 2, "steady"), (512, 1, "mixed"), (516, 3, "steady"),
+    (768, 2, "zero_blocks"), (1020, 1, "steady"), (1024, 1, "steady"), (1028, 2, "mixed"), (1540, 1, "steady")])
+def test_superblocks_match_oracle(cuda, n, batch, kind):
+    """Around the widths (384 columns, 512 from n = 1024) at which the accumulation of Q goes on to
+    another superblock, with a last one of several blocks, of one, and of 4 columns."""
+    test_block_factorisation_matches_oracle(cuda, n, batch, kind)
