@@ -153,8 +153,9 @@ def measured_peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}, "fallback"
 
 
-# tensor-core fp32 products take 4 tf32 MMAs (hi/lo split of both operands)
-TC_PRODUCTS = 4
+# a tensor-core fp32 product takes six bf16 MMAs (three planes of both operands), the time of three
+# tf32 ones at the bf16 rate's half (the QR's block updates take four tf32 MMAs, hi/lo split)
+TC_PRODUCTS = 3
 # TF32 dense matmul throughput of the GB300s, measured with `python bench.py --peaks`
 # (torch.matmul 8192^3 with TF32 allowed: best of 10, and back to back for 4 s); the summary is
 # profiles/peaks_gb300.md. The driver's MEASURED_PEAKS.json has the bf16 and HBM figures only.
@@ -162,10 +163,9 @@ TF32_TFLOPS = {"burst": 1047.2, "sustained": 951.8}
 
 # DRAM bytes (ncu dram__bytes_read.sum + dram__bytes_write.sum) per algorithmic byte, from one
 # full capture of each family's representative launch (profiles/): the QR's K = 128 trailing
-# update of an 8192 factor (0.89) and the power step of an 8192 factor, whose operand panels are
-# re-read across tiles (5.1). Applied to a family's average algorithmic bytes per launch, the
+# update of an 8192 factor (0.89). Applied to a family's average algorithmic bytes per launch, the
 # mixed launches of a family make it an estimate; the other families have no current capture.
-TRAFFIC_PER_ALGORITHMIC_BYTE = {"qr_update": 0.89, "gemm_tc": 5.12}
+TRAFFIC_PER_ALGORITHMIC_BYTE = {"qr_update": 0.89}
 
 
 def roofline(family, st, peaks, peak_src, products=None, dtype_ratio=2.0):
@@ -183,13 +183,13 @@ def roofline(family, st, peaks, peak_src, products=None, dtype_ratio=2.0):
                     frac=ach / FP32_SIMT_PEAK_TFLOPS,
                     peak_source="fp32 FMA peak of the CUDA cores, 152 SMs x 128 lanes x 2 x 2.07 GHz")
     # the kernels run inside a long step: the sustained tensor peak. fp32 products take
-    # TC_PRODUCTS tf32 MMAs at the measured TF32 rate; bf16 products (Muon) one MMA at the
+    # the time of TC_PRODUCTS tf32 MMAs at the measured TF32 rate; bf16 products (Muon) one MMA at the
     # measured bf16 rate
     products = TC_PRODUCTS if products is None else products
     if products > 1:
         tc_peak = TF32_TFLOPS["sustained"] / products
         tc_src = f"measured sustained tf32 dense ({TF32_TFLOPS['sustained']} TFLOP/s, bench.py --peaks) / {products}" \
-                 " (tf32 products per fp32 product)"
+                 " (an fp32 product as six bf16 products, the time of three tf32)"
     else:
         tc_peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
         tc_src = f"{peak_src} sustained bf16 dense"
@@ -626,7 +626,7 @@ def run_soap(args):
     launches = sum(v["launches"] for v in fams.values())
     roof = roofline(top, st, peaks, peak_src, products=1 if muon else TC_PRODUCTS, dtype_ratio=1.0 if muon else 2.0)
     if muon:
-        # the DRAM/algorithmic ratios above were measured for the fp32 (tf32 x4) kernels
+        # the DRAM/algorithmic ratios above were measured for the fp32 kernels
         roof["traffic"], roof["traffic_note"] = None, "not measured for the bf16 kernel"
     if iso and iso.get(top, {}).get("launches"):
         r = roofline(top, iso[top], peaks, peak_src)

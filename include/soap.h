@@ -104,7 +104,7 @@ soap_status_t soap_create(const soap_shape* shapes, int32_t n, const soap_hparam
 /* soap_create with a bound on the workspace. Besides the optimizer state proper (per matrix
  * M_hat and v, the factors L and R stored as their lower-triangular 32 x 32 tiles, the bases
  * Q_L and Q_R), a step needs a workspace for the operands it forms (the gradient copy and its
- * transpose, tf32 lo parts, Q^T, the unpacked factors, the QR's buffers, the rotation
+ * transpose, Q and Q^T as bf16 planes, the unpacked factors, the QR's buffers, the rotation
  * intermediates). Matrices are stepped in waves: runs of matrices whose workspace fits side by
  * side, the next wave reusing it. workspace_limit = 0 (what soap_create does) takes one wave
  * holding every matrix if that leaves 1 GiB + 1% of the device's memory free, else waves cut
@@ -197,8 +197,8 @@ void soap_destroy(soap_handle h);
 /* Kernel families the library launches. */
 typedef enum {
   SOAP_KERNEL_GEMM_SIMT = 0,   /* CUDA-core fp32 batched GEMM */
-  SOAP_KERNEL_GEMM_TC = 1,     /* tcgen05 batched GEMM: fp32-accurate (four TF32 products), or bf16 (Muon) */
-  SOAP_KERNEL_QR_PANEL = 2,    /* cluster panel factorisation of the QR */
+  SOAP_KERNEL_GEMM_TC = 1,     /* tcgen05 batched GEMM: fp32-accurate (six bf16 products, or four TF32), or bf16 (Muon) */
+  SOAP_KERNEL_QR_PANEL = 2,    /* factorisation of the QR's 128-column blocks */
   SOAP_KERNEL_ELEMENTWISE = 3, /* momentum, Adam, weight update */
   SOAP_KERNEL_OTHER = 4,       /* norms, identity fills */
   SOAP_KERNEL_QR_UPDATE = 5    /* tensor-core products of the QR's block updates */

@@ -1,4 +1,7 @@
-// fp32-accurate batched GEMM on the 5th-generation tensor cores (tcgen05, sm_103a).
+// fp32-accurate batched GEMM on the 5th-generation tensor cores (tcgen05, sm_103a), four TF32
+// products on 128 x 128 tiles: soap_gemm_tf32x4 and the QR's block products, whose operands change
+// from block to block and whose K of 128 leaves the bf16 planes' extra conversions unpaid (converted
+// in the kernel, the K = 128 update of 16 x 2048^2 took 176 us against 162, W 217 against 156).
 //
 //   C_b = alpha * A_b * B_{b mod bmod}^T + beta * C_b
 //

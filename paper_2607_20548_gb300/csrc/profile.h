@@ -14,8 +14,8 @@ namespace soap {
 
 enum KernelFamily : int {
   kFamGemmSimt = 0,   // CUDA-core fp32 GEMM
-  kFamGemmTc = 1,     // tcgen05 GEMM: fp32 as four TF32 products, or bf16 (Muon)
-  kFamQrPanel = 2,    // cluster panel factorisation of the QR
+  kFamGemmTc = 1,     // tcgen05 GEMM: fp32 as six bf16 products (or four TF32), or bf16 (Muon)
+  kFamQrPanel = 2,    // factorisation of the QR's 128-column blocks
   kFamElementwise = 3,// momentum / Adam / weight update
   kFamOther = 4,      // norms, identity fills
   kFamQrUpdate = 5,   // tensor-core products of the QR's block updates (at the roofline ridge)

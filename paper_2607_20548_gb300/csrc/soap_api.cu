@@ -48,7 +48,7 @@ struct ClassState {
   int count = 0;
   std::vector<int> members;
   size_t ptr_offset = 0;  // index of this class's params pointers in the pointer table
-  // tensor-core path (both dimensions multiples of 4): operand copies with lo parts in the
+  // tensor-core path (both dimensions multiples of 4): operands as bf16 planes in the
   // workspace, factors packed; otherwise CUDA cores with full factors
   bool tc = false;
   // working orientation transposed: a class preconditioned on its left only runs as the
@@ -443,7 +443,7 @@ soap_status_t accumulate_factors(soap_handle h, const ClassState& c, const View&
 
 // S2 + S3 for the preconditioned sides of one size group of a wave: P^T = Q^T F for each member
 // (F the unpacked factor, symmetric) into one batched input, one QR, then Q (into the state),
-// Q^T and the lo parts (into the slices' workspace) and the zero-column flags. The group runs
+// the planes of Q and Q^T (into the slices' workspace) and the zero-column flags. The group runs
 // on its own streams from the moment its members' factors are updated on the caller's stream,
 // concurrently with other groups.
 soap_status_t refresh_group(soap_handle h, const Wave& w, const QrGroup& g, cudaStream_t s) {
