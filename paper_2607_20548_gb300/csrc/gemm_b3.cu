@@ -106,7 +106,6 @@ __device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, u
 __device__ __forceinline__ int swz(int r, int j) { return r * 32 + ((((j >> 2) ^ (r & 7))) << 2) + (j & 3); }
 // The same for a 32 x 16 block (two rows to a 128-byte line), element (r, 4 q).
 __device__ __forceinline__ int swzh(int r, int q) { return r * 16 + ((q ^ ((r >> 1) & 3)) << 2); }
-__device__ __forceinline__ int swz16(int r, int q) { return (r >> 3) * 1024 + (r & 7) * 128 + ((q ^ (r & 7)) << 4); }
 
 // Tile t of a launch -> (m0, n0, batch index). Within a matrix the tiles go in groups of GM row
 // tiles, m fastest, so that the tiles in flight at a time share their row and column panels in L2.
@@ -163,8 +162,9 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t* acc_empty = acc_full + NACC;
   uint64_t* mma_done = acc_empty + NACC;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(mma_done + 1);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-  volatile int* consumed = abort_flag + 1;
+  tc::RingState* ring = reinterpret_cast<tc::RingState*>(tmem_holder + 1);  // [2]: this CTA's, the peer's
+  volatile int* abort_flag = &ring->abort;
+  volatile int* consumed = &ring->consumed;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = CG == 1 ? 0 : (int)(blockIdx.x & 1);
@@ -192,8 +192,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       tc::mbar_init(&acc_empty[a], EPI * CG);  // one arrival per epilogue warp
     }
     tc::mbar_init(mma_done, 1);
-    *abort_flag = 0;
-    *consumed = 0;
+    *ring = tc::RingState{};
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0 && lane == 0) {
@@ -240,11 +239,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           issued = g + 1;
         }
       }
-      if (*abort_flag && lead) {
-        // let copies already in flight land before the CTAs' shared memory goes away (the second
-        // CTA's copies count on this CTA's barriers too, and it waits at the last cluster barrier)
-        for (int gg = *consumed; gg < issued; ++gg) tc::wait<CG>(&full[gg % STAGES], (gg / STAGES) & 1, kWaitNs);
-      }
+      ring->issued = issued;
     }
   } else if (warp == 1) {
     if (lane == 0 && lead) {
@@ -283,6 +278,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           tc::commit<CG>(&acc_full[a]);  // hands the K block's sum to the epilogue warps
         }
       }
+      ring->accs = g;
       if (!ok) {
         *abort_flag = 1;
         if (ep.status) atomicOr(ep.status, kStatusTimeout);
@@ -464,12 +460,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   }
 
-  tc::tc_fence_before();
-  __syncthreads();
-  if (CG == 2) {  // the peer's arrivals and copies into this CTA's shared memory are over
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  }
+  tc::finish<CG, STAGES, NACC>(full, empty, acc_full, mma_done, ring, lead, C::STAGE, kWaitNs);
   if (warp == 1) {
     tc::tc_fence_after();
     if (CG == 1)

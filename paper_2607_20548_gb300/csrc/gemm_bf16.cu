@@ -115,8 +115,9 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t* acc_empty = acc_full + NACC;
   uint64_t* mma_done = acc_empty + NACC;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(mma_done + 1);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-  volatile int* consumed = abort_flag + 1;
+  tc::RingState* ring = reinterpret_cast<tc::RingState*>(tmem_holder + 1);  // [2]: this CTA's, the peer's
+  volatile int* abort_flag = &ring->abort;
+  volatile int* consumed = &ring->consumed;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = CG == 1 ? 0 : (int)(blockIdx.x & 1);
@@ -136,8 +137,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       tc::mbar_init(&acc_empty[a], EPI * CG);
     }
     tc::mbar_init(mma_done, 1);
-    *abort_flag = 0;
-    *consumed = 0;
+    *ring = tc::RingState{};
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0 && lane == 0) {
@@ -183,10 +183,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           issued = g + 1;
         }
       }
-      if (*abort_flag && lead) {
-        // let copies already in flight land before the CTAs' shared memory goes away
-        for (int gg = *consumed; gg < issued; ++gg) tc::wait<CG>(&full[gg % STAGES], (gg / STAGES) & 1, kWaitNs);
-      }
+      ring->issued = issued;
     }
   } else if (warp == 1) {
     if (lane == 0 && lead) {
@@ -215,7 +212,10 @@ __global__ void __launch_bounds__(THREADS, 1)
             tc::umma_f16<CG>(d, a_s + kk * 32, b_s + kk * 32, idesc, (kb | kk) != 0);
           tc::commit<CG>(&empty[s]);  // frees the stage once these MMAs have read it
         }
-        if (ok) tc::commit<CG>(&acc_full[a]);  // hands the tile's sum to the epilogue warps
+        if (ok) {
+          tc::commit<CG>(&acc_full[a]);  // hands the tile's sum to the epilogue warps
+          ring->accs = tl + 1;
+        }
       }
       if (!ok) *abort_flag = 1;
       if (g > 0) {  // every MMA issued has completed before the tensor memory is freed
@@ -302,12 +302,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   }
 
-  tc::tc_fence_before();
-  __syncthreads();
-  if (CG == 2) {  // the peer's arrivals and copies into this CTA's shared memory are over
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  }
+  tc::finish<CG, STAGES, NACC>(full, empty, acc_full, mma_done, ring, lead, C::STAGE, kWaitNs);
   if (warp == 1) {
     tc::tc_fence_after();
     if (CG == 1)

@@ -193,6 +193,71 @@ __device__ __forceinline__ void commit(uint64_t* bar) {
         : "memory");
 }
 
+// What the warps of a CTA that feed a pair's (or a CTA's) MMAs leave behind for finish(), in shared memory.
+struct RingState {
+  int abort;     // a wait gave up
+  int consumed;  // K blocks whose MMAs were issued (kept by the pair's first CTA)
+  int accs;      // accumulators handed to the epilogue warps (likewise)
+  int issued;    // K blocks whose copies this CTA issued
+};
+
+// The last thing every thread of a tile kernel does before its tensor memory is freed and its CTA
+// exits: nothing may then still arrive in the shared memory of either CTA. That is,
+//  * the commits' arrivals, which go to both CTAs on their own: each CTA waits for its own copies;
+//  * the arrivals of the epilogue warps, performed before the cluster barrier;
+//  * after a wait that gave up, copies in flight. Both CTAs' copies of a K block count on the first
+//    CTA's barrier, and one producer may have gone a block further than the other: the CTAs tell each
+//    other how far they got, the first one makes up the count of the halves that were never issued, or
+//    not expected, and the pair leaves together.
+// st[0] is this CTA's state, st[1] takes the peer's; every wait is bounded.
+template <int CG, int STAGES, int NACC>
+__device__ __forceinline__ void finish(uint64_t* full, uint64_t* empty, uint64_t* acc_full, uint64_t* mma_done,
+                                       RingState* st_, bool lead, uint32_t stage_bytes, uint64_t limit_ns) {
+  volatile RingState* st = st_;
+  tc_fence_before();
+  __syncthreads();
+  if (CG == 2) {
+    if (threadIdx.x < sizeof(RingState) / 4) {
+      const uint32_t dst = smem_u32(st_ + 1) + 4 * threadIdx.x;
+      const int v = reinterpret_cast<volatile int*>(st_)[threadIdx.x];
+      asm volatile(
+          "{\n\t.reg .b32 a;\n\t"
+          "mapa.shared::cluster.u32 a, %0, %1;\n\t"
+          "st.shared::cluster.b32 [a], %2;\n\t}\n" ::"r"(dst),
+          "r"(lead ? 1 : 0), "r"(v)
+          : "memory");
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+  if (threadIdx.x == 0) {
+    const int first = CG == 1 || lead ? 0 : 1;  // the first CTA's entry
+    const int consumed = st[first].consumed, accs = st[first].accs;
+    for (int g = consumed > STAGES ? consumed - STAGES : 0; g < consumed; ++g)
+      wait<CG>(&empty[g % STAGES], (g / STAGES) & 1, limit_ns);
+    for (int g = accs > NACC ? accs - NACC : 0; g < accs; ++g)
+      wait<CG>(&acc_full[g % NACC], (g / NACC) & 1, limit_ns);
+    if (consumed > 0) wait<CG>(mma_done, 0, limit_ns);
+    if (lead) {
+      const int mine = st[0].issued, theirs = CG == 2 ? st[1].issued : mine;
+      for (int g = consumed; g < mine || g < theirs; ++g) {
+        uint64_t* bar = &full[g % STAGES];
+        if (g >= mine) mbar_expect_tx(bar, stage_bytes);
+        if (g >= theirs)
+          asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(stage_bytes)
+                       : "memory");
+        wait<CG>(bar, (g / STAGES) & 1, limit_ns);
+      }
+    }
+  }
+  __syncwarp();
+  if (CG == 2 && (st[0].abort | st[1].abort)) {  // the same for all threads of both CTAs
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+}
+
 // tf32 value the tensor core reads from an fp32 word (13 low mantissa bits dropped), and
 // the lo part x - trunc(x) rounded to the nearest tf32 (so the tensor core reads it exactly).
 __device__ __forceinline__ float tf32_trunc(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
