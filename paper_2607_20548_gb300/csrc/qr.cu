@@ -85,7 +85,8 @@ struct PanelArgs {
   float* T_lo;
   float* Tt;           // [batch][NBO][NBO] T^T
   float* Tt_lo;
-  float* Ypart;        // [batch][MAXC][NBO][NB] per-CTA partial products S V_panel
+  float* Ypart;        // [batch][MAXC][NBO][NB] per-CTA partial products S V_panel (at first the
+                       // Gram matrices' place, which qr_block_left reads before any is written)
   uint8_t* skip;       // [batch][n]
   float* dsign;        // [batch][n] sign of R_pp (+1 for zero columns)
   const float* thresh; // [batch]
@@ -121,7 +122,7 @@ __global__ void __launch_bounds__(PT, 1) qr_panel_kernel(PanelArgs p) {
   const int C = (int)cluster.num_blocks();
   const int b = blockIdx.y;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (p.state[b] != kQrBlockColumns) return;  // factored without the column loop
+  if (!qr_block_left(p.state[b], p.Ypart, b, p.kbo)) return;  // factored without the column loop
 
   extern __shared__ float4 smem_dyn[];
   float* sA = reinterpret_cast<float*>(smem_dyn);  // [NB][LDS]: panel row jj, position offset i

@@ -15,22 +15,26 @@
 // are exactly the Householder vectors and the triangular factor of H_1 ... H_kbo = I - V T V^T
 // with the reflector convention of the column loop (R_jj of the reflectors is D_j R_jj; the
 // reconstruction of Householder vectors from an explicit Q, Ballard et al., "Reconstructing
-// Householder vectors from tall-skinny QR", applied to Q = A R^-1). In 32-bit arithmetic the
-// squared pivots of the Cholesky factor carry an absolute error of a few 2^-24 G_jj, so a pivot
-// is as accurate as Householder's only where column j keeps a good part of its norm after the
-// block's earlier columns are projected out. The block is therefore taken this way only if every
-// squared pivot is at least kRhoMin of its column's squared norm and every pivot is clear of the
-// zero-column threshold; a block whose columns are all below that threshold is skipped outright
-// (no reflectors); any other block is left to the column loop (qr_panel_kernel), which the state
-// word per matrix tells to run. In the steady state of a run P = F Q has nearly orthogonal
-// columns (the squared pivots are 0.9 and more of the squared norms); rank-deficient factors of
-// the first steps take the column loop.
+// Householder vectors from tall-skinny QR", applied to Q = A R^-1). In 32-bit arithmetic G carries
+// an error E of about 2^-24 in units of its column norms, and Q then misses orthogonality by
+// R^-T E R^-1: by E times the norm of the inverse of G^ = G scaled to a unit diagonal. The pivots do
+// not bound that norm (with every squared pivot at 0.4 of its column's squared norm it can exceed
+// 1e10). Its trace does: the eigenvalues of G^ add up to kbo, so that
+//   ||G^^-1|| <= tr(G^^-1) - kbo + 2,   tr(G^^-1) = sum_i G_ii ||row i of R^-1||^2,
+// and the kernel that forms T's rows solves for R^-1's beside them. The block is taken this way only
+// if the excess tr(G^^-1) - kbo is at most kQrMaxExcess and every pivot is clear of the zero-column
+// threshold; a block whose columns are all below that threshold is skipped outright (no reflectors);
+// any other block is left to the column loop: qr_panel_kernel asks qr_block_left, and writes
+// everything that a block factored here leaves behind. In the steady state of a run P = F Q has nearly
+// orthogonal columns (an excess of 0.1-6); blocks of its first steps (up to 250) and of rank-deficient
+// factors take the column loop.
 //
 //   qr_gram_kernel  G in up to 4 partial sums: tcgen05 products of 128 x 32 chunks, cluster
 //                   reduction through distributed shared memory
 //   qr_core_kernel  one CTA per matrix: Cholesky and elimination in one loop over the columns,
 //                   W^-1 formed in place in the finished columns (Gauss-Jordan)
-//   qr_form_kernel  V2 = -A2 W^-1 in tiles of 128 positions (tcgen05), and T's rows
+//   qr_form_kernel  V2 = -A2 W^-1 in tiles of 128 positions (tcgen05), T's rows, and the squares of
+//                   R^-1's
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -48,10 +52,8 @@ namespace {
 
 constexpr int NBO = kQrBlock;
 constexpr uint64_t kWaitNs = 2000000000ull;
-// Squared pivot over squared column norm below which a block goes to the column loop: at 0.25 the
-// pivots' error is 4 times Gram's, and the bases' error against 64 bits stays below the column
-// loop's (simulated in 32 bits over steady and early factors: 0.6-0.8e-6 against 0.9e-6; at 0.12,
-// 1.3e-6).
+// Squared pivot over squared column norm below which a block leaves for the column loop at once (its
+// excess is at least 3 then; blocks of a run that the excess admits have 0.5 and more).
 constexpr float kRhoMin = 0.25f;
 
 // byte offset of 16-byte unit q of row r in a tile of 128-byte rows, swizzled within 1024-byte
@@ -83,6 +85,12 @@ __device__ __forceinline__ void mma_chunk(uint32_t d, uint32_t a_hi, uint32_t a_
 // the matrix's first partial Gram matrix, which only the CTA that writes M reads.
 __device__ __forceinline__ float* block_m(const QrBlockArgs& p, int b) {
   return p.Gpart + (int64_t)b * kQrGramParts * NBO * NBO;
+}
+
+// What qr_block_left reads and the core kernel hands it, in place of the second partial Gram matrix:
+// the trace of G^^-1 by rows of a CTA of the form kernel, then G's diagonal.
+__device__ __forceinline__ float* block_trace(const QrBlockArgs& p, int b) {
+  return p.Gpart + ((int64_t)b * kQrGramParts + 1) * NBO * NBO;
 }
 
 constexpr int kThreads = 256;
@@ -617,6 +625,7 @@ __global__ void __launch_bounds__(kThreads, 1) qr_core_kernel(QrBlockArgs p, int
     }
   }
   if (tid == 0) p.state[b] = zero ? kQrBlockZero : fast ? kQrBlockFast : kQrBlockColumns;
+  if (tid < NBO) block_trace(p, b)[kQrTraceParts + tid] = sh.norm[tid];
   if (tid < kbo && (zero || fast)) {
     p.skip[(int64_t)b * n + k0 + tid] = zero ? 1 : 0;
     if (zero) p.dsign[(int64_t)b * n + k0 + tid] = 1.f;
@@ -625,10 +634,11 @@ __global__ void __launch_bounds__(kThreads, 1) qr_core_kernel(QrBlockArgs p, int
 
 // Blocks 0 .. kTBlocks-1 of a matrix: 16 rows of T each (two per warp), by the row solves
 // u (D R) = W_i and t V1^T = u (lane l holds columns 4 l .. 4 l + 3; each finished entry is
-// broadcast once), and 16 rows of V1, to Vt and to Vpos. The other blocks: V2 = -A2 W^-1 on 128
+// broadcast once), beside them x (D R) = e_i for the trace, and 16 rows of V1, to Vt and to Vpos. The
+// other blocks: V2 = -A2 W^-1 on 128
 // positions each, as tcgen05 products of 128 positions x 32 columns chunks; A's chunk is turned
 // position-major (with its lo part) in shared memory, each chunk has its own accumulator.
-constexpr int kTBlocks = 8;
+constexpr int kTBlocks = kQrTraceParts;
 constexpr int kFormLd = NBO + 4;
 constexpr int kFormSmem = NBO * kFormLd * 4 + 2 * 4 * kTile + 1024;
 constexpr int kSolveSmem = 2 * NBO * kFormLd * 4;
@@ -640,6 +650,7 @@ __device__ __forceinline__ void t_rows(const QrBlockArgs& p, int b, int rb, floa
   float* Rs = sm;                  // [128][132] D R, strictly upper
   float* Vs = sm + NBO * kFormLd;  // [128][132] V1^T, strictly upper
   __shared__ float s_inv[NBO];
+  __shared__ float s_trace[kThreads / 32];
   const float* Rb = p.Rf + (int64_t)b * n * NBO;
   const float* Wb = p.Wf + (int64_t)b * n * NBO;
   const float* M = block_m(p, b);
@@ -716,11 +727,14 @@ __device__ __forceinline__ void t_rows(const QrBlockArgs& p, int b, int rb, floa
   if (!zero) {
     // u_j = (u_j so far) / (D R)_jj, then t_j = u_j + (t_j so far): both solves advance together
     // (columns before a row's diagonal are zero and stay so)
-    float t[2][4];
+    float t[2][4], w[2][4], inv2[2] = {0.f, 0.f};  // w: e_i, then what is left of it; inv2: ||x||^2
 #pragma unroll
     for (int e = 0; e < 2; ++e)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) t[e][c] = 0.f;
+      for (int c = 0; c < 4; ++c) {
+        t[e][c] = 0.f;
+        w[e][c] = 4 * lane + c == i0 + e ? 1.f : 0.f;
+      }
 #pragma unroll 1
     for (int j4 = i0 >> 2; 4 * j4 < kbo; ++j4) {
 #pragma unroll
@@ -742,8 +756,18 @@ __device__ __forceinline__ void t_rows(const QrBlockArgs& p, int b, int rb, floa
           t[e][2] = fmaf(-y, v.z, t[e][2]);
           t[e][3] = fmaf(-y, v.w, t[e][3]);
           if (lane == j4) t[e][c] = y;
+          const float z = __shfl_sync(0xffffffffu, w[e][c], j4) * iv;
+          inv2[e] = fmaf(z, z, inv2[e]);
+          w[e][0] = fmaf(-z, r.x, w[e][0]);
+          w[e][1] = fmaf(-z, r.y, w[e][1]);
+          w[e][2] = fmaf(-z, r.z, w[e][2]);
+          w[e][3] = fmaf(-z, r.w, w[e][3]);
         }
       }
+    }
+    if (lane == 0) {
+      const float* norm = block_trace(p, b) + kQrTraceParts;
+      s_trace[warp] = (i0 < kbo ? inv2[0] * norm[i0] : 0.f) + (i0 + 1 < kbo ? inv2[1] * norm[i0 + 1] : 0.f);
     }
 #pragma unroll
     for (int e = 0; e < 2; ++e)
@@ -765,6 +789,11 @@ __device__ __forceinline__ void t_rows(const QrBlockArgs& p, int b, int rb, floa
 #pragma unroll
     for (int c = 0; c < 4; ++c) sm[(4 * lane + c) * 17 + 2 * warp + e] = u[e][c];
   __syncthreads();
+  if (tid == 0 && !zero) {
+    float x = 0.f;
+    for (int i = 0; i < kThreads / 32; ++i) x += s_trace[i];
+    block_trace(p, b)[rb] = x;
+  }
   for (int e = tid; e < NBO * 16; e += kThreads) {
     const int c = e >> 4, i = e & 15;
     const float t = sm[c * 17 + i];
