@@ -552,7 +552,7 @@ cudaError_t launch(int M, int N, int K, int batch, const B3Operand& A, const B3O
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = CG == 1 ? 0 : 1;
   return cudaLaunchKernelEx(&cfg, fn, ta, tb, p);
 }
 

@@ -203,19 +203,23 @@ struct RingState {
 
 // The last thing every thread of a tile kernel does before its tensor memory is freed and its CTA
 // exits: nothing may then still arrive in the shared memory of either CTA. That is,
-//  * the commits' arrivals, which go to both CTAs on their own: each CTA waits for its own copies;
+//  * the commits' arrivals, which go to both CTAs of a pair on their own: each waits for its own copies
+//    (a single CTA's epilogue has waited for the last of them);
 //  * the arrivals of the epilogue warps, performed before the cluster barrier;
 //  * after a wait that gave up, copies in flight. Both CTAs' copies of a K block count on the first
 //    CTA's barrier, and one producer may have gone a block further than the other: the CTAs tell each
 //    other how far they got, the first one makes up the count of the halves that were never issued, or
 //    not expected, and the pair leaves together.
-// st[0] is this CTA's state, st[1] takes the peer's; every wait is bounded.
+// st[0] is this CTA's state, st[1] takes the peer's; every wait is bounded. The waits of a warp's lanes
+// go side by side (in turn they cost a launch of few tiles up to a microsecond).
 template <int CG, int STAGES, int NACC>
 __device__ __forceinline__ void finish(uint64_t* full, uint64_t* empty, uint64_t* acc_full, uint64_t* mma_done,
                                        RingState* st_, bool lead, uint32_t stage_bytes, uint64_t limit_ns) {
+  static_assert(STAGES + NACC < 32, "a lane for every barrier");
   volatile RingState* st = st_;
   tc_fence_before();
   __syncthreads();
+  if (CG == 1 && !st[0].abort) return;
   if (CG == 2) {
     if (threadIdx.x < sizeof(RingState) / 4) {
       const uint32_t dst = smem_u32(st_ + 1) + 4 * threadIdx.x;
@@ -231,15 +235,19 @@ __device__ __forceinline__ void finish(uint64_t* full, uint64_t* empty, uint64_t
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {
     const int first = CG == 1 || lead ? 0 : 1;  // the first CTA's entry
-    const int consumed = st[first].consumed, accs = st[first].accs;
-    for (int g = consumed > STAGES ? consumed - STAGES : 0; g < consumed; ++g)
-      wait<CG>(&empty[g % STAGES], (g / STAGES) & 1, limit_ns);
-    for (int g = accs > NACC ? accs - NACC : 0; g < accs; ++g)
-      wait<CG>(&acc_full[g % NACC], (g / NACC) & 1, limit_ns);
-    if (consumed > 0) wait<CG>(mma_done, 0, limit_ns);
-    if (lead) {
+    const int consumed = st[first].consumed, accs = st[first].accs, l = (int)threadIdx.x;
+    if (l < STAGES) {
+      const int g = consumed - 1 - l;
+      if (g >= 0) wait<CG>(&empty[g % STAGES], (g / STAGES) & 1, limit_ns);
+    } else if (l < STAGES + NACC) {
+      const int g = accs - 1 - (l - STAGES);
+      if (g >= 0) wait<CG>(&acc_full[g % NACC], (g / NACC) & 1, limit_ns);
+    } else if (l == STAGES + NACC && consumed > 0) {
+      wait<CG>(mma_done, 0, limit_ns);
+    }
+    if (l == 0 && lead) {
       const int mine = st[0].issued, theirs = CG == 2 ? st[1].issued : mine;
       for (int g = consumed; g < mine || g < theirs; ++g) {
         uint64_t* bar = &full[g % STAGES];
@@ -250,8 +258,8 @@ __device__ __forceinline__ void finish(uint64_t* full, uint64_t* empty, uint64_t
         wait<CG>(bar, (g / STAGES) & 1, limit_ns);
       }
     }
+    __syncwarp();
   }
-  __syncwarp();
   if (CG == 2 && (st[0].abort | st[1].abort)) {  // the same for all threads of both CTAs
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
