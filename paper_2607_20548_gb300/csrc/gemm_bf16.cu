@@ -7,13 +7,15 @@
 // stored in bf16). A symmetric product (A = B, M = N) computes the tiles on or below the diagonal
 // only and stores each one below it in the mirror position too: two of the three products of an
 // iteration, X X^T and A A^T, at half the MMAs (the two halves' bits are the same: an element and
-// its mirror sum the same products in the same order).
+// its mirror sum the same products in the same order), where that saves more than the mirrored stores
+// cost.
 //
 // A pair of CTAs (cta_group::2) works on a 256 x 256 tile: with one CTA per 128 x 128 tile, shared
 // memory took 256 bytes of operand reads and refills per cycle of MMA time, twice what it sustains,
 // and the products ran at 0.46 of the sustained tensor peak. In the pair each CTA loads its own 128
-// rows of A and half of B's rows, and the same traffic feeds four times the MMAs. Products of at most
-// 128 rows or columns, and those too small to fill the SM pairs, keep one CTA per 128 x 128 tile.
+// rows of A and half of B's rows, and the same traffic feeds four times the MMAs. Small and ragged
+// products keep one CTA per 128 x 128 tile: which one is taken is decided on the estimated times at the
+// end of this file.
 //
 // Persistent clusters walk the output tiles in groups of row tiles. Warp 0 issues the TMA loads
 // of 64-element K slices (one 128-byte swizzle row per matrix row) into a ring, warp 1 of the
@@ -245,14 +247,26 @@ __global__ void __launch_bounds__(THREADS, 1)
       __nv_bfloat16* out_t = SYM ? (mirror ? ep.out + ob : nullptr)
                                  : (ep.out_t ? ep.out_t + (int64_t)b * ep.stride_t : nullptr);
       const int64_t ld_t = SYM ? ep.ld : ep.ld_t;
-#pragma unroll 1
+      // a single CTA's warp takes its 64 columns out of the accumulator at once; a pair's 128 go through
+      // the registers 32 at a time
+      constexpr int NV = CG == 1 ? C::NCH : 1;
+      float v[NV][32];
+      auto drained = [&] {
+        tc::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) tc::arrive_lead<CG>(&acc_empty[a]);
+      };
+      if (CG == 1) {
+#pragma unroll
+        for (int c = 0; c < NV; ++c) tc::tmem_ld32(lane_base + static_cast<uint32_t>(a * C::T + colbase + 32 * c), v[c]);
+        drained();
+      }
+#pragma unroll NV
       for (int c = 0; c < C::NCH; ++c) {
-        float o[32];
-        tc::tmem_ld32(lane_base + static_cast<uint32_t>(a * C::T + colbase + 32 * c), o);
-        if (c == C::NCH - 1) {  // the accumulator is drained
-          tc::tc_fence_before();
-          __syncwarp();
-          if (lane == 0) tc::arrive_lead<CG>(&acc_empty[a]);
+        float(&o)[32] = v[CG == 1 ? c : 0];
+        if (CG == 2) {
+          tc::tmem_ld32(lane_base + static_cast<uint32_t>(a * C::T + colbase + 32 * c), o);
+          if (c == C::NCH - 1) drained();
         }
         const int c0 = n0 + colbase + 32 * c;
         if (c0 >= N) continue;
@@ -286,7 +300,15 @@ __global__ void __launch_bounds__(THREADS, 1)
             if (c0 + 8 * u < N)
               *reinterpret_cast<uint4*>(dst + 8 * u) = make_uint4(w2[4 * u], w2[4 * u + 1], w2[4 * u + 2], w2[4 * u + 3]);
         }
-        if (out_t) {
+        if (CG == 1 && out_t) {
+          // for each column the warp's 32 rows are 32 consecutive elements
+          __nv_bfloat16* dst = out_t + (int64_t)c0 * ld_t + r;
+          const unsigned short* h = reinterpret_cast<const unsigned short*>(w2);
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (r < M && c0 + j < N) reinterpret_cast<unsigned short*>(dst)[(int64_t)j * ld_t] = h[j];
+        }
+        if (CG == 2 && out_t) {
           // two neighbouring rows of a column make a 4-byte word: even lanes take the even columns,
           // odd lanes the odd ones (M is a multiple of 8, so the rows of a pair are both in or out)
           const bool odd = lane & 1;
@@ -347,6 +369,27 @@ int64_t tile_count(int M, int N, int batch, int t, bool sym) {
   return (sym ? tm * (tm + 1) / 2 : tm * tn) * batch;
 }
 
+// Which kernel: one CTA or a pair per tile, and for a symmetric product all tiles or the lower ones
+// mirrored. The smallest estimate of  launch + waves * (K slices * slice + epilogue)  in us, the
+// coefficients fitted to 2800 products (sides 64 ... 3072, K 64 ... 8192, batches of 1 ... 64, each
+// timed in every form): the form taken is 0.5 % slower than the fastest on average. A pair's slice is
+// as long as a single CTA's and does four times the work, but its 128 x 256 values per CTA take the
+// epilogue's 8 warps two to three times as long, and partly empty tiles take whole ones' time. (Counting
+// waves alone sent short and ragged products to pairs and halves: 64 of 200 x 800, 16 steps, 1.39 ms;
+// 1.22 with all products whole on single CTAs.)
+enum Kind { kSingles, kLowerSingles, kPairs, kLowerPairs };
+Kind choose(int M, int N, int K, int batch, int sms, bool symmetric) {
+  const int slices = (K + BK - 1) / BK;
+  auto us = [&](int cg, bool lower, double launch, double slice, double epilogue) {
+    const int64_t slots = std::max(1, sms / cg), waves = (tile_count(M, N, batch, cg * BM, lower) + slots - 1) / slots;
+    return launch + waves * (slices * slice + epilogue);
+  };
+  if (!symmetric) return M > BM && N > BM && us(2, false, 6.4, 0.24, 9.9) < us(1, false, 4.3, 0.27, 3.5) ? kPairs : kSingles;
+  const double whole = us(1, false, 4.4, 0.26, 1.6), lower = us(1, true, 4.0, 0.30, 1.9);
+  if (M > BM && us(2, true, 5.9, 0.33, 4.0) < std::min(whole, lower)) return kLowerPairs;
+  return lower < whole ? kLowerSingles : kSingles;
+}
+
 template <int CG, bool SYM>
 cudaError_t launch(const CUtensorMap& ta, const CUtensorMap& tb, int M, int N, int K, int batch, const Bf16Epilogue& ep,
                    int dev, int sms, cudaStream_t s) {
@@ -372,7 +415,7 @@ cudaError_t launch(const CUtensorMap& ta, const CUtensorMap& tb, int M, int N, i
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = CG == 1 ? 0 : 1;  // (a launch with a cluster of one takes up to 0.3 us longer)
   return cudaLaunchKernelEx(&cfg, fn, ta, tb, M, N, K, batch, ep);
 }
 
@@ -386,28 +429,26 @@ cudaError_t gemm_bf16_nt(int M, int N, int K, int batch, const __nv_bfloat16* A,
   if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
   if (K <= 0 || batch > 65535 || (M & 7) || (N & 7) || (K & 7) || !ep.out) return cudaErrorInvalidValue;
   if ((ep.ld & 7) || (ep.stride & 7) || (ep.out_t && ((ep.ld_t & 1) || (ep.stride_t & 1)))) return cudaErrorInvalidValue;
-  // A A^T (and beta times a symmetric matrix): the lower tiles only, mirrored
-  const bool sym = A == B && M == N && lda == ldb && a_stride == b_stride && !ep.out_t && ep.symmetric;
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const bool symmetric = A == B && M == N && lda == ldb && a_stride == b_stride && !ep.out_t && ep.symmetric;
+  const Kind kind = choose(M, N, K, batch, sms, symmetric);
+  const bool sym = kind == kLowerSingles || kind == kLowerPairs;
   const double mn = (double)M * N * batch;
   ProfScope prof(kFamGemmTc, 2.0 * mn * K * (sym ? 0.5 : 1.0),
-                 2.0 * ((double)M * K + (sym ? 0.0 : (double)N * K)) * batch +
+                 2.0 * ((double)M * K + (symmetric ? 0.0 : (double)N * K)) * batch +
                      mn * (2 + (ep.out_t ? 2 : 0) + (ep.beta != 0.f && ep.cin ? 2 : 0)),
                  s);
   CUtensorMap ta, tb;
   if (!make_map(&ta, A, M, K, lda, a_stride, batch) || !make_map(&tb, B, N, K, ldb, b_stride, batch))
     return cudaErrorInvalidValue;
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // waves of single CTAs and of pairs: a K slice of a single CTA's 128 x 128 tile takes about as long
-  // (bound by shared memory) as one of a pair's 256 x 256
-  const int64_t w1 = (tile_count(M, N, batch, BM, sym) + sms - 1) / sms;
-  const int64_t w2 = (tile_count(M, N, batch, 2 * BM, sym) + sms / 2 - 1) / std::max(1, sms / 2);
-  if (M <= BM || N <= BM || w1 <= w2)
-    return sym ? launch<1, true>(ta, tb, M, N, K, batch, ep, dev, sms, s)
-               : launch<1, false>(ta, tb, M, N, K, batch, ep, dev, sms, s);
-  return sym ? launch<2, true>(ta, tb, M, N, K, batch, ep, dev, sms, s)
-             : launch<2, false>(ta, tb, M, N, K, batch, ep, dev, sms, s);
+  switch (kind) {
+    case kSingles: return launch<1, false>(ta, tb, M, N, K, batch, ep, dev, sms, s);
+    case kLowerSingles: return launch<1, true>(ta, tb, M, N, K, batch, ep, dev, sms, s);
+    case kPairs: return launch<2, false>(ta, tb, M, N, K, batch, ep, dev, sms, s);
+    default: return launch<2, true>(ta, tb, M, N, K, batch, ep, dev, sms, s);
+  }
 }
 
 }  // namespace soap
