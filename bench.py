@@ -153,13 +153,17 @@ def measured_peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}, "fallback"
 
 
-# a tensor-core fp32 product takes six bf16 MMAs (three planes of both operands), the time of three
-# tf32 ones at the bf16 rate's half (the QR's block updates take four tf32 MMAs, hi/lo split)
-TC_PRODUCTS = 3
 # TF32 dense matmul throughput of the GB300s, measured with `python bench.py --peaks`
 # (torch.matmul 8192^3 with TF32 allowed: best of 10, and back to back for 4 s); the summary is
 # profiles/peaks_gb300.md. The driver's MEASURED_PEAKS.json has the bf16 and HBM figures only.
 TF32_TFLOPS = {"burst": 1047.2, "sustained": 951.8}
+# A tensor-core fp32 product takes six bf16 MMAs (three planes of both operands): under the power cap the
+# time of 3.3 tf32 ones at the rates measured here (bf16 1728 TFLOP/s sustained), which puts its peak at
+# 1728 / 6 = 288 TFLOP/s. (A product in isolation runs at burst clocks: 1907.4 / 6 = 318.) The QR's block
+# updates, most of their family, take four tf32 MMAs (hi/lo split): 951.8 / 4 = 238.
+BF16_SUSTAINED_TFLOPS = 1728.0
+TC_PRODUCTS = 6 * TF32_TFLOPS["sustained"] / BF16_SUSTAINED_TFLOPS
+FAMILY_PRODUCTS = {"gemm_tc": TC_PRODUCTS, "qr_update": 4}
 
 # DRAM bytes (ncu dram__bytes_read.sum + dram__bytes_write.sum) per algorithmic byte, from one
 # full capture of each family's representative launch (profiles/): the QR's K = 128 trailing
@@ -168,7 +172,7 @@ TF32_TFLOPS = {"burst": 1047.2, "sustained": 951.8}
 TRAFFIC_PER_ALGORITHMIC_BYTE = {"qr_update": 0.89}
 
 
-def roofline(family, st, peaks, peak_src, products=None, dtype_ratio=2.0):
+def roofline(family, st, peaks, peak_src, products=None):
     """Roofline of one kernel family from its CUDA-event time and algorithmic FLOPs/bytes."""
     secs = st["ms"] / 1e3
     ratio = TRAFFIC_PER_ALGORITHMIC_BYTE.get(family)
@@ -182,14 +186,14 @@ def roofline(family, st, peaks, peak_src, products=None, dtype_ratio=2.0):
         return dict(base, bound="alu", achieved=ach, peak=FP32_SIMT_PEAK_TFLOPS, unit="TFLOP/s",
                     frac=ach / FP32_SIMT_PEAK_TFLOPS,
                     peak_source="fp32 FMA peak of the CUDA cores, 152 SMs x 128 lanes x 2 x 2.07 GHz")
-    # the kernels run inside a long step: the sustained tensor peak. fp32 products take
-    # the time of TC_PRODUCTS tf32 MMAs at the measured TF32 rate; bf16 products (Muon) one MMA at the
-    # driver-measured bf16 rate
-    products = TC_PRODUCTS if products is None else products
+    # the kernels run inside a long step: the sustained tensor peak. fp32 products take the time of
+    # FAMILY_PRODUCTS tf32 MMAs at the measured TF32 rate; bf16 products (Muon) one MMA at the
+    # measured bf16 rate
+    products = FAMILY_PRODUCTS.get(family, TC_PRODUCTS) if products is None else products
     if products > 1:
         tc_peak = TF32_TFLOPS["sustained"] / products
-        tc_src = f"measured sustained tf32 dense ({TF32_TFLOPS['sustained']} TFLOP/s, bench.py --peaks) / {products}" \
-                 " (an fp32 product as six bf16 products, the time of three tf32)"
+        tc_src = f"measured sustained tf32 dense ({TF32_TFLOPS['sustained']} TFLOP/s, bench.py --peaks) / 4" \
+            if products == 4 else f"measured sustained bf16 dense ({BF16_SUSTAINED_TFLOPS} TFLOP/s) / 6"
     else:
         tc_peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
         tc_src = f"{peak_src} sustained bf16 dense"
@@ -624,12 +628,12 @@ def run_soap(args):
     top = max(fams, key=lambda k: fams[k]["ms"])
     st = fams[top]
     launches = sum(v["launches"] for v in fams.values())
-    roof = roofline(top, st, peaks, peak_src, products=1 if muon else TC_PRODUCTS, dtype_ratio=1.0 if muon else 2.0)
+    roof = roofline(top, st, peaks, peak_src, products=1 if muon else None)
     if muon:
         # the DRAM/algorithmic ratios above were measured for the fp32 kernels
         roof["traffic"], roof["traffic_note"] = None, "not measured for the bf16 kernel"
     if iso and iso.get(top, {}).get("launches"):
-        r = roofline(top, iso[top], peaks, peak_src)
+        r = roofline(top, iso[top], peaks, peak_src, products=1 if muon else None)
         roof["isolated"] = {k: r[k] for k in ("bound", "achieved", "peak", "unit", "frac", "avg_launch_us")}
         roof["isolated"]["note"] = ("one further step with each launch timed alone (the device idle when it starts): "
                                     "the kernel's own rate; the figures above are live, beside the concurrent "
