@@ -110,20 +110,18 @@ __device__ __forceinline__ void mma_tf32_16x8x8(float (&d)[4], const uint32_t (&
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// The block's 32-column panels one after another, each spread over the cluster: CTA c holds
-// positions k + c*COLS .. of the panel rows in shared memory (row stride LDS, 16-byte aligned
-// rows). One launch per block, so that a block factored from its Gram matrix costs one launch that
-// returns at once (four, or eight with the column loop as a kernel of its own, cost 14-20 us).
+// One 32-column panel of a block, spread over the cluster: CTA c holds positions k + c*COLS .. of the
+// panel rows in shared memory (row stride LDS, 16-byte aligned rows). A function of its own, so that
+// the loop over the panels takes no registers from it (inlined, with 128 registers and spills, four
+// panels of a 2048-factor took 486 us instead of 441).
 template <int COLS>
-__global__ void __launch_bounds__(PT, 1) qr_panel_kernel(PanelArgs p) {
+__device__ __noinline__ void panel(const PanelArgs& p, int k, uint32_t tmem) {
   constexpr int LDS = COLS + 4;
   cg::cluster_group cluster = cg::this_cluster();
   const int c = (int)cluster.block_rank();
   const int C = (int)cluster.num_blocks();
   const int b = blockIdx.y;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (!qr_block_left(p.state[b], p.Ypart, b, p.kbo)) return;  // factored without the column loop
-
   extern __shared__ float4 smem_dyn[];
   float* sA = reinterpret_cast<float*>(smem_dyn);  // [NB][LDS]: panel row jj, position offset i
   __shared__ float s_part[2][NB];        // this CTA's partial [sigma | x . a_c]
@@ -149,9 +147,806 @@ __global__ void __launch_bounds__(PT, 1) qr_panel_kernel(PanelArgs p) {
   constexpr int SV_BYTES = COLS == PT ? SV_STG * A_BYTES + 2 * (A_BYTES + 2 * B_BYTES) + 1024 : STG * NBO * 36 * 4;
   __shared__ __align__(1024) uint8_t s_sv[SV_BYTES];
   __shared__ __align__(8) uint64_t s_mma_bar[2];
-  __shared__ uint32_t s_tmem;
 
   const int n = p.n, k0 = p.k0, kbo = p.kbo;
+  const int kb = min(NB, n - k);
+  const int jb = k - k0;                // panel offset inside its block
+  const int nrest = kbo - jb - kb;      // block rows after the panel
+  const int64_t nn = (int64_t)n * n;
+  float* At = p.At + (int64_t)b * nn;
+  const int pos0 = k + c * COLS;  // first position held by this CTA
+  const int npos = max(0, min(COLS, n - pos0));  // a multiple of 4
+
+  const int npad = (npos + 31) & ~31;  // positions read by the chunked S V product
+  {
+    const int q4n = npad / 4;
+    for (int e = tid; e < NB * q4n; e += PT) {
+      const int jj = e / q4n, i = 4 * (e % q4n);
+      const bool ok = jj < kb && i < npos;
+      const float* src = ok ? At + (int64_t)(k + jj) * n + pos0 + i : At;
+      const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(&sA[jj * LDS + i]));
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+  }
+  __syncthreads();
+  const float thresh = p.thresh[b];
+  int nonfinite = 0;
+
+  if constexpr (COLS == PT) {
+    // One position per thread: thread tid holds the panel rows' values at position tid in
+    // registers, the current row first (a[l] = row j + l; rows past the panel are zero), so
+    // that the per-column dot products and the reflector's update never touch shared memory;
+    // only v (row j) is written back, for the phases after the loop.
+    const int i = tid;
+    const bool have = i < npos;
+    float a[NB];
+#pragma unroll
+    for (int l = 0; l < NB; ++l) a[l] = (have && l < kb) ? sA[l * LDS + i] : 0.f;
+    for (int j = 0; j < kb; ++j) {
+      const int par = j & 1;
+      // this position's share of sigma (l = 0) and of x . a_(j+l) (l > 0), for positions
+      // strictly after the pivot (pivot = local position j of rank 0)
+      const float x = (have && (c != 0 || i > j)) ? a[0] : 0.f;
+      float v[NB];
+      // transposing butterfly over the warp: lane l ends with the warp's sum for row j + l
+#define SOAP_BFLY(o, nh)                                                   \
+  {                                                                        \
+    const bool up = (lane & (o)) != 0;                                     \
+    _Pragma("unroll") for (int q = 0; q < (nh); ++q) {                     \
+      const float keep = up ? v[q + (nh)] : v[q];                          \
+      const float send = up ? v[q] : v[q + (nh)];                          \
+      v[q] = keep + __shfl_xor_sync(0xffffffffu, send, (o));               \
+    }                                                                      \
+  }
+      if (kb - j > NB / 2) {
+#pragma unroll
+        for (int l = 0; l < NB; ++l) v[l] = x * a[l];
+        SOAP_BFLY(16, 16)
+        SOAP_BFLY(8, 8)
+        SOAP_BFLY(4, 4)
+        SOAP_BFLY(2, 2)
+        SOAP_BFLY(1, 1)
+      } else {
+        // at most 16 rows left (the rest of a[] is zero): the butterfly over the 16 live values
+        // within each half-warp (lane l ends with row j + (l mod 16)), then across the halves
+#pragma unroll
+        for (int l = 0; l < NB / 2; ++l) v[l] = x * a[l];
+        SOAP_BFLY(8, 8)
+        SOAP_BFLY(4, 4)
+        SOAP_BFLY(2, 2)
+        SOAP_BFLY(1, 1)
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
+      }
+#undef SOAP_BFLY
+      s_red[warp][lane] = v[0];
+      // rank 0's pivot position: alpha and the later rows' values there
+      if (c == 0 && i == j) {
+#pragma unroll
+        for (int l = 0; l < NB; ++l)
+          if (j + l < kb) s_pv[par][j + l] = a[l];
+      }
+      __syncthreads();
+      if (warp == 0) {
+        float sum = 0.f;
+#pragma unroll
+        for (int w = 0; w < NWARP; ++w) sum += s_red[w][lane];
+        if (j + lane < kb) s_part[par][j + lane] = sum;
+      }
+      cluster.sync();
+      // threads j..kb-1 reduce sigma and their own column's sum (in the same fixed order, so
+      // they all derive the same reflector) and form v^T a_tid
+      if (warp == 0) {
+        s_wl[lane] = 0.f;
+        __syncwarp();
+      }
+      if (tid >= j && tid < kb) {
+        float ps[MAXC], pd[MAXC];
+#pragma unroll
+        for (int q = 0; q < MAXC; ++q) {
+          if (q < C) {
+            const float* rp = cluster.map_shared_rank(&s_part[par][0], q);
+            ps[q] = rp[j];
+            pd[q] = rp[tid];
+          }
+        }
+        const float* pv0 = cluster.map_shared_rank(&s_pv[par][0], 0);
+        const float alpha = pv0[j], apiv = pv0[tid];
+        float d = 0.f, sigma = 0.f;
+#pragma unroll
+        for (int q = 0; q < MAXC; ++q) {
+          if (q < C) {
+            sigma += ps[q];
+            d += pd[q];
+          }
+        }
+        const float xnorm = sqrtf(fmaf(alpha, alpha, sigma));
+        const bool skip = !(xnorm > thresh);
+        float tau = 0.f, v0 = 1.f, rsign = 1.f;
+        if (!skip) {
+          if (sigma == 0.f) {
+            rsign = alpha < 0.f ? -1.f : 1.f;   // H = I, R_pp = alpha
+          } else {
+            const float beta = alpha >= 0.f ? -xnorm : xnorm;
+            v0 = alpha - beta;                   // same sign as alpha: no cancellation
+            tau = (beta - alpha) / beta;
+            rsign = beta < 0.f ? -1.f : 1.f;
+          }
+        }
+        if (tid == j) {
+          if (!isfinite(xnorm)) nonfinite = 1;
+          s_tau[j] = tau;
+          s_skip[j] = skip ? 1 : 0;
+          s_dsign[j] = rsign;
+          s_scal[0] = tau;
+          s_scal[1] = tau != 0.f ? 1.f / v0 : 0.f;
+        } else {
+          s_wl[tid - j] = tau != 0.f ? apiv + d / v0 : 0.f;  // v^T a_tid, with v = x / v0 after the pivot
+        }
+      }
+      __syncthreads();
+      const float tau = s_scal[0], rv0 = s_scal[1];
+      // v at this position (x / v0 after the pivot, 1 at it) and H_j = I - tau v v^T on the
+      // later rows, shifting them down one register; positions before the pivot only shift
+      if (have && (c != 0 || i >= j)) {
+        const bool at_pivot = (c == 0 && i == j);
+        const float vi = at_pivot ? 1.f : a[0] * rv0;
+        if (!at_pivot) sA[j * LDS + i] = vi;
+        if (tau != 0.f) {
+          const float tv = tau * vi;
+#pragma unroll
+          for (int l4 = 0; l4 < NB / 4; ++l4) {
+            const float4 w4 = reinterpret_cast<const float4*>(s_wl)[l4];
+            if (l4 > 0) a[4 * l4 - 1] = fmaf(-tv, w4.x, a[4 * l4]);
+            a[4 * l4] = fmaf(-tv, w4.y, a[4 * l4 + 1]);
+            a[4 * l4 + 1] = fmaf(-tv, w4.z, a[4 * l4 + 2]);
+            a[4 * l4 + 2] = fmaf(-tv, w4.w, a[4 * l4 + 3]);
+          }
+          a[NB - 1] = 0.f;
+        } else {
+#pragma unroll
+          for (int l = 0; l < NB - 1; ++l) a[l] = a[l + 1];
+          a[NB - 1] = 0.f;
+        }
+      } else {
+#pragma unroll
+        for (int l = 0; l < NB - 1; ++l) a[l] = a[l + 1];
+        a[NB - 1] = 0.f;
+      }
+      __syncthreads();  // s_wl, s_red and s_scal are rewritten by the next column
+    }
+  } else {
+    for (int j = 0; j < kb; ++j) {
+      const int par = j & 1;
+      // positions strictly after the pivot (pivot = local position j of rank 0)
+      const int ibeg = (c == 0) ? j + 1 : 0;
+      // partial sums over this CTA: sigma (cc = j) and x . a_cc (cc > j), kept locally; after
+      // the cluster barrier the threads that need them read every CTA's copy. Warp w takes
+      // columns j + w and j + w + 16 in one pass over x (kb - j <= 32 columns).
+      {
+        const int c1 = j + warp, c2 = c1 + NWARP;
+        if (c1 < kb) {
+          const bool h2 = c2 < kb;
+          float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, b0 = 0.f, b1 = 0.f, b2 = 0.f, b3 = 0.f;
+          const float* xr = sA + j * LDS;
+          const float* r1 = sA + c1 * LDS;
+          const float* r2 = sA + (h2 ? c2 : c1) * LDS;
+          int i = ibeg + lane;
+          for (; i + 96 < npos; i += 128) {
+            const float x0 = xr[i], x1 = xr[i + 32], x2 = xr[i + 64], x3 = xr[i + 96];
+            a0 = fmaf(x0, r1[i], a0);
+            a1 = fmaf(x1, r1[i + 32], a1);
+            a2 = fmaf(x2, r1[i + 64], a2);
+            a3 = fmaf(x3, r1[i + 96], a3);
+            b0 = fmaf(x0, r2[i], b0);
+            b1 = fmaf(x1, r2[i + 32], b1);
+            b2 = fmaf(x2, r2[i + 64], b2);
+            b3 = fmaf(x3, r2[i + 96], b3);
+          }
+          for (; i < npos; i += 32) {
+            const float x0 = xr[i];
+            a0 = fmaf(x0, r1[i], a0);
+            b0 = fmaf(x0, r2[i], b0);
+          }
+          float da = (a0 + a1) + (a2 + a3), db = (b0 + b1) + (b2 + b3);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            da += __shfl_xor_sync(0xffffffffu, da, o);
+            db += __shfl_xor_sync(0xffffffffu, db, o);
+          }
+          if (lane == 0) {
+            s_part[par][c1] = da;
+            if (h2) s_part[par][c2] = db;
+          }
+        }
+      }
+      if (c == 0 && tid >= j && tid < kb) s_pv[par][tid] = sA[tid * LDS + j];  // alpha (tid == j), a_tid at the pivot
+      cluster.sync();
+      // threads j..kb-1 reduce sigma and their own column's sum (in the same fixed order, so
+      // they all derive the same reflector) and form v^T a_tid
+      if (tid >= j && tid < kb) {
+        float ps[MAXC], pd[MAXC];
+#pragma unroll
+        for (int q = 0; q < MAXC; ++q) {
+          if (q < C) {
+            const float* rp = cluster.map_shared_rank(&s_part[par][0], q);
+            ps[q] = rp[j];
+            pd[q] = rp[tid];
+          }
+        }
+        const float* pv0 = cluster.map_shared_rank(&s_pv[par][0], 0);
+        const float alpha = pv0[j], apiv = pv0[tid];
+        float d = 0.f, sigma = 0.f;
+#pragma unroll
+        for (int q = 0; q < MAXC; ++q) {
+          if (q < C) {
+            sigma += ps[q];
+            d += pd[q];
+          }
+        }
+        const float xnorm = sqrtf(fmaf(alpha, alpha, sigma));
+        const bool skip = !(xnorm > thresh);
+        float tau = 0.f, v0 = 1.f, rsign = 1.f;
+        if (!skip) {
+          if (sigma == 0.f) {
+            rsign = alpha < 0.f ? -1.f : 1.f;   // H = I, R_pp = alpha
+          } else {
+            const float beta = alpha >= 0.f ? -xnorm : xnorm;
+            v0 = alpha - beta;                   // same sign as alpha: no cancellation
+            tau = (beta - alpha) / beta;
+            rsign = beta < 0.f ? -1.f : 1.f;
+          }
+        }
+        if (tid == j) {
+          if (!isfinite(xnorm)) nonfinite = 1;
+          s_tau[j] = tau;
+          s_skip[j] = skip ? 1 : 0;
+          s_dsign[j] = rsign;
+          s_scal[0] = tau;
+          s_scal[1] = tau != 0.f ? 1.f / v0 : 0.f;
+        } else if (tau != 0.f) {
+          s_w[tid] = apiv + d / v0;  // v^T a_tid, with v = x / v0 after the pivot
+        }
+      }
+      __syncthreads();
+      const float tau = s_scal[0], rv0 = s_scal[1];
+
+      // v after the pivot (x / v0, or 0 where H = I), and H_j = I - tau v v^T on the later
+      // panel rows; every thread owns its positions
+      const int piv = (c == 0) ? j : 0;  // local positions >= this take part
+      for (int i = piv + tid; i < npos; i += PT) {
+        const bool at_pivot = (c == 0 && i == j);
+        const float vi = at_pivot ? 1.f : sA[j * LDS + i] * rv0;
+        if (!at_pivot) sA[j * LDS + i] = vi;
+        if (tau != 0.f) {
+          const float tv = tau * vi;
+          for (int cc = j + 1; cc < kb; ++cc) sA[cc * LDS + i] = fmaf(-tv, s_w[cc], sA[cc * LDS + i]);
+        }
+      }
+      __syncthreads();
+    }
+  }
+  if (nonfinite) atomicOr(p.status, kStatusQrBreakdown);
+
+  // V with its unit diagonal and zeros before it (rank 0 holds the first kb positions)
+  if (c == 0) {
+    for (int e = tid; e < kb * kb; e += PT) {
+      const int jj = e / kb, i = e % kb;
+      if (i < jj) sA[jj * LDS + i] = 0.f;
+      else if (i == jj) sA[jj * LDS + i] = 1.f;
+    }
+  }
+  __syncthreads();
+
+  // V as rows of Vt (zeros at the block's positions before the panel) and as columns jb..
+  // of the block's position-major Vpos
+  float* Vt = p.Vt + (int64_t)b * nn;
+  float* Vt_lo = p.Vt_lo + (int64_t)b * nn;
+  float* Vpos = p.Vpos + (int64_t)b * n * NBO;
+  float* Vpos_lo = p.Vpos_lo + (int64_t)b * n * NBO;
+  {
+    const int q4n = npos / 4;
+    for (int e = tid; e < kb * q4n; e += PT) {
+      const int jj = e / q4n, q = e - jj * q4n;
+      const int64_t o = (int64_t)(k + jj) * n + pos0 + 4 * q;
+      const float4 v = *reinterpret_cast<const float4*>(&sA[jj * LDS + 4 * q]);
+      *reinterpret_cast<float4*>(Vt + o) = v;
+      *reinterpret_cast<float4*>(Vt_lo + o) = make_float4(tf32_lo(v.x), tf32_lo(v.y), tf32_lo(v.z), tf32_lo(v.w));
+    }
+  }
+  for (int e = tid; e < npos * (NB / 4); e += PT) {
+    const int i = e >> 3, g4 = 4 * (e & 7);  // rows kb.. of sA are zero
+    const float4 v = make_float4(sA[g4 * LDS + i], sA[(g4 + 1) * LDS + i], sA[(g4 + 2) * LDS + i], sA[(g4 + 3) * LDS + i]);
+    const int64_t o = (int64_t)(pos0 + i) * NBO + jb + g4;
+    *reinterpret_cast<float4*>(Vpos + o) = v;
+    *reinterpret_cast<float4*>(Vpos_lo + o) = make_float4(tf32_lo(v.x), tf32_lo(v.y), tf32_lo(v.z), tf32_lo(v.w));
+  }
+  if (c == 0) {
+    for (int jj = 0; jj < kb; ++jj)
+      for (int i = tid; i < jb; i += PT) {
+        const int64_t o = (int64_t)(k + jj) * n + k0 + i;
+        Vt[o] = 0.f;
+        Vt_lo[o] = 0.f;
+      }
+    for (int e = tid; e < jb * NB; e += PT) {
+      const int64_t o = (int64_t)(k0 + e / NB) * NBO + jb + e % NB;
+      Vpos[o] = 0.f;
+      Vpos_lo[o] = 0.f;
+    }
+  }
+  __syncthreads();  // this CTA's Vt rows are read back below
+
+  // Y = S V_panel over this CTA's positions, S = the block's rows k0 .. k0+kbo-1: the block's
+  // Householder vectors so far (rows before the panel's end, from Vt) and the block rows still
+  // to be factored (from At), with both operands split into tf32 hi and lo parts (four
+  // products: fp32 accuracy), each 32-position chunk summed afresh and added to fp32 registers,
+  // so that the tensor core's own accumulation never runs longer than 32 positions.
+  if constexpr (COLS == PT) {
+    // On the tcgen05 tensor cores: D[128 x 32] (tensor memory) = S chunk (A: 128 rows x 32
+    // positions) x V chunk^T (B: 32 rows x 32 positions), both K-major in the 128-byte-swizzled
+    // layout. S's rows other than the panel's are copied with cp.async straight into that
+    // layout, SV_STG - 1 chunks ahead, and each thread forms the lo part of the units it copied;
+    // the panel's rows of S and the V chunk (hi and lo) come from sA. Two accumulators and two
+    // lo sets alternate: while the MMAs of chunk ch run, warps 0-3 drain chunk ch-1 (warp w
+    // reads lanes 32w..) and its S stage is refilled.
+    uint8_t* sv = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(s_sv) + 1023) & ~uintptr_t(1023));
+    uint8_t* st_a = sv;                          // [SV_STG] S chunks (fp32, read by the MMA as its hi part)
+    uint8_t* st_lo = sv + SV_STG * A_BYTES;      // [2] S lo | V hi | V lo
+    constexpr int LO_SET = A_BYTES + 2 * B_BYTES;
+    const int nchunk = (npos + 31) / 32;
+    if (tid == 0) {
+      tc::mbar_init(&s_mma_bar[0], 1);
+      tc::mbar_init(&s_mma_bar[1], 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    // byte offset of 16-byte unit q of row r in a tile of 128-byte rows, swizzled within
+    // 1024-byte groups of 8 rows
+    auto swz16 = [](int r, int q) { return (r >> 3) * 1024 + (r & 7) * 128 + ((q ^ (r & 7)) << 4); };
+    auto issue = [&](int ch) {
+      uint8_t* dst = st_a + (ch % SV_STG) * A_BYTES;
+      for (int u = tid; u < NBO * 8; u += PT) {
+        const int r = u >> 3, q = u & 7;
+        if (r >= jb && r < jb + NB) continue;  // the panel's own rows: V, from sA
+        const int row = k0 + r, i = ch * 32 + 4 * q;
+        const bool ok = r < kbo && i < npos;  // zero-filled outside the block and past the positions
+        const float* src = ok ? (r < jb ? Vt : At) + (int64_t)row * n + pos0 + i : At;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(dst + swz16(r, q))),
+                     "l"(src), "r"(ok ? 16 : 0)
+                     : "memory");
+      }
+    };
+    auto lo4 = [](float4 x) { return make_float4(tf32_lo(x.x), tf32_lo(x.y), tf32_lo(x.z), tf32_lo(x.w)); };
+    float y[NB];
+#pragma unroll
+    for (int l = 0; l < NB; ++l) y[l] = 0.f;
+    for (int st0 = 0; st0 < SV_STG - 1; ++st0) {
+      if (st0 < nchunk) issue(st0);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    int issued = 0;  // chunks whose MMAs were issued
+    bool aborted = false, bad = false;
+    for (int ch = 0; ch < nchunk; ++ch) {
+      const int set = ch & 1;
+      // this thread's copies of chunk ch have landed: their lo parts; the panel's rows of S and
+      // the V chunk (hi and lo) from sA
+      asm volatile("cp.async.wait_group %0;" ::"n"(SV_STG - 2) : "memory");
+      {
+        uint8_t* a = st_a + (ch % SV_STG) * A_BYTES;
+        uint8_t* lo = st_lo + set * LO_SET;
+        for (int u = tid; u < NBO * 8; u += PT) {
+          const int r = u >> 3;
+          if (r >= jb && r < jb + NB) continue;
+          const int off = swz16(r, u & 7);
+          *reinterpret_cast<float4*>(lo + off) = lo4(*reinterpret_cast<const float4*>(a + off));
+        }
+        uint8_t* bh = lo + A_BYTES;
+        uint8_t* bl = bh + B_BYTES;
+        for (int u = tid; u < NB * 8; u += PT) {
+          const int jj = u >> 3, q = u & 7;
+          const float4 x = *reinterpret_cast<const float4*>(&sA[jj * LDS + ch * 32 + 4 * q]);
+          const float4 xl = lo4(x);
+          const int off = swz16(jj, q), offa = swz16(jb + jj, q);
+          *reinterpret_cast<float4*>(bh + off) = x;
+          *reinterpret_cast<float4*>(bl + off) = xl;
+          *reinterpret_cast<float4*>(a + offa) = x;
+          *reinterpret_cast<float4*>(lo + offa) = xl;
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      if (__syncthreads_or(bad)) {
+        aborted = true;
+        break;
+      }
+      // the MMAs of chunk ch (its lo set and accumulator were released in the previous pass)
+      if (tid == 0) {
+        tc::tc_fence_after();
+        constexpr uint32_t idesc = tc::idesc_tf32(NBO, NB);
+        const uint32_t d = tmem + (uint32_t)(set * 32);
+        const uint32_t a_hi = tc::smem_u32(st_a + (ch % SV_STG) * A_BYTES);
+        const uint32_t a_lo = tc::smem_u32(st_lo + set * LO_SET);
+        const uint32_t b_hi = a_lo + A_BYTES;
+        const uint32_t b_lo = b_hi + B_BYTES;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          const uint32_t off = kk * 32;  // 8 tf32 = 32 bytes along the positions
+          tc::umma_tf32(d, tc::desc_sw128(a_lo + off), tc::desc_sw128(b_lo + off), idesc, kk != 0);
+          tc::umma_tf32(d, tc::desc_sw128(a_lo + off), tc::desc_sw128(b_hi + off), idesc, 1u);
+          tc::umma_tf32(d, tc::desc_sw128(a_hi + off), tc::desc_sw128(b_lo + off), idesc, 1u);
+          tc::umma_tf32(d, tc::desc_sw128(a_hi + off), tc::desc_sw128(b_hi + off), idesc, 1u);
+        }
+        tc::umma_commit(&s_mma_bar[set]);
+      }
+      issued = ch + 1;
+      // while they run: chunk ch-1's MMAs have completed, so its accumulator is drained and its
+      // S stage refilled with chunk ch + SV_STG - 1
+      if (ch >= 1) {
+        bool ok = tc::mbar_wait(&s_mma_bar[(ch - 1) & 1], ((ch - 1) >> 1) & 1, kWaitNs);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) {
+          bad = true;
+        } else if (warp < 4) {
+          float v[32];
+          tc::tmem_ld32(tmem + (uint32_t)(((ch - 1) & 1) * 32) + ((uint32_t)(32 * warp) << 16), v);
+#pragma unroll
+          for (int l = 0; l < NB; ++l) y[l] += v[l];
+        }
+      }
+      if (!bad && ch + SV_STG - 1 < nchunk) issue(ch + SV_STG - 1);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      tc::tc_fence_before();
+    }
+    // the last chunk's sum; after a wait that gave up, only the wait for every issued MMA (with
+    // the full bound), so that the tensor memory is not freed under one
+    bool ok_last = true;
+    if (issued > 0)
+      ok_last = __all_sync(0xffffffffu, tc::mbar_wait(&s_mma_bar[(issued - 1) & 1], ((issued - 1) >> 1) & 1, kWaitNs));
+    if (!aborted && !bad && ok_last && issued > 0 && warp < 4) {
+      float v[32];
+      tc::tmem_ld32(tmem + (uint32_t)(((issued - 1) & 1) * 32) + ((uint32_t)(32 * warp) << 16), v);
+#pragma unroll
+      for (int l = 0; l < NB; ++l) y[l] += v[l];
+    }
+    if (aborted || bad || !ok_last) atomicOr(p.status, kStatusTimeout);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    if (tid == 0) {  // every wait on them is over; the next panel sets them up again
+      asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(tc::smem_u32(&s_mma_bar[0])) : "memory");
+      asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(tc::smem_u32(&s_mma_bar[1])) : "memory");
+    }
+    // this CTA's partial product, kept in shared memory (the S stages are free) for the cluster
+    if (warp < 4) {
+      float* yp = reinterpret_cast<float*>(sv) + (32 * warp + lane) * NB;
+#pragma unroll
+      for (int l4 = 0; l4 < NB / 4; ++l4)
+        *reinterpret_cast<float4*>(yp + 4 * l4) = make_float4(y[4 * l4], y[4 * l4 + 1], y[4 * l4 + 2], y[4 * l4 + 3]);
+    }
+  } else
+  // With 1024 positions per CTA (factors of at most 1024 rows): S is streamed through shared
+  // memory in 32-position chunks (cp.async, STG buffers, rows padded to 36 floats), and the
+  // product runs as warp-level m16n8k8 TF32 MMAs. Warp w owns rows 16 (w mod 8) .. +15 and
+  // columns 16 (w / 8) .. +15.
+  {
+    static_assert(NBO == 128 && NB == 32 && NWARP == 16, "8 x 2 warp tiles of 16 x 16");
+    constexpr int CH = 32;       // positions per chunk
+    constexpr int CHP = CH + 4;  // padded row stride of a staged chunk
+    const int gq = lane >> 2, tg = lane & 3;
+    const int m0 = 16 * (warp & 7), nb = 16 * (warp >> 3);
+    float y[2][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) y[0][e] = y[1][e] = 0.f;
+    const int nchunk = (npos + CH - 1) / CH;
+    auto issue = [&](int ch, int buf) {
+      float* dst = reinterpret_cast<float*>(s_sv) + buf * NBO * CHP;
+      for (int e = tid; e < NBO * (CH / 4); e += PT) {
+        const int r = e / (CH / 4), q4 = e % (CH / 4);
+        const int row = k0 + r, i = ch * CH + 4 * q4;
+        const bool ok = r < kbo && i < npos;
+        const float* src = ok ? ((row < k + kb) ? Vt : At) + (int64_t)row * n + pos0 + i : At;
+        const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst + r * CHP + 4 * q4));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int st0 = 0; st0 < STG - 1; ++st0) {
+      if (st0 < nchunk) issue(st0, st0);
+      else asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    for (int ch = 0; ch < nchunk; ++ch) {
+      if (ch + STG - 1 < nchunk) issue(ch + STG - 1, (ch + STG - 1) % STG);
+      else asm volatile("cp.async.commit_group;" ::: "memory");  // keeps the group count uniform
+      asm volatile("cp.async.wait_group %0;" ::"n"(STG - 1) : "memory");
+      __syncthreads();
+      const float* st = reinterpret_cast<const float*>(s_sv) + (ch % STG) * NBO * CHP;
+      const int i0 = ch * CH;
+      float d[2][4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) d[0][e] = d[1][e] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < CH / 8; ++ks) {
+        // positions past npos are zero in the staged chunk and in V (zero-filled copies)
+        const int kk = 8 * ks;
+        const float av[4] = {st[(m0 + gq) * CHP + kk + tg], st[(m0 + gq + 8) * CHP + kk + tg],
+                             st[(m0 + gq) * CHP + kk + tg + 4], st[(m0 + gq + 8) * CHP + kk + tg + 4]};
+        uint32_t ah[4], al[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) tf32_split(av[e], ah[e], al[e]);
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+          const float* vr = sA + (nb + 8 * nt + gq) * LDS + i0 + kk + tg;
+          uint32_t bh[2], bl[2];
+          tf32_split(vr[0], bh[0], bl[0]);
+          tf32_split(vr[4], bh[1], bl[1]);
+          mma_tf32_16x8x8(d[nt], al, bl);
+          mma_tf32_16x8x8(d[nt], al, bh);
+          mma_tf32_16x8x8(d[nt], ah, bl);
+          mma_tf32_16x8x8(d[nt], ah, bh);
+        }
+      }
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) y[nt][e] += d[nt][e];
+      __syncthreads();  // this buffer is refilled STG - 1 chunks later
+    }
+    float* yp = p.Ypart + ((int64_t)b * MAXC + c) * NBO * NB;
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt) {
+      const int col = nb + 8 * nt + 2 * tg;
+      *reinterpret_cast<float2*>(yp + (m0 + gq) * NB + col) = make_float2(y[nt][0], y[nt][1]);
+      *reinterpret_cast<float2*>(yp + (m0 + gq + 8) * NB + col) = make_float2(y[nt][2], y[nt][3]);
+    }
+  }
+  // T_panel from the Gram rows of Y, then U = X T_panel (in place) and Z (rows after the panel);
+  // every thread of the CTA takes part (the barriers inside)
+  auto form_tuz = [&]() {
+    // T of the panel from its Gram matrix g (rows jb.. of Y): T^-1 = diag(1/tau) + striu(g)
+    // (H_1 ... H_kb = I - V T V^T); a reflector with tau = 0 (v = 0) gets a zero row and column.
+    // Warp w solves columns w and w + 16 by back substitution, lane i holding x_i:
+    //   x_i = tau_i (delta_{i,cc} - sum_{i < l <= cc} g_il x_l)   (tau_i read as 1 where it is 0)
+    // Each solved x_l is broadcast once and every lane i < l adds g_il x_l to its running sum,
+    // so a step costs one shuffle instead of a warp-wide reduction.
+    for (int cc = warp; cc < NB; cc += NWARP) {
+      float x = 0.f, acc = 0.f;
+      for (int l = cc; l >= 0; --l) {
+        const float g = s_Y[jb + lane][l];
+        if (lane == l) {
+          const float tl = l < kb ? s_tau[l] : 0.f;
+          x = ((l == cc ? 1.f : 0.f) - acc) * (tl != 0.f ? tl : 1.f);
+        }
+        const float xl = __shfl_sync(0xffffffffu, x, l);
+        if (lane < l) acc = fmaf(g, xl, acc);
+      }
+      const bool live = cc < kb && s_tau[cc] != 0.f;
+      s_T[lane][cc] = (live && lane <= cc && lane < kb && s_tau[lane] != 0.f) ? x : 0.f;
+    }
+    __syncthreads();
+    // U = X T_panel with X = V_before^T V_panel (rows 0..jb-1 of Y), in place, and
+    // Z = (S_rest V_panel) T_panel for the block rows after the panel: thread (r, g) forms
+    // columns 8g .. 8g+7 of row r
+    {
+      const int r = tid >> 2, g8 = (tid & 3) * 8;
+      const bool act = r < kbo && (r < jb || r >= jb + kb);
+      float x[NB];
+#pragma unroll
+      for (int l = 0; l < NB; ++l) x[l] = act ? s_Y[r][l] : 0.f;
+      __syncthreads();  // every row is read before U overwrites it
+      if (act) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int cc = g8 + u;
+          float acc = 0.f;
+#pragma unroll
+          for (int l = 0; l < NB; ++l)
+            if (l <= cc) acc = fmaf(x[l], s_T[l][cc], acc);
+          if (r < jb) s_Y[r][cc] = acc;
+          else s_Z[r - jb - kb][cc] = acc;
+        }
+      }
+    }
+    __syncthreads();
+  };
+  if constexpr (COLS == PT) {
+    // The partial products reduced through distributed shared memory: CTA c sums rows
+    // r = c mod C of every CTA's partial, in a fixed order, and every CTA then gathers the summed
+    // rows and forms T_panel, U and Z itself (the same values on every CTA).
+    uint8_t* sv = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(s_sv) + 1023) & ~uintptr_t(1023));
+    float* P_own = reinterpret_cast<float*>(sv);
+    float* Ysum = P_own + NBO * NB;
+    cluster.sync();  // every CTA's partial is in place
+    for (int r = c + C * warp; r < kbo; r += C * NWARP) {
+      float part[MAXC];
+#pragma unroll
+      for (int q = 0; q < MAXC; ++q) part[q] = q < C ? cluster.map_shared_rank(P_own, q)[r * NB + lane] : 0.f;
+      float sum = 0.f;
+#pragma unroll
+      for (int q = 0; q < MAXC; ++q) sum += part[q];
+      Ysum[r * NB + lane] = sum;
+    }
+    cluster.sync();  // every summed row is in place
+    for (int e = tid; e < kbo * NB; e += PT) s_Y[e / NB][e % NB] = cluster.map_shared_rank(Ysum, (e / NB) % C)[e];
+    // (the peers may read this CTA's summed rows until the last barrier of the panel)
+    __syncthreads();
+    form_tuz();
+    __syncthreads();
+    if (c == 0 && tid < kb) {
+      p.skip[(int64_t)b * n + k + tid] = (uint8_t)s_skip[tid];
+      p.dsign[(int64_t)b * n + k + tid] = s_dsign[tid];
+    }
+  } else {
+    cluster.sync();  // orders the partials in global memory before rank 0 reads them
+    // rank 0 sums the partials, forms T_panel, U = X T_panel and Z, and hands Z, U and T_panel
+    // to the cluster through global memory (rank 0's slots of Ypart, free once it has summed
+    // them): Z at 0, U at 3072 (jb <= 96 rows), T_panel at 6144 floats
+    float* xg = p.Ypart + (int64_t)b * MAXC * NBO * NB;
+    float* Ug = xg + NREST * NB;
+    float* Tpg = xg + 2 * NREST * NB;
+    if (c == 0) {
+      // sum the partials in a fixed order
+      const float* yp = p.Ypart + (int64_t)b * MAXC * NBO * NB;
+      for (int e = tid; e < kbo * NB; e += PT) {
+        float part[MAXC];
+#pragma unroll
+        for (int q = 0; q < MAXC; ++q) part[q] = q < C ? yp[(int64_t)q * NBO * NB + e] : 0.f;
+        float sum = 0.f;
+#pragma unroll
+        for (int q = 0; q < MAXC; ++q) sum += part[q];
+        s_Y[e / NB][e % NB] = sum;
+      }
+      __syncthreads();
+      form_tuz();
+      __syncthreads();
+      for (int e = tid; e < nrest * NB; e += PT) xg[e] = s_Z[e / NB][e % NB];
+      for (int e = tid; e < jb * NB; e += PT) Ug[e] = s_Y[e / NB][e % NB];
+      for (int e = tid; e < NB * NB; e += PT) Tpg[e] = s_T[e / NB][e % NB];
+      if (tid < kb) {
+        p.skip[(int64_t)b * n + k + tid] = (uint8_t)s_skip[tid];
+        p.dsign[(int64_t)b * n + k + tid] = s_dsign[tid];
+      }
+    }
+    cluster.sync();  // Z, U and T_panel in global memory are visible to the cluster
+    if (c != 0) {
+      for (int e = tid; e < nrest * NB; e += PT) s_Z[e / NB][e % NB] = xg[e];
+      for (int e = tid; e < jb * NB; e += PT) s_Y[e / NB][e % NB] = Ug[e];
+      for (int e = tid; e < NB * NB; e += PT) s_T[e / NB][e % NB] = Tpg[e];
+    }
+    __syncthreads();
+  }
+  // the block's T, rows spread over the cluster (row r by CTA r mod C): column block jb =
+  // [-T_before U ; T_panel ; 0] and the row block jb left of it = 0
+  {
+    float* T = p.T + (int64_t)b * NBO * NBO;
+    float* T_lo = p.T_lo + (int64_t)b * NBO * NBO;
+    float* Tt = p.Tt + (int64_t)b * NBO * NBO;
+    float* Tt_lo = p.Tt_lo + (int64_t)b * NBO * NBO;
+    // the rows of T_before (written by the block's earlier panels) that this CTA's rows need,
+    // staged in shared memory with independent loads: the S V area is free (on the cluster path
+    // past its first 32 KB, the summed rows that peers may still read)
+    constexpr int TBS = NBO - NB;  // jb <= 96
+    float* Tb = reinterpret_cast<float*>(
+        COLS == PT ? ((reinterpret_cast<uintptr_t>(s_sv) + 1023) & ~uintptr_t(1023)) + 2 * NBO * NB * sizeof(float)
+                   : reinterpret_cast<uintptr_t>(s_sv));
+    static_assert(TBS * TBS * sizeof(float) <= (COLS == PT ? SV_BYTES - 1024 - 2 * NBO * NB * sizeof(float) : SV_BYTES),
+                  "T_before staging");
+    const int nrl = jb > c ? (jb - c + C - 1) / C : 0;  // this CTA's rows r = c + C rl below jb
+    for (int e = tid; e < nrl * jb; e += PT) {
+      const int rl = e / jb, l = e - rl * jb, rr = c + C * rl;
+      Tb[rl * TBS + l] = l >= rr ? T[rr * NBO + l] : 0.f;
+    }
+    __syncthreads();
+    // one entry (row r = c + C rl, column jb + cc) per work unit, the 32 units of a row on
+    // consecutive threads: the triangular product's long rows are spread over all threads in
+    // turn. On the cluster path the column block is also staged transposed, so that Tt's rows
+    // are written with consecutive stores.
+    const int nr = (NBO - c + C - 1) / C;  // this CTA's rows
+    float* stt = COLS == PT ? Tb + TBS * TBS : nullptr;  // [NB][NBO]: entry (cc, rl)
+    static_assert(COLS != PT || (TBS * TBS + NB * NBO) * sizeof(float) <= SV_BYTES - 1024 - 2 * NBO * NB * sizeof(float),
+                  "T column block staging");
+    for (int u = tid; u < nr * NB; u += PT) {
+      const int rl = u >> 5, cc = u & 31, r = c + C * rl;
+      float t = 0.f;
+      if (r < jb) {
+        const float* tb_row = Tb + rl * TBS;
+#pragma unroll 4
+        for (int l = r; l < jb; ++l) t = fmaf(-tb_row[l], s_Y[l][cc], t);
+      } else if (r < jb + NB) {
+        t = s_T[r - jb][cc];
+      }
+      const int col = jb + cc;
+      T[r * NBO + col] = t;
+      T_lo[r * NBO + col] = tf32_lo(t);
+      if (COLS == PT) {
+        stt[cc * NBO + rl] = t;
+      } else {
+        Tt[col * NBO + r] = t;
+        Tt_lo[col * NBO + r] = tf32_lo(t);
+      }
+    }
+    if (COLS == PT) {
+      __syncthreads();
+      for (int e = tid; e < NB * nr; e += PT) {
+        const int cc = e / nr, rl = e - cc * nr;
+        const float t = stt[cc * NBO + rl];
+        Tt[(jb + cc) * NBO + c + C * rl] = t;
+        Tt_lo[(jb + cc) * NBO + c + C * rl] = tf32_lo(t);
+      }
+    }
+    // the row block jb left of the panel is zero: T's rows jb.. and Tt's columns jb.. there
+    for (int e = tid; e < NB * jb; e += PT) {
+      const int rr = jb + e / jb, col = e % jb;
+      if (rr % C != c) continue;
+      T[rr * NBO + col] = 0.f;
+      T_lo[rr * NBO + col] = 0.f;
+    }
+    for (int e = tid; e < NB * jb; e += PT) {
+      const int col = e / NB, rr = jb + e % NB;
+      if (rr % C != c) continue;
+      Tt[col * NBO + rr] = 0.f;
+      Tt_lo[col * NBO + rr] = 0.f;
+    }
+  }
+
+  // the panel's reflectors on the block rows after it: a_r -= Z_r V^T at this CTA's
+  // positions, eight rows at a time (eight independent loads in flight), then four, then one
+  for (int i = tid; i < npos; i += PT) {
+    float v[NB];
+#pragma unroll
+    for (int jj = 0; jj < NB; ++jj) v[jj] = sA[jj * LDS + i];
+    float* a = At + (int64_t)(k + kb) * n + pos0 + i;
+    int r = 0;
+    for (; r + 8 <= nrest; r += 8) {
+      float x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = a[(int64_t)(r + u) * n];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        float acc = 0.f;
+#pragma unroll
+        for (int j4 = 0; j4 < NB / 4; ++j4) {
+          const float4 z = *reinterpret_cast<const float4*>(&s_Z[r + u][4 * j4]);
+          acc = fmaf(z.x, v[4 * j4], fmaf(z.y, v[4 * j4 + 1], fmaf(z.z, v[4 * j4 + 2], fmaf(z.w, v[4 * j4 + 3], acc))));
+        }
+        a[(int64_t)(r + u) * n] = x[u] - acc;
+      }
+    }
+    for (; r + 4 <= nrest; r += 4) {
+      float x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = a[(int64_t)(r + u) * n];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float acc = 0.f;
+#pragma unroll
+        for (int j4 = 0; j4 < NB / 4; ++j4) {
+          const float4 z = *reinterpret_cast<const float4*>(&s_Z[r + u][4 * j4]);
+          acc = fmaf(z.x, v[4 * j4], fmaf(z.y, v[4 * j4 + 1], fmaf(z.z, v[4 * j4 + 2], fmaf(z.w, v[4 * j4 + 3], acc))));
+        }
+        a[(int64_t)(r + u) * n] = x[u] - acc;
+      }
+    }
+    for (; r < nrest; ++r) {
+      float acc = 0.f;
+#pragma unroll
+      for (int jj = 0; jj < NB; ++jj) acc = fmaf(s_Z[r][jj], v[jj], acc);
+      a[(int64_t)r * n] -= acc;
+    }
+  }
+  // the next panel's positions are shifted by 32: it reads rows that the other CTAs updated
+  cluster.sync();
+}
+
+// The block's panels one after another, for a matrix whose block was not factored from its Gram matrix.
+// One launch per block, so that a block that was costs one launch that returns at once (four, or eight
+// with the column loop as a kernel of its own, cost 14-20 us).
+template <int COLS>
+__global__ void __launch_bounds__(PT, 1) qr_panel_kernel(const __grid_constant__ PanelArgs p) {
+  const int b = blockIdx.y, warp = threadIdx.x >> 5;
+  if (!qr_block_left(p.state[b], p.Ypart, b, p.kbo)) return;  // factored without the column loop
+
+  __shared__ uint32_t s_tmem;
   uint32_t tmem = 0;
   if constexpr (COLS == PT) {
     if (warp == 0) {
@@ -164,798 +959,7 @@ __global__ void __launch_bounds__(PT, 1) qr_panel_kernel(PanelArgs p) {
     tc::tc_fence_after();
     tmem = s_tmem;
   }
-  for (int k = k0; k < k0 + kbo; k += NB) {
-    const int kb = min(NB, n - k);
-    const int jb = k - k0;                // panel offset inside its block
-    const int nrest = kbo - jb - kb;      // block rows after the panel
-    const int64_t nn = (int64_t)n * n;
-    float* At = p.At + (int64_t)b * nn;
-    const int pos0 = k + c * COLS;  // first position held by this CTA
-    const int npos = max(0, min(COLS, n - pos0));  // a multiple of 4
-
-    const int npad = (npos + 31) & ~31;  // positions read by the chunked S V product
-    {
-      const int q4n = npad / 4;
-      for (int e = tid; e < NB * q4n; e += PT) {
-        const int jj = e / q4n, i = 4 * (e % q4n);
-        const bool ok = jj < kb && i < npos;
-        const float* src = ok ? At + (int64_t)(k + jj) * n + pos0 + i : At;
-        const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(&sA[jj * LDS + i]));
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    __syncthreads();
-    const float thresh = p.thresh[b];
-    int nonfinite = 0;
-
-    if constexpr (COLS == PT) {
-      // One position per thread: thread tid holds the panel rows' values at position tid in
-      // registers, the current row first (a[l] = row j + l; rows past the panel are zero), so
-      // that the per-column dot products and the reflector's update never touch shared memory;
-      // only v (row j) is written back, for the phases after the loop.
-      const int i = tid;
-      const bool have = i < npos;
-      float a[NB];
-#pragma unroll
-      for (int l = 0; l < NB; ++l) a[l] = (have && l < kb) ? sA[l * LDS + i] : 0.f;
-      for (int j = 0; j < kb; ++j) {
-        const int par = j & 1;
-        // this position's share of sigma (l = 0) and of x . a_(j+l) (l > 0), for positions
-        // strictly after the pivot (pivot = local position j of rank 0)
-        const float x = (have && (c != 0 || i > j)) ? a[0] : 0.f;
-        float v[NB];
-        // transposing butterfly over the warp: lane l ends with the warp's sum for row j + l
-#define SOAP_BFLY(o, nh)                                                   \
-    {                                                                        \
-      const bool up = (lane & (o)) != 0;                                     \
-      _Pragma("unroll") for (int q = 0; q < (nh); ++q) {                     \
-        const float keep = up ? v[q + (nh)] : v[q];                          \
-        const float send = up ? v[q] : v[q + (nh)];                          \
-        v[q] = keep + __shfl_xor_sync(0xffffffffu, send, (o));               \
-      }                                                                      \
-    }
-        if (kb - j > NB / 2) {
-#pragma unroll
-          for (int l = 0; l < NB; ++l) v[l] = x * a[l];
-          SOAP_BFLY(16, 16)
-          SOAP_BFLY(8, 8)
-          SOAP_BFLY(4, 4)
-          SOAP_BFLY(2, 2)
-          SOAP_BFLY(1, 1)
-        } else {
-          // at most 16 rows left (the rest of a[] is zero): the butterfly over the 16 live values
-          // within each half-warp (lane l ends with row j + (l mod 16)), then across the halves
-#pragma unroll
-          for (int l = 0; l < NB / 2; ++l) v[l] = x * a[l];
-          SOAP_BFLY(8, 8)
-          SOAP_BFLY(4, 4)
-          SOAP_BFLY(2, 2)
-          SOAP_BFLY(1, 1)
-          v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
-        }
-#undef SOAP_BFLY
-        s_red[warp][lane] = v[0];
-        // rank 0's pivot position: alpha and the later rows' values there
-        if (c == 0 && i == j) {
-#pragma unroll
-          for (int l = 0; l < NB; ++l)
-            if (j + l < kb) s_pv[par][j + l] = a[l];
-        }
-        __syncthreads();
-        if (warp == 0) {
-          float sum = 0.f;
-#pragma unroll
-          for (int w = 0; w < NWARP; ++w) sum += s_red[w][lane];
-          if (j + lane < kb) s_part[par][j + lane] = sum;
-        }
-        cluster.sync();
-        // threads j..kb-1 reduce sigma and their own column's sum (in the same fixed order, so
-        // they all derive the same reflector) and form v^T a_tid
-        if (warp == 0) {
-          s_wl[lane] = 0.f;
-          __syncwarp();
-        }
-        if (tid >= j && tid < kb) {
-          float ps[MAXC], pd[MAXC];
-#pragma unroll
-          for (int q = 0; q < MAXC; ++q) {
-            if (q < C) {
-              const float* rp = cluster.map_shared_rank(&s_part[par][0], q);
-              ps[q] = rp[j];
-              pd[q] = rp[tid];
-            }
-          }
-          const float* pv0 = cluster.map_shared_rank(&s_pv[par][0], 0);
-          const float alpha = pv0[j], apiv = pv0[tid];
-          float d = 0.f, sigma = 0.f;
-#pragma unroll
-          for (int q = 0; q < MAXC; ++q) {
-            if (q < C) {
-              sigma += ps[q];
-              d += pd[q];
-            }
-          }
-          const float xnorm = sqrtf(fmaf(alpha, alpha, sigma));
-          const bool skip = !(xnorm > thresh);
-          float tau = 0.f, v0 = 1.f, rsign = 1.f;
-          if (!skip) {
-            if (sigma == 0.f) {
-              rsign = alpha < 0.f ? -1.f : 1.f;   // H = I, R_pp = alpha
-            } else {
-              const float beta = alpha >= 0.f ? -xnorm : xnorm;
-              v0 = alpha - beta;                   // same sign as alpha: no cancellation
-              tau = (beta - alpha) / beta;
-              rsign = beta < 0.f ? -1.f : 1.f;
-            }
-          }
-          if (tid == j) {
-            if (!isfinite(xnorm)) nonfinite = 1;
-            s_tau[j] = tau;
-            s_skip[j] = skip ? 1 : 0;
-            s_dsign[j] = rsign;
-            s_scal[0] = tau;
-            s_scal[1] = tau != 0.f ? 1.f / v0 : 0.f;
-          } else {
-            s_wl[tid - j] = tau != 0.f ? apiv + d / v0 : 0.f;  // v^T a_tid, with v = x / v0 after the pivot
-          }
-        }
-        __syncthreads();
-        const float tau = s_scal[0], rv0 = s_scal[1];
-        // v at this position (x / v0 after the pivot, 1 at it) and H_j = I - tau v v^T on the
-        // later rows, shifting them down one register; positions before the pivot only shift
-        if (have && (c != 0 || i >= j)) {
-          const bool at_pivot = (c == 0 && i == j);
-          const float vi = at_pivot ? 1.f : a[0] * rv0;
-          if (!at_pivot) sA[j * LDS + i] = vi;
-          if (tau != 0.f) {
-            const float tv = tau * vi;
-#pragma unroll
-            for (int l4 = 0; l4 < NB / 4; ++l4) {
-              const float4 w4 = reinterpret_cast<const float4*>(s_wl)[l4];
-              if (l4 > 0) a[4 * l4 - 1] = fmaf(-tv, w4.x, a[4 * l4]);
-              a[4 * l4] = fmaf(-tv, w4.y, a[4 * l4 + 1]);
-              a[4 * l4 + 1] = fmaf(-tv, w4.z, a[4 * l4 + 2]);
-              a[4 * l4 + 2] = fmaf(-tv, w4.w, a[4 * l4 + 3]);
-            }
-            a[NB - 1] = 0.f;
-          } else {
-#pragma unroll
-            for (int l = 0; l < NB - 1; ++l) a[l] = a[l + 1];
-            a[NB - 1] = 0.f;
-          }
-        } else {
-#pragma unroll
-          for (int l = 0; l < NB - 1; ++l) a[l] = a[l + 1];
-          a[NB - 1] = 0.f;
-        }
-        __syncthreads();  // s_wl, s_red and s_scal are rewritten by the next column
-      }
-    } else {
-      for (int j = 0; j < kb; ++j) {
-        const int par = j & 1;
-        // positions strictly after the pivot (pivot = local position j of rank 0)
-        const int ibeg = (c == 0) ? j + 1 : 0;
-        // partial sums over this CTA: sigma (cc = j) and x . a_cc (cc > j), kept locally; after
-        // the cluster barrier the threads that need them read every CTA's copy. Warp w takes
-        // columns j + w and j + w + 16 in one pass over x (kb - j <= 32 columns).
-        {
-          const int c1 = j + warp, c2 = c1 + NWARP;
-          if (c1 < kb) {
-            const bool h2 = c2 < kb;
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, b0 = 0.f, b1 = 0.f, b2 = 0.f, b3 = 0.f;
-            const float* xr = sA + j * LDS;
-            const float* r1 = sA + c1 * LDS;
-            const float* r2 = sA + (h2 ? c2 : c1) * LDS;
-            int i = ibeg + lane;
-            for (; i + 96 < npos; i += 128) {
-              const float x0 = xr[i], x1 = xr[i + 32], x2 = xr[i + 64], x3 = xr[i + 96];
-              a0 = fmaf(x0, r1[i], a0);
-              a1 = fmaf(x1, r1[i + 32], a1);
-              a2 = fmaf(x2, r1[i + 64], a2);
-              a3 = fmaf(x3, r1[i + 96], a3);
-              b0 = fmaf(x0, r2[i], b0);
-              b1 = fmaf(x1, r2[i + 32], b1);
-              b2 = fmaf(x2, r2[i + 64], b2);
-              b3 = fmaf(x3, r2[i + 96], b3);
-            }
-            for (; i < npos; i += 32) {
-              const float x0 = xr[i];
-              a0 = fmaf(x0, r1[i], a0);
-              b0 = fmaf(x0, r2[i], b0);
-            }
-            float da = (a0 + a1) + (a2 + a3), db = (b0 + b1) + (b2 + b3);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-              da += __shfl_xor_sync(0xffffffffu, da, o);
-              db += __shfl_xor_sync(0xffffffffu, db, o);
-            }
-            if (lane == 0) {
-              s_part[par][c1] = da;
-              if (h2) s_part[par][c2] = db;
-            }
-          }
-        }
-        if (c == 0 && tid >= j && tid < kb) s_pv[par][tid] = sA[tid * LDS + j];  // alpha (tid == j), a_tid at the pivot
-        cluster.sync();
-        // threads j..kb-1 reduce sigma and their own column's sum (in the same fixed order, so
-        // they all derive the same reflector) and form v^T a_tid
-        if (tid >= j && tid < kb) {
-          float ps[MAXC], pd[MAXC];
-#pragma unroll
-          for (int q = 0; q < MAXC; ++q) {
-            if (q < C) {
-              const float* rp = cluster.map_shared_rank(&s_part[par][0], q);
-              ps[q] = rp[j];
-              pd[q] = rp[tid];
-            }
-          }
-          const float* pv0 = cluster.map_shared_rank(&s_pv[par][0], 0);
-          const float alpha = pv0[j], apiv = pv0[tid];
-          float d = 0.f, sigma = 0.f;
-#pragma unroll
-          for (int q = 0; q < MAXC; ++q) {
-            if (q < C) {
-              sigma += ps[q];
-              d += pd[q];
-            }
-          }
-          const float xnorm = sqrtf(fmaf(alpha, alpha, sigma));
-          const bool skip = !(xnorm > thresh);
-          float tau = 0.f, v0 = 1.f, rsign = 1.f;
-          if (!skip) {
-            if (sigma == 0.f) {
-              rsign = alpha < 0.f ? -1.f : 1.f;   // H = I, R_pp = alpha
-            } else {
-              const float beta = alpha >= 0.f ? -xnorm : xnorm;
-              v0 = alpha - beta;                   // same sign as alpha: no cancellation
-              tau = (beta - alpha) / beta;
-              rsign = beta < 0.f ? -1.f : 1.f;
-            }
-          }
-          if (tid == j) {
-            if (!isfinite(xnorm)) nonfinite = 1;
-            s_tau[j] = tau;
-            s_skip[j] = skip ? 1 : 0;
-            s_dsign[j] = rsign;
-            s_scal[0] = tau;
-            s_scal[1] = tau != 0.f ? 1.f / v0 : 0.f;
-          } else if (tau != 0.f) {
-            s_w[tid] = apiv + d / v0;  // v^T a_tid, with v = x / v0 after the pivot
-          }
-        }
-        __syncthreads();
-        const float tau = s_scal[0], rv0 = s_scal[1];
-
-        // v after the pivot (x / v0, or 0 where H = I), and H_j = I - tau v v^T on the later
-        // panel rows; every thread owns its positions
-        const int piv = (c == 0) ? j : 0;  // local positions >= this take part
-        for (int i = piv + tid; i < npos; i += PT) {
-          const bool at_pivot = (c == 0 && i == j);
-          const float vi = at_pivot ? 1.f : sA[j * LDS + i] * rv0;
-          if (!at_pivot) sA[j * LDS + i] = vi;
-          if (tau != 0.f) {
-            const float tv = tau * vi;
-            for (int cc = j + 1; cc < kb; ++cc) sA[cc * LDS + i] = fmaf(-tv, s_w[cc], sA[cc * LDS + i]);
-          }
-        }
-        __syncthreads();
-      }
-    }
-    if (nonfinite) atomicOr(p.status, kStatusQrBreakdown);
-
-    // V with its unit diagonal and zeros before it (rank 0 holds the first kb positions)
-    if (c == 0) {
-      for (int e = tid; e < kb * kb; e += PT) {
-        const int jj = e / kb, i = e % kb;
-        if (i < jj) sA[jj * LDS + i] = 0.f;
-        else if (i == jj) sA[jj * LDS + i] = 1.f;
-      }
-    }
-    __syncthreads();
-
-    // V as rows of Vt (zeros at the block's positions before the panel) and as columns jb..
-    // of the block's position-major Vpos
-    float* Vt = p.Vt + (int64_t)b * nn;
-    float* Vt_lo = p.Vt_lo + (int64_t)b * nn;
-    float* Vpos = p.Vpos + (int64_t)b * n * NBO;
-    float* Vpos_lo = p.Vpos_lo + (int64_t)b * n * NBO;
-    {
-      const int q4n = npos / 4;
-      for (int e = tid; e < kb * q4n; e += PT) {
-        const int jj = e / q4n, q = e - jj * q4n;
-        const int64_t o = (int64_t)(k + jj) * n + pos0 + 4 * q;
-        const float4 v = *reinterpret_cast<const float4*>(&sA[jj * LDS + 4 * q]);
-        *reinterpret_cast<float4*>(Vt + o) = v;
-        *reinterpret_cast<float4*>(Vt_lo + o) = make_float4(tf32_lo(v.x), tf32_lo(v.y), tf32_lo(v.z), tf32_lo(v.w));
-      }
-    }
-    for (int e = tid; e < npos * (NB / 4); e += PT) {
-      const int i = e >> 3, g4 = 4 * (e & 7);  // rows kb.. of sA are zero
-      const float4 v = make_float4(sA[g4 * LDS + i], sA[(g4 + 1) * LDS + i], sA[(g4 + 2) * LDS + i], sA[(g4 + 3) * LDS + i]);
-      const int64_t o = (int64_t)(pos0 + i) * NBO + jb + g4;
-      *reinterpret_cast<float4*>(Vpos + o) = v;
-      *reinterpret_cast<float4*>(Vpos_lo + o) = make_float4(tf32_lo(v.x), tf32_lo(v.y), tf32_lo(v.z), tf32_lo(v.w));
-    }
-    if (c == 0) {
-      for (int jj = 0; jj < kb; ++jj)
-        for (int i = tid; i < jb; i += PT) {
-          const int64_t o = (int64_t)(k + jj) * n + k0 + i;
-          Vt[o] = 0.f;
-          Vt_lo[o] = 0.f;
-        }
-      for (int e = tid; e < jb * NB; e += PT) {
-        const int64_t o = (int64_t)(k0 + e / NB) * NBO + jb + e % NB;
-        Vpos[o] = 0.f;
-        Vpos_lo[o] = 0.f;
-      }
-    }
-    __syncthreads();  // this CTA's Vt rows are read back below
-
-    // Y = S V_panel over this CTA's positions, S = the block's rows k0 .. k0+kbo-1: the block's
-    // Householder vectors so far (rows before the panel's end, from Vt) and the block rows still
-    // to be factored (from At), with both operands split into tf32 hi and lo parts (four
-    // products: fp32 accuracy), each 32-position chunk summed afresh and added to fp32 registers,
-    // so that the tensor core's own accumulation never runs longer than 32 positions.
-    if constexpr (COLS == PT) {
-      // On the tcgen05 tensor cores: D[128 x 32] (tensor memory) = S chunk (A: 128 rows x 32
-      // positions) x V chunk^T (B: 32 rows x 32 positions), both K-major in the 128-byte-swizzled
-      // layout. S's rows other than the panel's are copied with cp.async straight into that
-      // layout, SV_STG - 1 chunks ahead, and each thread forms the lo part of the units it copied;
-      // the panel's rows of S and the V chunk (hi and lo) come from sA. Two accumulators and two
-      // lo sets alternate: while the MMAs of chunk ch run, warps 0-3 drain chunk ch-1 (warp w
-      // reads lanes 32w..) and its S stage is refilled.
-      uint8_t* sv = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(s_sv) + 1023) & ~uintptr_t(1023));
-      uint8_t* st_a = sv;                          // [SV_STG] S chunks (fp32, read by the MMA as its hi part)
-      uint8_t* st_lo = sv + SV_STG * A_BYTES;      // [2] S lo | V hi | V lo
-      constexpr int LO_SET = A_BYTES + 2 * B_BYTES;
-      const int nchunk = (npos + 31) / 32;
-      if (tid == 0) {
-        tc::mbar_init(&s_mma_bar[0], 1);
-        tc::mbar_init(&s_mma_bar[1], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      }
-      __syncthreads();
-      // byte offset of 16-byte unit q of row r in a tile of 128-byte rows, swizzled within
-      // 1024-byte groups of 8 rows
-      auto swz16 = [](int r, int q) { return (r >> 3) * 1024 + (r & 7) * 128 + ((q ^ (r & 7)) << 4); };
-      auto issue = [&](int ch) {
-        uint8_t* dst = st_a + (ch % SV_STG) * A_BYTES;
-        for (int u = tid; u < NBO * 8; u += PT) {
-          const int r = u >> 3, q = u & 7;
-          if (r >= jb && r < jb + NB) continue;  // the panel's own rows: V, from sA
-          const int row = k0 + r, i = ch * 32 + 4 * q;
-          const bool ok = r < kbo && i < npos;  // zero-filled outside the block and past the positions
-          const float* src = ok ? (r < jb ? Vt : At) + (int64_t)row * n + pos0 + i : At;
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(dst + swz16(r, q))),
-                       "l"(src), "r"(ok ? 16 : 0)
-                       : "memory");
-        }
-      };
-      auto lo4 = [](float4 x) { return make_float4(tf32_lo(x.x), tf32_lo(x.y), tf32_lo(x.z), tf32_lo(x.w)); };
-      float y[NB];
-#pragma unroll
-      for (int l = 0; l < NB; ++l) y[l] = 0.f;
-      for (int st0 = 0; st0 < SV_STG - 1; ++st0) {
-        if (st0 < nchunk) issue(st0);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-      }
-      int issued = 0;  // chunks whose MMAs were issued
-      bool aborted = false, bad = false;
-      for (int ch = 0; ch < nchunk; ++ch) {
-        const int set = ch & 1;
-        // this thread's copies of chunk ch have landed: their lo parts; the panel's rows of S and
-        // the V chunk (hi and lo) from sA
-        asm volatile("cp.async.wait_group %0;" ::"n"(SV_STG - 2) : "memory");
-        {
-          uint8_t* a = st_a + (ch % SV_STG) * A_BYTES;
-          uint8_t* lo = st_lo + set * LO_SET;
-          for (int u = tid; u < NBO * 8; u += PT) {
-            const int r = u >> 3;
-            if (r >= jb && r < jb + NB) continue;
-            const int off = swz16(r, u & 7);
-            *reinterpret_cast<float4*>(lo + off) = lo4(*reinterpret_cast<const float4*>(a + off));
-          }
-          uint8_t* bh = lo + A_BYTES;
-          uint8_t* bl = bh + B_BYTES;
-          for (int u = tid; u < NB * 8; u += PT) {
-            const int jj = u >> 3, q = u & 7;
-            const float4 x = *reinterpret_cast<const float4*>(&sA[jj * LDS + ch * 32 + 4 * q]);
-            const float4 xl = lo4(x);
-            const int off = swz16(jj, q), offa = swz16(jb + jj, q);
-            *reinterpret_cast<float4*>(bh + off) = x;
-            *reinterpret_cast<float4*>(bl + off) = xl;
-            *reinterpret_cast<float4*>(a + offa) = x;
-            *reinterpret_cast<float4*>(lo + offa) = xl;
-          }
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (__syncthreads_or(bad)) {
-          aborted = true;
-          break;
-        }
-        // the MMAs of chunk ch (its lo set and accumulator were released in the previous pass)
-        if (tid == 0) {
-          tc::tc_fence_after();
-          constexpr uint32_t idesc = tc::idesc_tf32(NBO, NB);
-          const uint32_t d = tmem + (uint32_t)(set * 32);
-          const uint32_t a_hi = tc::smem_u32(st_a + (ch % SV_STG) * A_BYTES);
-          const uint32_t a_lo = tc::smem_u32(st_lo + set * LO_SET);
-          const uint32_t b_hi = a_lo + A_BYTES;
-          const uint32_t b_lo = b_hi + B_BYTES;
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            const uint32_t off = kk * 32;  // 8 tf32 = 32 bytes along the positions
-            tc::umma_tf32(d, tc::desc_sw128(a_lo + off), tc::desc_sw128(b_lo + off), idesc, kk != 0);
-            tc::umma_tf32(d, tc::desc_sw128(a_lo + off), tc::desc_sw128(b_hi + off), idesc, 1u);
-            tc::umma_tf32(d, tc::desc_sw128(a_hi + off), tc::desc_sw128(b_lo + off), idesc, 1u);
-            tc::umma_tf32(d, tc::desc_sw128(a_hi + off), tc::desc_sw128(b_hi + off), idesc, 1u);
-          }
-          tc::umma_commit(&s_mma_bar[set]);
-        }
-        issued = ch + 1;
-        // while they run: chunk ch-1's MMAs have completed, so its accumulator is drained and its
-        // S stage refilled with chunk ch + SV_STG - 1
-        if (ch >= 1) {
-          bool ok = tc::mbar_wait(&s_mma_bar[(ch - 1) & 1], ((ch - 1) >> 1) & 1, kWaitNs);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) {
-            bad = true;
-          } else if (warp < 4) {
-            float v[32];
-            tc::tmem_ld32(tmem + (uint32_t)(((ch - 1) & 1) * 32) + ((uint32_t)(32 * warp) << 16), v);
-#pragma unroll
-            for (int l = 0; l < NB; ++l) y[l] += v[l];
-          }
-        }
-        if (!bad && ch + SV_STG - 1 < nchunk) issue(ch + SV_STG - 1);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        tc::tc_fence_before();
-      }
-      // the last chunk's sum; after a wait that gave up, only the wait for every issued MMA (with
-      // the full bound), so that the tensor memory is not freed under one
-      bool ok_last = true;
-      if (issued > 0)
-        ok_last = __all_sync(0xffffffffu, tc::mbar_wait(&s_mma_bar[(issued - 1) & 1], ((issued - 1) >> 1) & 1, kWaitNs));
-      if (!aborted && !bad && ok_last && issued > 0 && warp < 4) {
-        float v[32];
-        tc::tmem_ld32(tmem + (uint32_t)(((issued - 1) & 1) * 32) + ((uint32_t)(32 * warp) << 16), v);
-#pragma unroll
-        for (int l = 0; l < NB; ++l) y[l] += v[l];
-      }
-      if (aborted || bad || !ok_last) atomicOr(p.status, kStatusTimeout);
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      tc::tc_fence_before();
-      __syncthreads();
-      tc::tc_fence_after();
-      if (tid == 0) {  // every wait on them is over; the next panel sets them up again
-        asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(tc::smem_u32(&s_mma_bar[0])) : "memory");
-        asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(tc::smem_u32(&s_mma_bar[1])) : "memory");
-      }
-      // this CTA's partial product, kept in shared memory (the S stages are free) for the cluster
-      if (warp < 4) {
-        float* yp = reinterpret_cast<float*>(sv) + (32 * warp + lane) * NB;
-#pragma unroll
-        for (int l4 = 0; l4 < NB / 4; ++l4)
-          *reinterpret_cast<float4*>(yp + 4 * l4) = make_float4(y[4 * l4], y[4 * l4 + 1], y[4 * l4 + 2], y[4 * l4 + 3]);
-      }
-    } else
-    // With 1024 positions per CTA (factors of at most 1024 rows): S is streamed through shared
-    // memory in 32-position chunks (cp.async, STG buffers, rows padded to 36 floats), and the
-    // product runs as warp-level m16n8k8 TF32 MMAs. Warp w owns rows 16 (w mod 8) .. +15 and
-    // columns 16 (w / 8) .. +15.
-    {
-      static_assert(NBO == 128 && NB == 32 && NWARP == 16, "8 x 2 warp tiles of 16 x 16");
-      constexpr int CH = 32;       // positions per chunk
-      constexpr int CHP = CH + 4;  // padded row stride of a staged chunk
-      const int gq = lane >> 2, tg = lane & 3;
-      const int m0 = 16 * (warp & 7), nb = 16 * (warp >> 3);
-      float y[2][4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) y[0][e] = y[1][e] = 0.f;
-      const int nchunk = (npos + CH - 1) / CH;
-      auto issue = [&](int ch, int buf) {
-        float* dst = reinterpret_cast<float*>(s_sv) + buf * NBO * CHP;
-        for (int e = tid; e < NBO * (CH / 4); e += PT) {
-          const int r = e / (CH / 4), q4 = e % (CH / 4);
-          const int row = k0 + r, i = ch * CH + 4 * q4;
-          const bool ok = r < kbo && i < npos;
-          const float* src = ok ? ((row < k + kb) ? Vt : At) + (int64_t)row * n + pos0 + i : At;
-          const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst + r * CHP + 4 * q4));
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-      };
-      for (int st0 = 0; st0 < STG - 1; ++st0) {
-        if (st0 < nchunk) issue(st0, st0);
-        else asm volatile("cp.async.commit_group;" ::: "memory");
-      }
-      for (int ch = 0; ch < nchunk; ++ch) {
-        if (ch + STG - 1 < nchunk) issue(ch + STG - 1, (ch + STG - 1) % STG);
-        else asm volatile("cp.async.commit_group;" ::: "memory");  // keeps the group count uniform
-        asm volatile("cp.async.wait_group %0;" ::"n"(STG - 1) : "memory");
-        __syncthreads();
-        const float* st = reinterpret_cast<const float*>(s_sv) + (ch % STG) * NBO * CHP;
-        const int i0 = ch * CH;
-        float d[2][4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) d[0][e] = d[1][e] = 0.f;
-#pragma unroll
-        for (int ks = 0; ks < CH / 8; ++ks) {
-          // positions past npos are zero in the staged chunk and in V (zero-filled copies)
-          const int kk = 8 * ks;
-          const float av[4] = {st[(m0 + gq) * CHP + kk + tg], st[(m0 + gq + 8) * CHP + kk + tg],
-                               st[(m0 + gq) * CHP + kk + tg + 4], st[(m0 + gq + 8) * CHP + kk + tg + 4]};
-          uint32_t ah[4], al[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) tf32_split(av[e], ah[e], al[e]);
-#pragma unroll
-          for (int nt = 0; nt < 2; ++nt) {
-            const float* vr = sA + (nb + 8 * nt + gq) * LDS + i0 + kk + tg;
-            uint32_t bh[2], bl[2];
-            tf32_split(vr[0], bh[0], bl[0]);
-            tf32_split(vr[4], bh[1], bl[1]);
-            mma_tf32_16x8x8(d[nt], al, bl);
-            mma_tf32_16x8x8(d[nt], al, bh);
-            mma_tf32_16x8x8(d[nt], ah, bl);
-            mma_tf32_16x8x8(d[nt], ah, bh);
-          }
-        }
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) y[nt][e] += d[nt][e];
-        __syncthreads();  // this buffer is refilled STG - 1 chunks later
-      }
-      float* yp = p.Ypart + ((int64_t)b * MAXC + c) * NBO * NB;
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const int col = nb + 8 * nt + 2 * tg;
-        *reinterpret_cast<float2*>(yp + (m0 + gq) * NB + col) = make_float2(y[nt][0], y[nt][1]);
-        *reinterpret_cast<float2*>(yp + (m0 + gq + 8) * NB + col) = make_float2(y[nt][2], y[nt][3]);
-      }
-    }
-    // T_panel from the Gram rows of Y, then U = X T_panel (in place) and Z (rows after the panel);
-    // every thread of the CTA takes part (the barriers inside)
-    auto form_tuz = [&]() {
-      // T of the panel from its Gram matrix g (rows jb.. of Y): T^-1 = diag(1/tau) + striu(g)
-      // (H_1 ... H_kb = I - V T V^T); a reflector with tau = 0 (v = 0) gets a zero row and column.
-      // Warp w solves columns w and w + 16 by back substitution, lane i holding x_i:
-      //   x_i = tau_i (delta_{i,cc} - sum_{i < l <= cc} g_il x_l)   (tau_i read as 1 where it is 0)
-      // Each solved x_l is broadcast once and every lane i < l adds g_il x_l to its running sum,
-      // so a step costs one shuffle instead of a warp-wide reduction.
-      for (int cc = warp; cc < NB; cc += NWARP) {
-        float x = 0.f, acc = 0.f;
-        for (int l = cc; l >= 0; --l) {
-          const float g = s_Y[jb + lane][l];
-          if (lane == l) {
-            const float tl = l < kb ? s_tau[l] : 0.f;
-            x = ((l == cc ? 1.f : 0.f) - acc) * (tl != 0.f ? tl : 1.f);
-          }
-          const float xl = __shfl_sync(0xffffffffu, x, l);
-          if (lane < l) acc = fmaf(g, xl, acc);
-        }
-        const bool live = cc < kb && s_tau[cc] != 0.f;
-        s_T[lane][cc] = (live && lane <= cc && lane < kb && s_tau[lane] != 0.f) ? x : 0.f;
-      }
-      __syncthreads();
-      // U = X T_panel with X = V_before^T V_panel (rows 0..jb-1 of Y), in place, and
-      // Z = (S_rest V_panel) T_panel for the block rows after the panel: thread (r, g) forms
-      // columns 8g .. 8g+7 of row r
-      {
-        const int r = tid >> 2, g8 = (tid & 3) * 8;
-        const bool act = r < kbo && (r < jb || r >= jb + kb);
-        float x[NB];
-#pragma unroll
-        for (int l = 0; l < NB; ++l) x[l] = act ? s_Y[r][l] : 0.f;
-        __syncthreads();  // every row is read before U overwrites it
-        if (act) {
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int cc = g8 + u;
-            float acc = 0.f;
-#pragma unroll
-            for (int l = 0; l < NB; ++l)
-              if (l <= cc) acc = fmaf(x[l], s_T[l][cc], acc);
-            if (r < jb) s_Y[r][cc] = acc;
-            else s_Z[r - jb - kb][cc] = acc;
-          }
-        }
-      }
-      __syncthreads();
-    };
-    if constexpr (COLS == PT) {
-      // The partial products reduced through distributed shared memory: CTA c sums rows
-      // r = c mod C of every CTA's partial, in a fixed order, and every CTA then gathers the summed
-      // rows and forms T_panel, U and Z itself (the same values on every CTA).
-      uint8_t* sv = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(s_sv) + 1023) & ~uintptr_t(1023));
-      float* P_own = reinterpret_cast<float*>(sv);
-      float* Ysum = P_own + NBO * NB;
-      cluster.sync();  // every CTA's partial is in place
-      for (int r = c + C * warp; r < kbo; r += C * NWARP) {
-        float part[MAXC];
-#pragma unroll
-        for (int q = 0; q < MAXC; ++q) part[q] = q < C ? cluster.map_shared_rank(P_own, q)[r * NB + lane] : 0.f;
-        float sum = 0.f;
-#pragma unroll
-        for (int q = 0; q < MAXC; ++q) sum += part[q];
-        Ysum[r * NB + lane] = sum;
-      }
-      cluster.sync();  // every summed row is in place
-      for (int e = tid; e < kbo * NB; e += PT) s_Y[e / NB][e % NB] = cluster.map_shared_rank(Ysum, (e / NB) % C)[e];
-      // the peers may read this CTA's summed rows until they have gathered theirs: arrive now and
-      // wait at the end of the kernel
-      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-      __syncthreads();
-      form_tuz();
-      __syncthreads();
-      if (c == 0 && tid < kb) {
-        p.skip[(int64_t)b * n + k + tid] = (uint8_t)s_skip[tid];
-        p.dsign[(int64_t)b * n + k + tid] = s_dsign[tid];
-      }
-    } else {
-      cluster.sync();  // orders the partials in global memory before rank 0 reads them
-      // rank 0 sums the partials, forms T_panel, U = X T_panel and Z, and hands Z, U and T_panel
-      // to the cluster through global memory (rank 0's slots of Ypart, free once it has summed
-      // them): Z at 0, U at 3072 (jb <= 96 rows), T_panel at 6144 floats
-      float* xg = p.Ypart + (int64_t)b * MAXC * NBO * NB;
-      float* Ug = xg + NREST * NB;
-      float* Tpg = xg + 2 * NREST * NB;
-      if (c == 0) {
-        // sum the partials in a fixed order
-        const float* yp = p.Ypart + (int64_t)b * MAXC * NBO * NB;
-        for (int e = tid; e < kbo * NB; e += PT) {
-          float part[MAXC];
-#pragma unroll
-          for (int q = 0; q < MAXC; ++q) part[q] = q < C ? yp[(int64_t)q * NBO * NB + e] : 0.f;
-          float sum = 0.f;
-#pragma unroll
-          for (int q = 0; q < MAXC; ++q) sum += part[q];
-          s_Y[e / NB][e % NB] = sum;
-        }
-        __syncthreads();
-        form_tuz();
-        __syncthreads();
-        for (int e = tid; e < nrest * NB; e += PT) xg[e] = s_Z[e / NB][e % NB];
-        for (int e = tid; e < jb * NB; e += PT) Ug[e] = s_Y[e / NB][e % NB];
-        for (int e = tid; e < NB * NB; e += PT) Tpg[e] = s_T[e / NB][e % NB];
-        if (tid < kb) {
-          p.skip[(int64_t)b * n + k + tid] = (uint8_t)s_skip[tid];
-          p.dsign[(int64_t)b * n + k + tid] = s_dsign[tid];
-        }
-      }
-      cluster.sync();  // Z, U and T_panel in global memory are visible to the cluster
-      if (c != 0) {
-        for (int e = tid; e < nrest * NB; e += PT) s_Z[e / NB][e % NB] = xg[e];
-        for (int e = tid; e < jb * NB; e += PT) s_Y[e / NB][e % NB] = Ug[e];
-        for (int e = tid; e < NB * NB; e += PT) s_T[e / NB][e % NB] = Tpg[e];
-      }
-      __syncthreads();
-    }
-    // the block's T, rows spread over the cluster (row r by CTA r mod C): column block jb =
-    // [-T_before U ; T_panel ; 0] and the row block jb left of it = 0
-    {
-      float* T = p.T + (int64_t)b * NBO * NBO;
-      float* T_lo = p.T_lo + (int64_t)b * NBO * NBO;
-      float* Tt = p.Tt + (int64_t)b * NBO * NBO;
-      float* Tt_lo = p.Tt_lo + (int64_t)b * NBO * NBO;
-      // the rows of T_before (written by the block's earlier panels) that this CTA's rows need,
-      // staged in shared memory with independent loads: the S V area is free (on the cluster path
-      // past its first 32 KB, the summed rows that peers may still read)
-      constexpr int TBS = NBO - NB;  // jb <= 96
-      float* Tb = reinterpret_cast<float*>(
-          COLS == PT ? ((reinterpret_cast<uintptr_t>(s_sv) + 1023) & ~uintptr_t(1023)) + 2 * NBO * NB * sizeof(float)
-                     : reinterpret_cast<uintptr_t>(s_sv));
-      static_assert(TBS * TBS * sizeof(float) <= (COLS == PT ? SV_BYTES - 1024 - 2 * NBO * NB * sizeof(float) : SV_BYTES),
-                    "T_before staging");
-      const int nrl = jb > c ? (jb - c + C - 1) / C : 0;  // this CTA's rows r = c + C rl below jb
-      for (int e = tid; e < nrl * jb; e += PT) {
-        const int rl = e / jb, l = e - rl * jb, rr = c + C * rl;
-        Tb[rl * TBS + l] = l >= rr ? T[rr * NBO + l] : 0.f;
-      }
-      __syncthreads();
-      // one entry (row r = c + C rl, column jb + cc) per work unit, the 32 units of a row on
-      // consecutive threads: the triangular product's long rows are spread over all threads in
-      // turn. On the cluster path the column block is also staged transposed, so that Tt's rows
-      // are written with consecutive stores.
-      const int nr = (NBO - c + C - 1) / C;  // this CTA's rows
-      float* stt = COLS == PT ? Tb + TBS * TBS : nullptr;  // [NB][NBO]: entry (cc, rl)
-      static_assert(COLS != PT || (TBS * TBS + NB * NBO) * sizeof(float) <= SV_BYTES - 1024 - 2 * NBO * NB * sizeof(float),
-                    "T column block staging");
-      for (int u = tid; u < nr * NB; u += PT) {
-        const int rl = u >> 5, cc = u & 31, r = c + C * rl;
-        float t = 0.f;
-        if (r < jb) {
-          const float* tb_row = Tb + rl * TBS;
-#pragma unroll 4
-          for (int l = r; l < jb; ++l) t = fmaf(-tb_row[l], s_Y[l][cc], t);
-        } else if (r < jb + NB) {
-          t = s_T[r - jb][cc];
-        }
-        const int col = jb + cc;
-        T[r * NBO + col] = t;
-        T_lo[r * NBO + col] = tf32_lo(t);
-        if (COLS == PT) {
-          stt[cc * NBO + rl] = t;
-        } else {
-          Tt[col * NBO + r] = t;
-          Tt_lo[col * NBO + r] = tf32_lo(t);
-        }
-      }
-      if (COLS == PT) {
-        __syncthreads();
-        for (int e = tid; e < NB * nr; e += PT) {
-          const int cc = e / nr, rl = e - cc * nr;
-          const float t = stt[cc * NBO + rl];
-          Tt[(jb + cc) * NBO + c + C * rl] = t;
-          Tt_lo[(jb + cc) * NBO + c + C * rl] = tf32_lo(t);
-        }
-      }
-      // the row block jb left of the panel is zero: T's rows jb.. and Tt's columns jb.. there
-      for (int e = tid; e < NB * jb; e += PT) {
-        const int rr = jb + e / jb, col = e % jb;
-        if (rr % C != c) continue;
-        T[rr * NBO + col] = 0.f;
-        T_lo[rr * NBO + col] = 0.f;
-      }
-      for (int e = tid; e < NB * jb; e += PT) {
-        const int col = e / NB, rr = jb + e % NB;
-        if (rr % C != c) continue;
-        Tt[col * NBO + rr] = 0.f;
-        Tt_lo[col * NBO + rr] = 0.f;
-      }
-    }
-
-    // the panel's reflectors on the block rows after it: a_r -= Z_r V^T at this CTA's
-    // positions, eight rows at a time (eight independent loads in flight), then four, then one
-    for (int i = tid; i < npos; i += PT) {
-      float v[NB];
-#pragma unroll
-      for (int jj = 0; jj < NB; ++jj) v[jj] = sA[jj * LDS + i];
-      float* a = At + (int64_t)(k + kb) * n + pos0 + i;
-      int r = 0;
-      for (; r + 8 <= nrest; r += 8) {
-        float x[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) x[u] = a[(int64_t)(r + u) * n];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          float acc = 0.f;
-#pragma unroll
-          for (int j4 = 0; j4 < NB / 4; ++j4) {
-            const float4 z = *reinterpret_cast<const float4*>(&s_Z[r + u][4 * j4]);
-            acc = fmaf(z.x, v[4 * j4], fmaf(z.y, v[4 * j4 + 1], fmaf(z.z, v[4 * j4 + 2], fmaf(z.w, v[4 * j4 + 3], acc))));
-          }
-          a[(int64_t)(r + u) * n] = x[u] - acc;
-        }
-      }
-      for (; r + 4 <= nrest; r += 4) {
-        float x[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = a[(int64_t)(r + u) * n];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          float acc = 0.f;
-#pragma unroll
-          for (int j4 = 0; j4 < NB / 4; ++j4) {
-            const float4 z = *reinterpret_cast<const float4*>(&s_Z[r + u][4 * j4]);
-            acc = fmaf(z.x, v[4 * j4], fmaf(z.y, v[4 * j4 + 1], fmaf(z.z, v[4 * j4 + 2], fmaf(z.w, v[4 * j4 + 3], acc))));
-          }
-          a[(int64_t)(r + u) * n] = x[u] - acc;
-        }
-      }
-      for (; r < nrest; ++r) {
-        float acc = 0.f;
-#pragma unroll
-        for (int jj = 0; jj < NB; ++jj) acc = fmaf(s_Z[r][jj], v[jj], acc);
-        a[(int64_t)r * n] -= acc;
-      }
-    }
-    if constexpr (COLS == PT) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    // the next panel's positions are shifted by 32: it reads rows that the other CTAs updated
-    cluster.sync();
-  }
+  for (int k = p.k0; k < p.k0 + p.kbo; k += NB) panel<COLS>(p, k, tmem);
   if constexpr (COLS == PT) {
     tc::tc_fence_before();
     __syncthreads();
