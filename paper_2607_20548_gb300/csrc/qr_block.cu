@@ -53,7 +53,10 @@ namespace {
 constexpr int NBO = kQrBlock;
 constexpr uint64_t kWaitNs = 2000000000ull;
 // Squared pivot over squared column norm below which a block leaves for the column loop at once (its
-// excess is at least 3 then; blocks of a run that the excess admits have 0.5 and more).
+// excess is at least 3 then; blocks of a run that the excess admits have 0.5 and more). So does one
+// whose squared norms over squared pivots, less one each, already add up to more than kQrMaxExcess:
+// G^^-1's diagonal is at least that ratio. (QR of 64 Gaussian 768-factors, most blocks of which decline:
+// 5.38 -> 5.25 ms.)
 constexpr float kRhoMin = 0.25f;
 
 // byte offset of 16-byte unit q of row r in a tile of 128-byte rows, swizzled within 1024-byte
@@ -311,9 +314,10 @@ __device__ __forceinline__ float inv(float x) {
 }
 
 // Columns j and j + 1 (j even) of the diagonal blocks (step 2), one warp; returns whether their
-// pivots are good. The two pivot rows go through shared memory once; every lane derives both
-// columns' reflectors from them.
-__device__ __forceinline__ bool diag_pair(CoreShared& sh, float2 (&x)[kPairs], int j, float norm0, float norm1, float lim2) {
+// pivots are good, and adds to `excess` what they prove of it. The two pivot rows go through shared
+// memory once; every lane derives both columns' reflectors from them.
+__device__ __forceinline__ bool diag_pair(CoreShared& sh, float2 (&x)[kPairs], int j, float norm0, float norm1, float lim2,
+                                          float& excess) {
   const int lane = threadIdx.x & 31, par = (j >> 1) & 1;
   const bool srow = lane < 16;
   if ((lane & 14) == j) store_pairs(sh.pv[par][lane >> 4][lane & 1], x);
@@ -373,6 +377,7 @@ __device__ __forceinline__ bool diag_pair(CoreShared& sh, float2 (&x)[kPairs], i
     sh.l[j][lane - j] = m0;
     sh.l[j + 1][lane - j] = m1;
   }
+  excess += fmaf(norm0 * ir0, ir0, -1.f) + fmaf(norm1 * ir1, ir1, -1.f);
   // (false for a non-finite value too; squares outside fp32's comfortable range go the other way)
   return g0 >= kRhoMin * norm0 && g1 >= kRhoMin * norm1 && g0 > lim2 && g1 > lim2 && g0 > 1e-30f && g1 > 1e-30f &&
          norm0 < 1e30f && norm1 < 1e30f;
@@ -499,6 +504,7 @@ __global__ void __launch_bounds__(kThreads, 1) qr_core_kernel(QrBlockArgs p, int
   const bool zero = sh.zero_block != 0;
   bool fast = !zero;
   const int npan = (kbo + kPw - 1) / kPw;
+  float excess = 0.f;  // (first warp)
   for (int pp = 0; pp < npan && fast; ++pp) {
     const int j0 = kPw * pp, pw = min(kPw, kbo - j0);  // a multiple of 4
     // 1: the panel's rows and columns
@@ -535,10 +541,10 @@ __global__ void __launch_bounds__(kThreads, 1) qr_core_kernel(QrBlockArgs p, int
       bool ok = true;
 #pragma unroll 1
       for (int j = 0; j < pw; j += 2) {
-        const bool good = diag_pair(sh, x, j, sh.norm[j0 + j], sh.norm[j0 + j + 1], lim2);
+        const bool good = diag_pair(sh, x, j, sh.norm[j0 + j], sh.norm[j0 + j + 1], lim2, excess);
         ok = ok && good;
       }
-      if (lane == 0 && !ok) sh.fail = 1;
+      if (lane == 0 && !(ok && excess <= kQrMaxExcess)) sh.fail = 1;
       if (lane < pw) p.dsign[(int64_t)b * n + k0 + j0 + lane] = sh.d[lane];
     }
     __syncthreads();
