@@ -1185,16 +1185,15 @@ soap_status_t state_get_impl(soap_handle h, int32_t idx, int32_t which, void* ds
     if (c.right) SOAP_CUDA(h, soap::planes_transpose(v.QR, soap::Planes(), v.QRt, nullptr, nc, 1, s));
     SOAP_CUDA(h, soap::split_planes(x, v.Mc, c.tr ? nc : m, c.tr ? m : nc, s));
     if (!(c.left && c.right)) {
-      // the step's product [X | M_hat] Q for this matrix alone (bit-identical), written in the
-      // original orientation
+      // the step's product [X | M_hat] Q for this matrix alone, written in the original orientation
       const int rr = c.tr ? nc : m, cc = c.tr ? m : nc;
       SOAP_CUDA(h, soap::gemm_b3(rr, cc, cc, 1, b3_op(v.Mc, 1), b3_op(c.tr ? v.QLt : v.QRt, 1),
                                  epi(h, h->Gp, c.tr ? rr : cc, mn, c.tr ? 1 : 0, 1.f, 0.f), s));
       SOAP_CUDA(h, cudaMemcpyAsync(dst, h->Gp, bytes, cudaMemcpyDefault, s));
       return SOAP_OK;
     }
-    // the same tensor-core products, on the same operands, as the step's rotation of M_hat:
-    // bit-identical to the m the last step used
+    // the same products of the same operands as the step's rotation of M_hat (which may have run on
+    // other tiles: those are chosen by the size of the whole batch)
     const soap::Planes Yt = soap::planes_in(h->YMt, nc, m, 1);
     SOAP_CUDA(h, soap::gemm_b3(m, nc, nc, 1, b3_op(v.Mc, 1), b3_op(v.QRt, 1), epi(h, Yt, 1), s));
     SOAP_CUDA(h, soap::gemm_b3(m, nc, m, 1, b3_op(v.QLt, 1), b3_op(Yt, 1), epi(h, h->Gp, nc, mn, 0, 1.f, 0.f), s));
