@@ -86,7 +86,7 @@ struct PanelArgs {
   float* Tt;           // [batch][NBO][NBO] T^T
   float* Tt_lo;
   float* Ypart;        // [batch][MAXC][NBO][NB] per-CTA partial products S V_panel (at first the
-                       // Gram matrices' place, which qr_block_left reads before any is written)
+                       // Gram matrices' place, which block_left reads before any is written)
   uint8_t* skip;       // [batch][n]
   float* dsign;        // [batch][n] sign of R_pp (+1 for zero columns)
   const float* thresh; // [batch]
@@ -938,13 +938,64 @@ __device__ __noinline__ void panel(const PanelArgs& p, int k, uint32_t tmem) {
   cluster.sync();
 }
 
+// Whether the column loop has to factor this matrix's block (also where a value is not finite). The
+// trace decides in nearly every case; where it is not close enough, ||G^^-1||_F^2 = ||X X^T||_F^2 with X
+// from qr_block_inverse takes a few us (the column loop 440 a block): warp w has the rows w + 16 r, lane l
+// the columns l + 32 c on and above the diagonal, and X is zero before its diagonal. By the trace alone
+// the 24-layer stack's first steps took 2553 ms, 2352 with this.
+constexpr int kInvLd = NBO + 4;
+constexpr int kInvSmem = NBO * kInvLd * 4;
+__device__ __forceinline__ bool block_left(const PanelArgs& p, int b, float* sm) {
+  const int state = p.state[b];
+  const float excess = qr_block_excess(p.Ypart, b, p.kbo);
+  if (state != kQrBlockFast) return state == kQrBlockColumns;
+  if (excess <= kQrMaxExcess) return false;
+  __shared__ float s_sum[NWARP];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float* X = qr_block_inverse(p.Ypart, b);
+  for (int e = tid; e < NBO * NBO / 4; e += PT)
+    *reinterpret_cast<float4*>(sm + (e >> 5) * kInvLd + 4 * (e & 31)) = reinterpret_cast<const float4*>(X)[e];
+  __syncthreads();
+  float sum = 0.f;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    float acc[8];
+#pragma unroll
+    for (int r = 0; r < 2 * c + 2; ++r) acc[r] = 0.f;
+#pragma unroll 2
+    for (int k = 32 * c; k < NBO; k += 4) {
+      const float4 y = *reinterpret_cast<const float4*>(sm + (lane + 32 * c) * kInvLd + k);
+#pragma unroll
+      for (int r = 0; r < 2 * c + 2; ++r) {
+        const float4 x = *reinterpret_cast<const float4*>(sm + (warp + 16 * r) * kInvLd + k);
+        acc[r] = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, acc[r]))));
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 2 * c + 2; ++r) {
+      const int i = warp + 16 * r, j = lane + 32 * c;
+      sum = fmaf(j > i ? 2.f : j == i ? 1.f : 0.f, acc[r] * acc[r], sum);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (lane == 0) s_sum[warp] = sum;
+  __syncthreads();
+  float norm2 = 0.f;
+#pragma unroll
+  for (int w = 0; w < NWARP; ++w) norm2 += s_sum[w];
+  return !(norm2 <= kQrMaxInverse * kQrMaxInverse);
+}
+
 // The block's panels one after another, for a matrix whose block was not factored from its Gram matrix.
 // One launch per block, so that a block that was costs one launch that returns at once (four, or eight
 // with the column loop as a kernel of its own, cost 14-20 us).
 template <int COLS>
 __global__ void __launch_bounds__(PT, 1) qr_panel_kernel(const __grid_constant__ PanelArgs p) {
   const int b = blockIdx.y, warp = threadIdx.x >> 5;
-  if (!qr_block_left(p.state[b], p.Ypart, b, p.kbo)) return;  // factored without the column loop
+  extern __shared__ float4 smem_dyn[];
+  if (!block_left(p, b, reinterpret_cast<float*>(smem_dyn))) return;  // factored without the column loop
+  __syncthreads();
 
   __shared__ uint32_t s_tmem;
   uint32_t tmem = 0;
@@ -1044,7 +1095,7 @@ template <int COLS>
 cudaError_t prepare_panel(PanelKernel* pk, bool wide) {
   pk->fn = qr_panel_kernel<COLS>;
   pk->cols = COLS;
-  pk->smem = (size_t)NB * (COLS + 4) * sizeof(float);
+  pk->smem = std::max<size_t>((size_t)NB * (COLS + 4) * sizeof(float), kInvSmem);
   cudaError_t e = cudaFuncSetAttribute(pk->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pk->smem);
   if (e == cudaSuccess && wide) e = cudaFuncSetAttribute(pk->fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   return e;

@@ -21,13 +21,15 @@
 // not bound that norm (with every squared pivot at 0.4 of its column's squared norm it can exceed
 // 1e10). Its trace does: the eigenvalues of G^ add up to kbo, so that
 //   ||G^^-1|| <= tr(G^^-1) - kbo + 2,   tr(G^^-1) = sum_i G_ii ||row i of R^-1||^2,
-// and the kernel that forms T's rows solves for R^-1's beside them. The block is taken this way only
-// if the excess tr(G^^-1) - kbo is at most kQrMaxExcess and every pivot is clear of the zero-column
+// and the kernel that forms T's rows solves for R^-1's beside them. So does its Frobenius norm, which
+// is closer where many directions have lost a little each (the first steps of a run) and takes a
+// product of R^-1 by its transpose. The block is taken this way only if the excess tr(G^^-1) - kbo is at
+// most kQrMaxExcess, or ||G^^-1||_F at most kQrMaxInverse, and every pivot is clear of the zero-column
 // threshold; a block whose columns are all below that threshold is skipped outright (no reflectors);
-// any other block is left to the column loop: qr_panel_kernel asks qr_block_left, and writes
-// everything that a block factored here leaves behind. In the steady state of a run P = F Q has nearly
-// orthogonal columns (an excess of 0.1-6); blocks of its first steps (up to 250) and of rank-deficient
-// factors take the column loop.
+// any other block is left to the column loop: qr_panel_kernel decides, and writes everything that a
+// block factored here leaves behind. In the steady state of a run P = F Q has nearly orthogonal columns
+// (an excess of 0.1-6); a part of the first steps' blocks and those of rank-deficient factors take the
+// column loop.
 //
 //   qr_gram_kernel  G in up to 4 partial sums: tcgen05 products of 128 x 32 chunks, cluster
 //                   reduction through distributed shared memory
@@ -52,11 +54,11 @@ namespace {
 
 constexpr int NBO = kQrBlock;
 constexpr uint64_t kWaitNs = 2000000000ull;
-// Squared pivot over squared column norm below which a block leaves for the column loop at once (its
-// excess is at least 3 then; blocks of a run that the excess admits have 0.5 and more). So does one
-// whose squared norms over squared pivots, less one each, already add up to more than kQrMaxExcess:
-// G^^-1's diagonal is at least that ratio. (QR of 64 Gaussian 768-factors, most blocks of which decline:
-// 5.38 -> 5.25 ms.)
+// Squared pivot over squared column norm below which a block leaves for the column loop at once (blocks
+// of a run that the rule admits have 0.5 and more). So does one whose squared norms over squared pivots,
+// squared, already add up to more than kQrMaxInverse^2: G^^-1's diagonal is at least those ratios.
+// (Ending at the trace's limit in this way, QR of 64 Gaussian 768-factors, most blocks of which decline,
+// went from 5.38 to 5.25 ms.)
 constexpr float kRhoMin = 0.25f;
 
 // byte offset of 16-byte unit q of row r in a tile of 128-byte rows, swizzled within 1024-byte
@@ -90,8 +92,9 @@ __device__ __forceinline__ float* block_m(const QrBlockArgs& p, int b) {
   return p.Gpart + (int64_t)b * kQrGramParts * NBO * NBO;
 }
 
-// What qr_block_left reads and the core kernel hands it, in place of the second partial Gram matrix:
-// the trace of G^^-1 by rows of a CTA of the form kernel, then G's diagonal.
+// What the panel kernel decides on, and what the core kernel hands over for it, in place of the second partial Gram matrix:
+// the trace of G^^-1 by rows of a CTA of the form kernel, then G's diagonal. R^-1 scaled likewise takes
+// the place of the third.
 __device__ __forceinline__ float* block_trace(const QrBlockArgs& p, int b) {
   return p.Gpart + ((int64_t)b * kQrGramParts + 1) * NBO * NBO;
 }
@@ -314,10 +317,10 @@ __device__ __forceinline__ float inv(float x) {
 }
 
 // Columns j and j + 1 (j even) of the diagonal blocks (step 2), one warp; returns whether their
-// pivots are good, and adds to `excess` what they prove of it. The two pivot rows go through shared
+// pivots are good, and adds to `inverse2` what they prove of ||G^^-1||_F^2. The two pivot rows go through shared
 // memory once; every lane derives both columns' reflectors from them.
 __device__ __forceinline__ bool diag_pair(CoreShared& sh, float2 (&x)[kPairs], int j, float norm0, float norm1, float lim2,
-                                          float& excess) {
+                                          float& inverse2) {
   const int lane = threadIdx.x & 31, par = (j >> 1) & 1;
   const bool srow = lane < 16;
   if ((lane & 14) == j) store_pairs(sh.pv[par][lane >> 4][lane & 1], x);
@@ -377,7 +380,8 @@ __device__ __forceinline__ bool diag_pair(CoreShared& sh, float2 (&x)[kPairs], i
     sh.l[j][lane - j] = m0;
     sh.l[j + 1][lane - j] = m1;
   }
-  excess += fmaf(norm0 * ir0, ir0, -1.f) + fmaf(norm1 * ir1, ir1, -1.f);
+  const float inv0 = norm0 * ir0 * ir0, inv1 = norm1 * ir1 * ir1;
+  inverse2 += fmaf(inv0, inv0, inv1 * inv1);
   // (false for a non-finite value too; squares outside fp32's comfortable range go the other way)
   return g0 >= kRhoMin * norm0 && g1 >= kRhoMin * norm1 && g0 > lim2 && g1 > lim2 && g0 > 1e-30f && g1 > 1e-30f &&
          norm0 < 1e30f && norm1 < 1e30f;
@@ -504,7 +508,7 @@ __global__ void __launch_bounds__(kThreads, 1) qr_core_kernel(QrBlockArgs p, int
   const bool zero = sh.zero_block != 0;
   bool fast = !zero;
   const int npan = (kbo + kPw - 1) / kPw;
-  float excess = 0.f;  // (first warp)
+  float inverse2 = 0.f;  // (first warp)
   for (int pp = 0; pp < npan && fast; ++pp) {
     const int j0 = kPw * pp, pw = min(kPw, kbo - j0);  // a multiple of 4
     // 1: the panel's rows and columns
@@ -541,10 +545,10 @@ __global__ void __launch_bounds__(kThreads, 1) qr_core_kernel(QrBlockArgs p, int
       bool ok = true;
 #pragma unroll 1
       for (int j = 0; j < pw; j += 2) {
-        const bool good = diag_pair(sh, x, j, sh.norm[j0 + j], sh.norm[j0 + j + 1], lim2, excess);
+        const bool good = diag_pair(sh, x, j, sh.norm[j0 + j], sh.norm[j0 + j + 1], lim2, inverse2);
         ok = ok && good;
       }
-      if (lane == 0 && !(ok && excess <= kQrMaxExcess)) sh.fail = 1;
+      if (lane == 0 && !(ok && inverse2 <= kQrMaxInverse * kQrMaxInverse)) sh.fail = 1;
       if (lane < pw) p.dsign[(int64_t)b * n + k0 + j0 + lane] = sh.d[lane];
     }
     __syncthreads();
@@ -733,12 +737,12 @@ __device__ __forceinline__ void t_rows(const QrBlockArgs& p, int b, int rb, floa
   if (!zero) {
     // u_j = (u_j so far) / (D R)_jj, then t_j = u_j + (t_j so far): both solves advance together
     // (columns before a row's diagonal are zero and stay so)
-    float t[2][4], w[2][4], inv2[2] = {0.f, 0.f};  // w: e_i, then what is left of it; inv2: ||x||^2
+    float t[2][4], w[2][4], x0[2][4], inv2[2] = {0.f, 0.f};  // w: e_i, then what is left of it; inv2: ||x||^2
 #pragma unroll
     for (int e = 0; e < 2; ++e)
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        t[e][c] = 0.f;
+        t[e][c] = x0[e][c] = 0.f;
         w[e][c] = 4 * lane + c == i0 + e ? 1.f : 0.f;
       }
 #pragma unroll 1
@@ -764,6 +768,7 @@ __device__ __forceinline__ void t_rows(const QrBlockArgs& p, int b, int rb, floa
           if (lane == j4) t[e][c] = y;
           const float z = __shfl_sync(0xffffffffu, w[e][c], j4) * iv;
           inv2[e] = fmaf(z, z, inv2[e]);
+          if (lane == j4) x0[e][c] = z;
           w[e][0] = fmaf(-z, r.x, w[e][0]);
           w[e][1] = fmaf(-z, r.y, w[e][1]);
           w[e][2] = fmaf(-z, r.z, w[e][2]);
@@ -771,9 +776,17 @@ __device__ __forceinline__ void t_rows(const QrBlockArgs& p, int b, int rb, floa
         }
       }
     }
-    if (lane == 0) {
+    {
       const float* norm = block_trace(p, b) + kQrTraceParts;
-      s_trace[warp] = (i0 < kbo ? inv2[0] * norm[i0] : 0.f) + (i0 + 1 < kbo ? inv2[1] * norm[i0 + 1] : 0.f);
+      float trace = 0.f;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float g = i0 + e < kbo ? norm[i0 + e] : 0.f, f = sqrtf(g);
+        trace = fmaf(inv2[e], g, trace);
+        *reinterpret_cast<float4*>(block_trace(p, b) + NBO * NBO + (i0 + e) * NBO + 4 * lane) =
+            make_float4(f * x0[e][0], f * x0[e][1], f * x0[e][2], f * x0[e][3]);
+      }
+      if (lane == 0) s_trace[warp] = trace;
     }
 #pragma unroll
     for (int e = 0; e < 2; ++e)

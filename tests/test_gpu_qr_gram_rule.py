@@ -52,9 +52,10 @@ def _well(n, rng):
     return F @ F.T / (4 * n) + np.eye(n)
 
 
-@pytest.mark.parametrize("kind,rho", [("random", 0.27), ("random", 0.35), ("random", 0.5), ("bidiagonal", 0.3),
-                                      ("bidiagonal", 0.4), ("plain bidiagonal", 0.35), ("previous", 0.45),
-                                      ("one small", 256), ("one small", 32)])
+@pytest.mark.parametrize("kind,rho", [
+    ("random", 0.27), ("random", 0.35), ("random", 0.5), ("random", 0.7), ("random", 0.8), ("bidiagonal", 0.3),
+    ("bidiagonal", 0.4), ("bidiagonal", 0.8), ("plain bidiagonal", 0.35), ("previous", 0.45), ("one small", 256),
+    ("one small", 32), ("one small", 20)])
 def test_ill_conditioned_blocks(cuda, kind, rho):
     rng = np.random.default_rng(int(100 * rho))
     R = {"random": lambda: _random(N, rho, rng), "bidiagonal": lambda: _bidiagonal(N, rho),
